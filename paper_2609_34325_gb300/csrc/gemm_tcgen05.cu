@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
   };
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       int it = 0;
       bool ok = true;
       for (int pr = cid; ok && pr < num_pairs; pr += n_clusters) {
@@ -345,7 +345,8 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
       s.issued = it;
     }
   } else if (warp == 1) {
-    if (lane == 0 && kPair && rank == 0) {
+    const bool issuer = elect_one();
+    if (issuer && kPair && rank == 0) {
       // pair MMA issuer: M = 256 over both CTAs, D in both CTAs' TMEM
       constexpr uint32_t idesc = idesc_bf16(2 * BM, BN, false);
       int it = 0, ti = 0;
@@ -377,7 +378,7 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
       s.consumed = it;
       mma_commit_pair(&s.drain, 0x1);
       mbar_wait_limited(&s.drain, 0, kWaitLimitNs);
-    } else if (lane == 0) {
+    } else if (issuer) {
      if constexpr (!kPair) {
       constexpr uint32_t idesc = idesc_bf16(BM, BN, false);
       int it = 0, ti = 0;
