@@ -22,10 +22,10 @@ LIB_PATH = os.path.join(HERE, "libdora.so")
 # first K/V load, so a wait runs out (tests/test_gpu_timeout.py).
 TIMEOUT_TEST_LIB_PATH = os.path.join(HERE, "libdora_timeout_test.so")
 TIMEOUT_TEST_FLAGS = ["-DDORA_TEST_WITHHOLD_KV_LOAD", "-DDORA_TEST_WAIT_LIMIT_NS=5000000ull"]
-SOURCES = ["token_ops.cu", "gemm_tcgen05.cu", "attn_tcgen05.cu", "attn_exchange_tcgen05.cu",
-           "api.cu", "noalloc.cu", "actor.cu", "embed_head.cu", "training.cu"]
-# the attention translation units, rebuilt with the test flags for the timeout-path library
-ATTN_SOURCES = ("attn_tcgen05.cu", "attn_exchange_tcgen05.cu")
+SOURCES = ["token_ops.cu", "gemm_tcgen05.cu", "attn_tcgen05.cu", "api.cu", "noalloc.cu",
+           "actor.cu", "embed_head.cu", "training.cu"]
+# the attention translation unit, rebuilt with the test flags for the timeout-path library
+ATTN_SOURCES = ("attn_tcgen05.cu",)
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

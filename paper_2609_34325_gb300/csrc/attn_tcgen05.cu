@@ -1,103 +1,352 @@
-// Packed variable-length multi-head self-attention on tcgen05 tensor cores,
-// the kernel for images longer than 256 tokens (launch_varlen_attn below picks
-// it when max_seqlen > 256; shorter batches run attn_exchange_tcgen05.cu).
+// Packed variable-length multi-head self-attention on tcgen05 tensor cores.
 // For image i (rows [cu[i], cu[i+1]) of the packed buffer) and head h:
 //     O = softmax(Q K^T * scale) V
 // with no attention across images and no padding (Sec. 3.5 "Inference").
 //
-// Work unit = (image, head, 128-row query tile); a unit walks its keys in
-// chunks of 128 ("steps").  One persistent CTA per SM owns a contiguous range
-// of image-heads, split by estimated cost, and runs its steps through a
-// pipeline in which no role waits on the softmax's own previous work:
-//   warp 0       walks the CTA's units, loads Q and K/V chunks by TMA (the two
-//                query tiles of an image of up to 256 tokens share the chunks),
-//                and publishes a descriptor per step and per unit.  No other
-//                role keeps unit bookkeeping.
-//   warps 1-3    MMA issuers (one thread each): warp 1 issues S(j) = Q K^T
-//                (M=128, N=keys rounded to 16, K=64) into S/P buffer j mod 2,
-//                once both PVs of step j-2 are done with that buffer; warp
-//                2 + h issues O_h (+)= P_h(j) V_h for key half h (keys
-//                64h .. 64h+63 of the chunk).  A tcgen05.mma takes about 120
-//                cycles to issue, so the two halves' PVs go out in parallel.
-//   warps 4-11   softmax, two threads per query row (TMEM lane): warps 4-7
-//                take key half 0 of every step, warps 8-11 half 1, 64 S
-//                columns each, held in registers.  Each half keeps its own
-//                running reference maximum, row sum and O accumulator for the
-//                unit, so the two threads of a row never exchange anything.
-//                A half's reference maximum is set on the unit's first chunk
-//                and raised only when a later chunk exceeds it by more than
-//                2^8 (then its O is rescaled in TMEM); otherwise P stays below
-//                2^8 in the old frame, which bf16 and fp32 hold exactly.  A
-//                half writes its P (bf16) over the first 32 of its own 64 S
-//                columns, and zeroes the V rows of the chunk's last 16-key
-//                group that lie past the image when they fall in its half.
-//   warps 12-15  epilogue: once a unit's last PVs are done, the two halves'
-//                partial results are merged, O = (a_0 O_0 + a_1 O_1) /
-//                (a_0 l_0 + a_1 l_1) with a_h = 2^(m_h - max(m_0, m_1)), and
-//                stored through shared memory four whole rows per store.
-// TMEM (512 columns): S/P buffers 0-127 and 128-255; O_0 and O_1 of units of
-// even parity in 256-319 and 320-383, of odd parity in 384-447 and 448-511,
-// so a unit's PVs never wait for the previous unit's epilogue.  Rows past the image are computed but never stored;
-// keys past it are masked, and V rows past it are zeroed so stale data cannot
-// leak through 0 * NaN.
-#include "attn_common.cuh"
+// Work unit = (image, pair of heads, 128-row query tile); a unit walks its keys
+// in chunks of up to 96 ("steps"), the image's 32-key blocks dealt evenly over
+// the fewest chunks (197 tokens: 96 + 64 + 37).  One persistent CTA per SM owns
+// a contiguous range of units, split by estimated cost.  The two heads of a
+// unit run on two groups, each with its own softmax warps (one thread per query
+// row), PV issuer and half of tensor memory, so that the exponentials of one
+// cover the barriers and tensor-memory loads of the other:
+//   warp 0       walks the CTA's units, loads the Q tiles of both heads with one
+//                TMA box, and per chunk K and V of both heads with one box each
+//                (boxes of the rows needed, rounded up to 32), and publishes a
+//                descriptor per step and per unit.  Everything a unit needs is
+//                the same for both heads but the column, so this one thread
+//                keeps up with units of 65 tokens (1,300 cycles each; walking
+//                one head a unit it took 2,000 and was the limit there).
+//   warp 1       issues S(j) = Q K^T (M=128, N=keys rounded to 16, K=64) of both
+//                groups into their S/P buffers j mod 2, once PV(j - 2) is done.
+//   warps 2, 3   issue O (+)= P(j) V of group 0 and 1, P read from the buffer that
+//                S(j) was in.
+//   warps 4-11   softmax, four warps per group: the maximum comes with the loads
+//                of S (tcgen05.ld.red), then S is read again 32 columns at a time
+//                for 2^x, the row sum and P (bf16), written over columns already
+//                read.  Within a unit the reference maximum is only raised when
+//                a later chunk exceeds it by more than 2^8, and then O is rescaled
+//                in TMEM; otherwise P stays below 2^8 in the old frame, which bf16
+//                and fp32 hold exactly as well.  The softmax also zeroes the V rows
+//                of a chunk's last 16-key group that lie past the image.
+//   warps 12-15  epilogue of both groups: when a unit's last PV is done, O / row
+//                sum, each thread storing its row's 128 bytes.
+// TMEM (256 columns a group): S/P buffers at 0 and 96, O at 192.  Rows past the
+// image are computed but never stored; keys past it are masked, and V rows past
+// it are zeroed so stale data cannot leak through 0 * NaN.
+//
+// What bounds it: the serial chain of a step (about 1,700 cycles for 80 keys: the
+// maximum 350, the exponentials 1,100 with both groups on the MUFU, the hand-offs
+// the rest) and the instruction cache.  The roles' code together must stay in
+// it: a softmax unrolled per chunk length (64 KB more code) ran 238 us where this
+// loop over 32 columns runs 77, and the inlined waits of all roles are why the
+// loader and issuers have one call site for each.  Measured against the kernel
+// before it (two threads a row exchanging maxima, MMAs issued from a lane-0
+// branch, one query tile at a time), us: 256 x 197 tokens x 12 heads 93.7 ->
+// 76.7, the same after one and two deletions 69.9 -> 50.5 and 33.0 -> 26.0, 64 x
+// 577 x 12 136.9 -> 109.5, 128 x 257 x 12 91.0 -> 66.1.
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+#include <math.h>
+#include <stdint.h>
+
+#include "dora_ptx.cuh"
+#include "token_ops.cuh"
 
 namespace dora {
 namespace attn {
-namespace split {
 
-constexpr int kSpBufs = 2;      // S/P buffers, used by steps in turn
-__device__ __forceinline__ uint32_t tmem_sp(int b) { return 128u * static_cast<uint32_t>(b); }
-// O of key half h for units of parity up (two units in flight)
-__device__ __forceinline__ uint32_t tmem_o(int h, int up) {
-  return 128u * kSpBufs + 128u * static_cast<uint32_t>(up) + 64u * static_cast<uint32_t>(h);
+constexpr int BQ = 128;         // query rows per unit
+constexpr int KC = 96;          // keys per step, at most
+constexpr int HD = 64;
+constexpr int kStages = 3;      // K/V chunk ring, two heads' chunks each
+constexpr int kDescRing = 8;    // step descriptors in flight
+constexpr int kUnitRing = 4;    // unit descriptors in flight
+constexpr int kThreads = 512;   // 16 warps, 128 registers a thread at launch
+constexpr int kSoftRegs = 152;  // softmax warps (4-11)
+constexpr int kOtherRegs = 96;  // the other eight
+constexpr int kSoftWarp0 = 4;
+constexpr int kEpiWarp0 = 12;
+constexpr uint32_t kTmemCols = 512;
+constexpr float kRescaleLog2 = 8.f;    // raise the reference maximum past 2^8
+constexpr uint32_t kSleepNs = 200000;  // waiting threads sleep instead of spinning
+static_assert(8 * 32 * (kSoftRegs + kOtherRegs) <= kThreads * 128, "registers");
+
+__device__ __forceinline__ uint32_t tmem_sp(int g, int b) {
+  return 256u * static_cast<uint32_t>(g) + 96u * static_cast<uint32_t>(b);
 }
-static_assert(128 * kSpBufs + 4 * 64 <= 512, "TMEM columns");
+__device__ __forceinline__ uint32_t tmem_o(int g) { return 256u * static_cast<uint32_t>(g) + 192u; }
+
+// Tensor maps of the packed qkv buffer as [3 heads][t_cap rows][64 columns]:
+// m[i] has boxes of 32 (i + 1) rows of two neighbouring heads.
+struct QkvMaps {
+  CUtensorMap m[BQ / 32];
+};
 
 // Step descriptor (one 32-bit word).
-constexpr uint32_t kDStage = 0x3u;        // K/V stage
-constexpr uint32_t kDKvPar = 1u << 2;     // phase parity of that stage's load
-constexpr uint32_t kDLast0 = 1u << 3;     // key half 0's last chunk of this unit
-constexpr uint32_t kDLast1 = 1u << 4;     // key half 1's last chunk of this unit
-constexpr uint32_t kDUPar = 1u << 5;      // unit parity: Q buffer
-constexpr uint32_t kDQPar = 1u << 6;      // phase parity of the unit's Q load
-constexpr uint32_t kDRelease = 1u << 7;   // the K/V stage is free after this step's PV
-constexpr uint32_t kDUFirst = 1u << 8;    // first chunk of the unit (S waits for Q)
-constexpr uint32_t kDULast = 1u << 25;    // last chunk of the unit (S frees Q)
+constexpr uint32_t kDStage = 0x7u;        // K/V stage
+constexpr uint32_t kDKvPar = 1u << 3;     // phase parity of that stage's load
+constexpr uint32_t kDFirst = 1u << 4;     // first key chunk of a unit
+constexpr uint32_t kDLast = 1u << 5;      // last key chunk of a unit
 constexpr uint32_t kDEnd = 1u << 31;      // no more steps
-__device__ __forceinline__ int d_kc(uint32_t d) { return static_cast<int>((d >> 9) & 0xFFu); }
-__device__ __forceinline__ int d_rows(uint32_t d) { return static_cast<int>((d >> 17) & 0xFFu); }
-__device__ __forceinline__ int d_slot(uint32_t d) { return static_cast<int>((d >> 26) & 0x3u); }
+__device__ __forceinline__ int d_kc(uint32_t d) { return static_cast<int>((d >> 8) & 0x7Fu); }
+__device__ __forceinline__ int d_blocks(uint32_t d) { return (d_kc(d) + 31) >> 5; }
+__device__ __forceinline__ int d_rows(uint32_t d) { return static_cast<int>((d >> 16) & 0xFFu); }
 
 struct Smem {
-  uint16_t q[2][BQ * HD];       // 2 x 16 KB, by unit parity
-  uint16_t k[kStages][KC * HD]; // 4 x 16 KB
-  uint16_t v[kStages][KC * HD]; // 4 x 16 KB
-  uint4 ostage[4][32 * 8];      // per epilogue warp: 32 output rows of 128 bytes
-  float2 lm[kUnitRing][2][BQ];  // (row sum, reference maximum) of each half, by unit slot
+  uint16_t q[2][2][BQ * HD];    // 16 KB each: by unit parity and group
+  uint16_t k[kStages][2][KC * HD];   // 12 KB each: by stage and group
+  uint16_t v[kStages][2][KC * HD];
+  float lsum[2][4][BQ];         // row sums, by group and unit mod 4
   uint64_t q_full[2];
   uint64_t q_empty[2];
   uint64_t kv_full[kStages];
-  uint64_t kv_empty[kStages];
-  uint64_t s_full[kSpBufs];     // S of a step in S/P buffer b
-  uint64_t p_full[kSpBufs][2];  // half h's P written over its S (one arrival per warp)
-  uint64_t p_free[kSpBufs];     // both PVs of buffer b done
-  uint64_t o_done[2][2];        // last PV of a unit into O_h (unit parity) done
-  uint64_t o_free[2][2];        // O_h (unit parity) read out (one arrival per epilogue warp)
-  uint64_t l_full[kUnitRing][2];  // a half's row sums of a unit published
+  uint64_t kv_empty[kStages];   // one arrival per group
+  uint64_t s_full[2][2];        // S of a step in the group's S/P buffer b
+  uint64_t p_full[2][2];        // P written over it (one arrival per softmax warp)
+  uint64_t p_free[2][2];        // PV of buffer b done
+  uint64_t o_done[2];           // last PV of a unit done
+  uint64_t o_free[2];           // O read out (one arrival per epilogue warp)
+  uint64_t l_full[2][4];        // row sums of a unit (one arrival per softmax warp)
   uint64_t sd_full[kDescRing];  // step descriptor published
   uint64_t sd_empty[kDescRing]; // ... read by the three issuers and the eight softmax warps
   uint64_t ud_full[kUnitRing];  // unit descriptor published
-  uint64_t ud_empty[kUnitRing]; // ... and the unit finished by the four epilogue warps
+  uint64_t ud_empty[kUnitRing]; // ... read by the four epilogue warps
   uint64_t drain[3];
   uint32_t sdesc[kDescRing];
   uint32_t urow[kUnitRing];     // first output row of the unit
-  uint32_t uhead[kUnitRing];    // head | rows << 16 | key halves used << 24
+  uint32_t uhead[kUnitRing];    // first head | rows << 16
   uint32_t tmem_base;
   int abort_flag;
-  int ih_begin, ih_end;
+  int img_begin, unit_begin, img_end, unit_end;   // the CTA's units
   int q_issued, kv_issued;
 };
+static_assert(sizeof(Smem) <= 227 * 1024, "shared memory");
+
+// The map's box from row y of heads z and z + 1, one behind the other in dst.
+__device__ __forceinline__ void tma_load_heads(void* dst, const CUtensorMap* map, uint64_t* bar,
+                                               int y, int z) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(y), "r"(z), "r"(smem_u32(bar))
+      : "memory");
+}
+
+// Rows of the image with bounds [b0, b1), clamped to the buffer (0 when its
+// start lies outside); lo receives its first row.
+__device__ __forceinline__ int clamp_rows(int b0, int b1, int t_cap, int& lo) {
+  lo = b0;
+  const int n = b1 - b0;
+  if (lo < 0 || lo > t_cap) {
+    lo = 0;
+    return 0;
+  }
+  return n < 0 ? 0 : (n > t_cap - lo ? t_cap - lo : n);
+}
+
+// Query tiles of an image of n rows, and the estimated cost of one: its 16-key
+// groups plus a fixed part (about four groups' worth of hand-offs, Q load and
+// output).
+__device__ __forceinline__ int tiles_of(int n) { return (n + BQ - 1) / BQ; }
+__device__ __forceinline__ int unit_cost(int n) { return (n + 15) / 16 + 4; }
+
+// A CTA's units, in image-major, head, query-tile order.  The next image's end
+// is fetched an image ahead.
+struct Walker {
+  const int32_t* cu;
+  int batch, pairs, t_cap, img_end, unit_end;
+  int img, unit, pair, qt, n, nqt, lo, hi, ahead;
+  __device__ __forceinline__ void load_image() {
+    const int b0 = hi;
+    hi = ahead;
+    if (img + 2 <= batch) ahead = __ldg(cu + img + 2);
+    n = clamp_rows(b0, hi, t_cap, lo);
+    nqt = tiles_of(n);
+  }
+  __device__ __forceinline__ bool done() const {
+    return img > img_end || (img == img_end && unit >= unit_end) || img >= batch;
+  }
+  __device__ __forceinline__ void settle() {      // to an image with a unit at `unit`
+    while (!done() && unit >= pairs * nqt) {
+      ++img;
+      unit = pair = qt = 0;
+      if (img < batch) load_image();
+    }
+  }
+  __device__ __forceinline__ void start(const int32_t* c, int b, int p, int tc, int ib, int ub,
+                                        int ie, int ue) {
+    cu = c;
+    batch = b;
+    pairs = p;
+    t_cap = tc;
+    img = ib;
+    unit = ub;
+    img_end = ie;
+    unit_end = ue;
+    pair = qt = n = nqt = lo = hi = ahead = 0;
+    if (img >= batch) return;
+    hi = __ldg(cu + img);
+    ahead = __ldg(cu + img + 1);
+    load_image();
+    if (nqt > 0) {
+      pair = unit / nqt;
+      qt = unit - pair * nqt;
+    }
+    settle();
+  }
+  __device__ __forceinline__ void next() {
+    ++unit;
+    if (++qt == nqt) {
+      qt = 0;
+      ++pair;
+    }
+    settle();
+  }
+};
+
+// Whole warp: the CTA's units, [(ib, ub), (ie, ue)) as (image, unit of the
+// image).  A unit belongs to CTA floor(C * grid / total), C being the cost of
+// the units before it; CTA 0 also checks every image against the buffer and
+// max_seqlen.  With several units a CTA the bounds are moved up to whole pairs
+// of query tiles, which share their K/V loads.  Each lane owns a contiguous
+// block of images whose bounds it reads as one batch of independent loads, so
+// the whole search costs about two memory round trips for any batch.
+__device__ inline void find_range(const int32_t* cu, int batch, int pairs, int t_cap,
+                                  int max_seqlen, int32_t* status, int& ib, int& ub, int& ie,
+                                  int& ue) {
+  const int lane = threadIdx.x & 31;
+  const int per = (batch + 31) / 32;
+  const int i0 = min(batch, lane * per), i1 = min(batch, i0 + per);
+  long long mine = 0;                   // this lane's images: cost, one head pair
+  int c_last = 0;                       // its last unit's cost
+#pragma unroll 1
+  for (int k0 = i0; k0 < i1; k0 += 8) {
+    int bnd[9];
+#pragma unroll
+    for (int t = 0; t < 9; ++t) bnd[t] = (k0 + t <= i1) ? __ldg(cu + k0 + t) : 0;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      if (k0 + t < i1) {
+        int lo;
+        const int n = clamp_rows(bnd[t], bnd[t + 1], t_cap, lo);
+        if (n > 0) {
+          c_last = unit_cost(n);
+          mine += static_cast<long long>(tiles_of(n)) * c_last;
+        }
+        if (blockIdx.x == 0) {
+          const int l0 = bnd[t], len = bnd[t + 1] - l0;
+          if (l0 < 0 || l0 > t_cap || len > t_cap - l0 || len > max_seqlen)
+            record_status(status, DORA_ERR_DEVICE_SEQLEN);
+        }
+      }
+    }
+  }
+  long long incl = mine;                // one head pair's cost up to this lane's last image
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  const long long one_pair = __shfl_sync(0xffffffffu, incl, 31);
+  const long long total = one_pair * pairs, G = gridDim.x, bx = blockIdx.x;
+  // first unit with C * G >= x ((batch, 0) if none): C grows along the order, so
+  // it lies in the first lane whose last unit reaches x, found by that lane
+  // walking its own images (their bounds are in L1 by now)
+  auto locate = [&](long long x, int& img, int& unit) {
+    const bool has = c_last > 0 && (pairs * incl - c_last) * G >= x;
+    const unsigned m = __ballot_sync(0xffffffffu, has);
+    img = batch;
+    unit = 0;
+    if (m == 0u) return;
+    const int owner = __ffs(m) - 1;
+    if (lane == owner) {
+      long long pre = pairs * (incl - mine);      // cost of the units before image i0
+      for (int i = i0; i < i1; ++i) {
+        int lo;
+        const int n = clamp_rows(cu[i], cu[i + 1], t_cap, lo);
+        if (n == 0) continue;
+        const int nqt = tiles_of(n);
+        const long long c = unit_cost(n), u = static_cast<long long>(pairs) * nqt;
+        if ((pre + (u - 1) * c) * G >= x) {
+          const long long need = x - pre * G;
+          long long w = need > 0 ? (need + c * G - 1) / (c * G) : 0;
+          img = i;
+          unit = static_cast<int>(w);
+          break;
+        }
+        pre += u * c;
+      }
+    }
+    img = __shfl_sync(0xffffffffu, img, owner);
+    unit = __shfl_sync(0xffffffffu, unit, owner);
+  };
+  ib = ie = batch;
+  ub = ue = 0;
+  if (one_pair == 0) return;
+#pragma unroll 1
+  for (int e = 0; e < 2; ++e) {
+    int img = batch, unit = 0;
+    if (bx + e < G) locate((bx + e) * total, img, unit);
+    if (e == 0) {
+      ib = img;
+      ub = unit;
+    } else {
+      ie = img;
+      ue = unit;
+    }
+  }
+}
+
+__device__ __forceinline__ bool wait_one(uint64_t* bar, uint32_t parity, volatile int* abort) {
+  return mbar_wait_sleep(bar, parity, abort, kSleepNs);
+}
+__device__ __forceinline__ bool wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort) {
+  return __all_sync(0xffffffffu, wait_one(bar, parity, abort)) != 0;
+}
+
+// One arrival for the whole warp, after every lane's prior tcgen05 accesses.
+__device__ __forceinline__ void warp_arrive(uint64_t* bar) {
+  tc_fence_before();
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
+}
+
+// -infinity in `count` (1 to 15) columns from taddr on, of this lane's row.
+__device__ __forceinline__ void mask_columns(uint32_t taddr, int count) {
+  const uint32_t v = __float_as_uint(-INFINITY);
+  if (count & 8) {
+    const uint32_t v8[8] = {v, v, v, v, v, v, v, v};
+    tmem_st8(taddr, v8);
+    taddr += 8;
+  }
+  if (count & 4) {
+    tmem_st4(taddr, v);
+    taddr += 4;
+  }
+  if (count & 2) {
+    tmem_st2(taddr, v);
+    taddr += 2;
+  }
+  if (count & 1) tmem_st1(taddr, v);
+  tmem_st_wait();
+}
+
+// p = 2^(s scale - m) of N values, summed into l0 and l1 and packed to bf16.
+template <int N>
+__device__ __forceinline__ void exp_pack(const uint32_t (&a)[N], uint32_t (&p)[N / 2], uint64_t sc,
+                                         uint64_t nm, uint64_t& l0, uint64_t& l1) {
+#pragma unroll
+  for (int e = 0; e < N; e += 2) {
+    float x0, x1;
+    f2_unpack(f2_fma(f2_pack(__uint_as_float(a[e]), __uint_as_float(a[e + 1])), sc, nm), x0, x1);
+    const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
+    if (e & 2) l1 = f2_add(l1, f2_pack(p0, p1));
+    else l0 = f2_add(l0, f2_pack(p0, p1));
+    p[e >> 1] = pack_bf16x2(p0, p1);
+  }
+}
 
 __global__ void __launch_bounds__(kThreads, 1)
     varlen_attn_kernel(const __grid_constant__ QkvMaps mp, const int32_t* __restrict__ cu,
@@ -116,54 +365,47 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int dim = heads * HD;
 
   if (threadIdx.x == 64) {
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&s.q_full[b], 1);
-      mbar_init(&s.q_empty[b], 1);
-      for (int h = 0; h < 2; ++h) {
-        mbar_init(&s.o_done[h][b], 1);
-        mbar_init(&s.o_free[h][b], 4);
+    for (int g = 0; g < 2; ++g) {
+      for (int b = 0; b < 2; ++b) {
+        mbar_init(&s.s_full[g][b], 1);
+        mbar_init(&s.p_full[g][b], 4);
+        mbar_init(&s.p_free[g][b], 1);
       }
-    }
-    for (int b = 0; b < kSpBufs; ++b) {
-      mbar_init(&s.s_full[b], 1);
-      mbar_init(&s.p_full[b][0], 4);
-      mbar_init(&s.p_full[b][1], 4);
-      mbar_init(&s.p_free[b], 2);
-    }
-    for (int i = 0; i < kUnitRing; ++i) {
-      mbar_init(&s.l_full[i][0], 4);
-      mbar_init(&s.l_full[i][1], 4);
-    }
-    for (int i = 0; i < kStages; ++i) {
-      mbar_init(&s.kv_full[i], 1);
-      mbar_init(&s.kv_empty[i], 2);                 // released by both PV issuers
+      mbar_init(&s.q_full[g], 1);
+      mbar_init(&s.q_empty[g], 1);
+      mbar_init(&s.o_done[g], 1);
+      mbar_init(&s.o_free[g], 4);
+      for (int i = 0; i < 4; ++i) mbar_init(&s.l_full[g][i], 4);
+      mbar_init(&s.drain[g], 1);
     }
     for (int i = 0; i < kDescRing; ++i) {
       mbar_init(&s.sd_full[i], 1);
       mbar_init(&s.sd_empty[i], 11);
     }
+    for (int i = 0; i < kStages; ++i) {
+      mbar_init(&s.kv_full[i], 1);
+      mbar_init(&s.kv_empty[i], 2);
+    }
     for (int i = 0; i < kUnitRing; ++i) {
       mbar_init(&s.ud_full[i], 1);
       mbar_init(&s.ud_empty[i], 4);
     }
-    for (int i = 0; i < 3; ++i) mbar_init(&s.drain[i], 1);
+    mbar_init(&s.drain[2], 1);
     s.abort_flag = 0;
     s.q_issued = s.kv_issued = 0;
     fence_barrier_init();
-    tma_prefetch_desc(&mp.m128);
-    tma_prefetch_desc(&mp.m64);
-    tma_prefetch_desc(&mp.m32);
-    tma_prefetch_desc(&mp.m16);
   }
-  if (warp == 1) tmem_alloc(&s.tmem_base, kTmemCols);
+  if (warp == 3) tmem_alloc(&s.tmem_base, kTmemCols);
   // the set-up above overlaps the previous kernel; global memory waits for it
   pdl_wait();
   if (warp == 0) {
-    long long b, e;
-    find_range(cu, batch, heads, t_cap, max_seqlen, status, b, e);
+    int ib, ub, ie, ue;
+    find_range(cu, batch, (heads + 1) / 2, t_cap, max_seqlen, status, ib, ub, ie, ue);
     if (lane == 0) {
-      s.ih_begin = static_cast<int>(b);
-      s.ih_end = static_cast<int>(e);
+      s.img_begin = ib;
+      s.unit_begin = ub;
+      s.img_end = ie;
+      s.unit_end = ue;
     }
   }
   tc_fence_before();
@@ -171,67 +413,53 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = s.tmem_base;
   volatile int* abort = &s.abort_flag;
-  const int ih_b = s.ih_begin, ih_e = s.ih_end;
 
-  if (warp == 0) {
-    // ---------------- scheduler + TMA producer ----------------
-    if (lane == 0) {
-      Walker wk;
-      wk.start(cu, heads, t_cap, ih_b, ih_e);
-      int u = 0, loads = 0, dn = 0;
-      int prev_stage[2] = {0, 0}, prev_par[2] = {0, 0};
-      bool reuse_this = false;      // this unit reads the previous unit's K/V chunks
-      bool ok = true;
-      auto desc = [&](uint32_t d) -> bool {
-        const int i = dn % kDescRing;
-        if (!mbar_wait_sleep(&s.sd_empty[i], ((dn / kDescRing) & 1) ^ 1, abort, kSleepNs))
-          return false;
-        s.sdesc[i] = d;
-        mbar_arrive(&s.sd_full[i]);
-        ++dn;
-        return true;
-      };
-      while (ok && !wk.done()) {
-        const int n = wk.n, nch = (n + KC - 1) / KC;
-        const int rows = min(BQ, n - wk.qt * BQ);
-        Walker nx = wk;
-        nx.next();
-        // the next unit (the image-head's other query tile) reads the same chunks
-        const bool reuse_next = !nx.done() && nx.ih == wk.ih && nch <= 2;
-        // key half 1 has keys in a chunk of more than 64 keys: every chunk but
-        // a short last one; none when the image has 64 tokens or fewer
-        const int kc_last = n - (nch - 1) * KC;
-        const int last1 = kc_last > 64 ? nch - 1 : nch - 2;
-        const uint32_t gmask = n > 64 ? 3u : 1u;
-        const int slot = u % kUnitRing;
-        {
-          // the slot is free once the epilogue has finished unit u - kUnitRing
-          if (!mbar_wait_sleep(&s.ud_empty[slot], ((u / kUnitRing) & 1) ^ 1, abort, kSleepNs))
-            break;
-          s.urow[slot] = static_cast<uint32_t>(wk.lo + wk.qt * BQ);
-          s.uhead[slot] = static_cast<uint32_t>(wk.head) | (static_cast<uint32_t>(rows) << 16) |
-                          (gmask << 24);
-          mbar_arrive(&s.ud_full[slot]);
-        }
-        const int qb = u & 1;
-        if (!mbar_wait_sleep(&s.q_empty[qb], ((u >> 1) & 1) ^ 1, abort, kSleepNs)) break;
-        const int rows16 = (rows + 15) & ~15;
-        mbar_arrive_expect_tx(&s.q_full[qb], static_cast<uint32_t>(rows16 * HD * 2));
-        load_rows(mp, s.q[qb], &s.q_full[qb], wk.head * HD, wk.lo + wk.qt * BQ, rows16);
-        s.q_issued = u + 1;
-        int cur_stage[2] = {0, 0}, cur_par[2] = {0, 0};
-        for (int c = 0; ok && c < nch; ++c) {
-          int stg, par;
-          if (reuse_this) {
-            stg = prev_stage[c];
-            par = prev_par[c];
-          } else {
-            stg = loads % kStages;
-            par = (loads / kStages) & 1;
-            if (!mbar_wait_sleep(&s.kv_empty[stg], par ^ 1, abort, kSleepNs)) {
-              ok = false;
-              break;
-            }
+  if (warp < kSoftWarp0) {
+    setmaxnreg_dec<kOtherRegs>();
+    if (warp == 0) {
+      // ---------------- scheduler + TMA producer ----------------
+      if (elect_one()) {
+        Walker wk;
+        wk.start(cu, batch, (heads + 1) / 2, t_cap, s.img_begin, s.unit_begin, s.img_end,
+                 s.unit_end);
+        int loads = 0, stg = 0;
+        uint32_t par = 0;                       // chunks loaded; their stage and its phase parity
+        int dn = 0;                             // steps published
+        int u = 0;                              // units begun
+        bool ok = true;
+        int n_of = -1, nch = 0, base = 0, more = 0;   // chunks of images of n_of rows
+        auto desc = [&](uint32_t d) -> bool {
+          const int i = dn % kDescRing;
+          if (!wait_one(&s.sd_empty[i], ((dn / kDescRing) & 1) ^ 1, abort)) return false;
+          s.sdesc[i] = d;
+          mbar_arrive(&s.sd_full[i]);
+          ++dn;
+          return true;
+        };
+        for (; ok && !wk.done(); wk.next(), ++u) {
+          // the unit's Q tiles and its descriptor
+          const int i = u % kUnitRing, qb = u & 1, row = wk.lo + wk.qt * BQ;
+          const int rows = min(BQ, wk.n - wk.qt * BQ), r32 = (rows + 31) >> 5;
+          if (!(ok = wait_one(&s.q_empty[qb], ((u >> 1) & 1) ^ 1, abort))) break;
+          mbar_arrive_expect_tx(&s.q_full[qb], 2 * r32 * 32 * HD * 2);
+          tma_load_heads(s.q[qb], &mp.m[r32 - 1], &s.q_full[qb], row, 2 * wk.pair);
+          s.q_issued = u + 1;
+          if (!(ok = wait_one(&s.ud_empty[i], ((u / kUnitRing) & 1) ^ 1, abort))) break;
+          s.urow[i] = static_cast<uint32_t>(row);
+          s.uhead[i] = static_cast<uint32_t>(2 * wk.pair) | (static_cast<uint32_t>(rows) << 16);
+          mbar_arrive(&s.ud_full[i]);
+          // its K/V chunks: the 32-key blocks dealt over the fewest chunks
+          if (wk.n != n_of) {
+            n_of = wk.n;
+            const int blocks = (n_of + 31) >> 5;
+            nch = (blocks + KC / 32 - 1) / (KC / 32);
+            base = blocks / nch;
+            more = blocks - base * nch;
+          }
+          int off = 0;
+          for (int c = 0; c < nch; ++c) {
+            const int cb = base + (c < more ? 1 : 0);       // 32-key blocks of the chunk
+            if (!(ok = wait_one(&s.kv_empty[stg], par ^ 1, abort))) break;
 #ifdef DORA_TEST_WITHHOLD_KV_LOAD
             // timeout-path test library only: CTA 0 never issues its first K/V
             // load nor its expected bytes, so the S issuer's bounded wait on
@@ -241,308 +469,269 @@ __global__ void __launch_bounds__(kThreads, 1)
             constexpr bool withhold = false;
 #endif
             if (!withhold) {
-              const int kc16 = (min(KC, n - c * KC) + 15) & ~15;
-              mbar_arrive_expect_tx(&s.kv_full[stg], static_cast<uint32_t>(2 * kc16 * HD * 2));
-              const int row = wk.lo + c * KC;
-              load_rows(mp, s.k[stg], &s.kv_full[stg], dim + wk.head * HD, row, kc16);
-              load_rows(mp, s.v[stg], &s.kv_full[stg], 2 * dim + wk.head * HD, row, kc16);
+              mbar_arrive_expect_tx(&s.kv_full[stg], 4 * cb * 32 * HD * 2);
+              tma_load_heads(s.k[stg], &mp.m[cb - 1], &s.kv_full[stg], wk.lo + off,
+                             heads + 2 * wk.pair);
+              tma_load_heads(s.v[stg], &mp.m[cb - 1], &s.kv_full[stg], wk.lo + off,
+                             2 * (heads + wk.pair));
             }
-            ++loads;
-            s.kv_issued = loads;
+            s.kv_issued = ++loads;
+            ok = desc(static_cast<uint32_t>(stg) | (par ? kDKvPar : 0u) | (c == 0 ? kDFirst : 0u) |
+                      (c == nch - 1 ? kDLast : 0u) |
+                      (static_cast<uint32_t>(min(32 * cb, n_of - off)) << 8) |
+                      (static_cast<uint32_t>(rows) << 16));
+            if (!ok) break;
+            if (++stg == kStages) {
+              stg = 0;
+              par ^= 1u;
+            }
+            off += 32 * cb;
           }
-          if (c < 2) {
-            cur_stage[c] = stg;
-            cur_par[c] = par;
-          }
-          const uint32_t d =
-              static_cast<uint32_t>(stg) | (par ? kDKvPar : 0u) | (c == nch - 1 ? kDLast0 : 0u) |
-              (c == last1 ? kDLast1 : 0u) | ((u & 1) ? kDUPar : 0u) |
-              (((u >> 1) & 1) ? kDQPar : 0u) | (reuse_next ? 0u : kDRelease) |
-              (c == 0 ? kDUFirst : 0u) | (c == nch - 1 ? kDULast : 0u) |
-              (static_cast<uint32_t>(min(KC, n - c * KC)) << 9) |
-              (static_cast<uint32_t>(rows) << 17) | (static_cast<uint32_t>(slot) << 26);
-          ok = desc(d);
         }
-        prev_stage[0] = cur_stage[0];
-        prev_stage[1] = cur_stage[1];
-        prev_par[0] = cur_par[0];
-        prev_par[1] = cur_par[1];
-        reuse_this = reuse_next;
-        ++u;
-        wk = nx;
-      }
-      if (ok && desc(kDEnd)) {
-        const int i = u % kUnitRing;      // no more units
-        if (mbar_wait_sleep(&s.ud_empty[i], ((u / kUnitRing) & 1) ^ 1, abort, kSleepNs)) {
-          s.uhead[i] = 0xFFFFFFFFu;
-          mbar_arrive(&s.ud_full[i]);
+        if (ok && desc(kDEnd)) {
+          const int i = u % kUnitRing;          // no more units
+          if (wait_one(&s.ud_empty[i], ((u / kUnitRing) & 1) ^ 1, abort)) {
+            s.uhead[i] = 0xFFFFFFFFu;
+            mbar_arrive(&s.ud_full[i]);
+          }
         }
       }
-    }
-  } else if (warp >= 1 && warp <= 3) {
-    // ---------------- MMA issuers: warp 1 issues S, warp 2 + h the PV of key half h ----------------
-    // Each reads every step descriptor.  The only order between them is
-    // explicit: S(j + kSpBufs) waits until both PVs of step j have read S/P
-    // buffer j mod kSpBufs.
-    if (lane == 0) {
-      int uses[2] = {0, 0};        // units started in O_h, by unit parity (PV issuer of half h)
-      for (int j = 0;; ++j) {
-        const int i = j % kDescRing;
-        if (!mbar_wait_sleep(&s.sd_full[i], (j / kDescRing) & 1, abort, kSleepNs)) break;
-        const uint32_t d = s.sdesc[i];
-        mbar_arrive(&s.sd_empty[i]);
-        if (d & kDEnd) break;
-        const int stg = static_cast<int>(d & kDStage);
-        const int up = (d & kDUPar) ? 1 : 0;
-        const int b = j % kSpBufs;
-        const uint32_t bph = static_cast<uint32_t>(j / kSpBufs) & 1u;   // buffer use parity
-        if (warp == 1) {
-          // S(j) = Q K^T into S/P buffer b
-          if ((d & kDUFirst) &&
-              !mbar_wait_sleep(&s.q_full[up], (d & kDQPar) ? 1u : 0u, abort, kSleepNs))
-            break;
-          if (!mbar_wait_sleep(&s.kv_full[stg], (d & kDKvPar) ? 1u : 0u, abort, kSleepNs)) break;
-          // the buffer's previous P has been read by its PV (step j - kSpBufs)
-          if (j >= kSpBufs && !mbar_wait_sleep(&s.p_free[b], bph ^ 1u, abort, kSleepNs)) break;
-          tc_fence_after();
-          const uint64_t qd = sdesc_sw128(smem_u32(s.q[up]), 16, 1024);
-          const uint64_t kd = sdesc_sw128(smem_u32(s.k[stg]), 16, 1024);
-          const uint32_t id_s = idesc_bf16(BQ, (d_kc(d) + 15) & ~15, false);
-          const uint32_t dt = tmem + tmem_sp(b);
-          mma_bf16_ss(dt, qd, kd, id_s, 0u);
-          mma_bf16_ss(dt, qd + 2, kd + 2, id_s, 1u);
-          mma_bf16_ss(dt, qd + 4, kd + 4, id_s, 1u);
-          mma_bf16_ss(dt, qd + 6, kd + 6, id_s, 1u);
-          mma_commit(&s.s_full[b]);
-          if (d & kDULast) mma_commit(&s.q_empty[up]);
-        } else {
-          // O_h (+)= P_h(j) V_h over the step's keys 64h .. 64h + 63
+    } else if (warp == 1) {
+      // ---------------- S issuer of both groups ----------------
+      // S(j) = Q K^T of a group goes into S/P buffer j mod 2 once PV(j - 2) has read
+      // its P there.
+      if (elect_one()) {
+        int u = 0;                              // units whose S are all issued
+        bool ok = true;
+        for (int j = 0; ok; ++j) {
+          const int i = j % kDescRing, b = j & 1, qb = u & 1;
+          if (!wait_one(&s.sd_full[i], (j / kDescRing) & 1, abort)) break;
+          const uint32_t d = s.sdesc[i];
+          mbar_arrive(&s.sd_empty[i]);
+          if (d & kDEnd) break;
+          const int stg = static_cast<int>(d & kDStage), groups = (d_kc(d) + 15) >> 4;
+          if (!wait_one(&s.kv_full[stg], (d & kDKvPar) ? 1u : 0u, abort)) break;
+          if ((d & kDFirst) && !wait_one(&s.q_full[qb], (u >> 1) & 1, abort)) break;
+          const uint32_t id_s = idesc_bf16(BQ, 16 * groups, false);
+          // a load of two heads puts the second right behind the first
+          const int q_step = ((d_rows(d) + 31) & ~31) * HD, k_step = 32 * d_blocks(d) * HD;
+#pragma unroll 1
+          for (int g = 0; g < 2; ++g) {
+            if (j >= 2 && !(ok = wait_one(&s.p_free[g][b], ((j >> 1) - 1) & 1, abort))) break;
+            tc_fence_after();
+            const uint64_t qd = sdesc_sw128(smem_u32(&s.q[qb][0][0] + g * q_step), 16, 1024);
+            const uint64_t kd = sdesc_sw128(smem_u32(&s.k[stg][0][0] + g * k_step), 16, 1024);
+            const uint32_t dt = tmem + tmem_sp(g, b);
+            mma_bf16_ss(dt, qd, kd, id_s, 0u);
+            mma_bf16_ss(dt, qd + 2, kd + 2, id_s, 1u);
+            mma_bf16_ss(dt, qd + 4, kd + 4, id_s, 1u);
+            mma_bf16_ss(dt, qd + 6, kd + 6, id_s, 1u);
+            mma_commit(&s.s_full[g][b]);
+          }
+          if (d & kDLast) {
+            mma_commit(&s.q_empty[qb]);
+            ++u;
+          }
+        }
+        mma_commit(&s.drain[2]);
+        mbar_wait_limited(&s.drain[2], 0, kWaitLimitNs);
+      }
+    } else {
+      // ---------------- PV issuer of group g ----------------
+      // O (+)= P(j) V once P(j) is written and, on a unit's first chunk, the
+      // epilogue has read the group's previous O.
+      if (elect_one()) {
+        const int g = warp - 2;
+        int up = 0;                             // units whose PVs are all issued
+        for (int j = 0;; ++j) {
+          const int i = j % kDescRing, b = j & 1;
+          if (!wait_one(&s.sd_full[i], (j / kDescRing) & 1, abort)) break;
+          const uint32_t d = s.sdesc[i];
+          mbar_arrive(&s.sd_empty[i]);
+          if (d & kDEnd) break;
+          const int nk = (d_kc(d) + 15) >> 4, stg = static_cast<int>(d & kDStage);
+          const uint64_t vd =
+              sdesc_sw128(smem_u32(&s.v[stg][0][0] + g * 32 * d_blocks(d) * HD), 1024, 1024);
+          const uint32_t ot = tmem + tmem_o(g), at = tmem + tmem_sp(g, b);
           constexpr uint32_t id_o = idesc_bf16(BQ, HD, true);
-          const int h = warp - 2;
-          const int kh = min(max(d_kc(d) - 64 * h, 0), 64);   // keys of this half
-          const bool first = (d & kDUFirst) != 0 && kh > 0;
-          // O_h held the half's part of an earlier unit until the epilogue read it
-          if (first) {
-            if (uses[up] > 0 &&
-                !mbar_wait_sleep(&s.o_free[h][up], static_cast<uint32_t>(uses[up] - 1) & 1u,
-                                 abort, kSleepNs))
-              break;
-            ++uses[up];
-          }
-          if (!mbar_wait_sleep(&s.p_full[b][h], bph, abort, kSleepNs)) break;
+          if ((d & kDFirst) && up > 0 && !wait_one(&s.o_free[g], (up - 1) & 1, abort)) break;
+          if (!wait_one(&s.p_full[g][b], (j >> 1) & 1, abort)) break;
           tc_fence_after();
-          if (kh > 0) {
-            const int nk = (kh + 15) >> 4;
-            // V rows 64h .. : 16 keys are 2048 bytes of the 128-byte-swizzled tile
-            const uint64_t vd = sdesc_sw128(smem_u32(s.v[stg] + 64 * h * HD), 1024, 1024);
-            const uint32_t dt = tmem + tmem_o(h, up), at = tmem + tmem_sp(b) + 64u * h;
-            mma_bf16_ts(dt, at, vd, id_o, first ? 0u : 1u);
+          mma_bf16_ts(ot, at, vd, id_o, (d & kDFirst) ? 0u : 1u);
 #pragma unroll
-            for (int kk = 1; kk < 4; ++kk)       // 16 keys: 8 P columns
-              if (kk < nk) mma_bf16_ts(dt, at + 8u * kk, vd + 128u * kk, id_o, 1u);
+          for (int kk = 1; kk < KC / 16; ++kk)   // 16 keys: 2048 bytes of V, 8 P columns
+            if (kk < nk) mma_bf16_ts(ot, at + 8u * kk, vd + 128u * kk, id_o, 1u);
+          mma_commit(&s.p_free[g][b]);
+          if (d & kDLast) {
+            mma_commit(&s.o_done[g]);
+            ++up;
           }
-          mma_commit(&s.p_free[b]);
-          if (d & (h == 0 ? kDLast0 : kDLast1)) mma_commit(&s.o_done[h][up]);
-          if (d & kDRelease) mma_commit(&s.kv_empty[stg]);
+          mma_commit(&s.kv_empty[stg]);
         }
+        mma_commit(&s.drain[g]);
+        mbar_wait_limited(&s.drain[g], 0, kWaitLimitNs);
       }
-      mma_commit(&s.drain[warp - 1]);
-      mbar_wait_limited(&s.drain[warp - 1], 0, kWaitLimitNs);
     }
-  } else if (warp >= kSoftWarp0 && warp < kEpiWarp0) {
-    // ---------------- softmax: key half h of every step, two threads per row ----------------
-    const int h = (warp - kSoftWarp0) >> 2;
+  } else if (warp < kEpiWarp0) {
+    // ---------------- softmax: one thread per query row ----------------
+    setmaxnreg_inc<kSoftRegs>();
+    const int g = (warp - kSoftWarp0) >> 2;
     const int quarter = warp & 3;
     const int r = quarter * 32 + lane;                   // query row of the tile (TMEM lane)
     const uint32_t lane_sel = static_cast<uint32_t>(quarter * 32) << 16;
-    float m_ref = 0.f, l = 0.f;                          // the half's frame and row sum
+    const uint64_t sc = f2_pack(scale_log2, scale_log2);
+    float m_ref = 0.f, l = 0.f;                          // reference (log2 units), row sum
+    int u = 0;                                           // units finished
     auto step = [&](int j, uint32_t d) -> bool {
-      const int kc = d_kc(d), kc16 = (kc + 15) & ~15;
-      const int kh = min(max(kc - 64 * h, 0), 64);       // keys in this half
-      const bool live = quarter * 32 < d_rows(d) && kh > 0;   // warp-uniform
-      const int b = j % kSpBufs;
-      const uint32_t bph = static_cast<uint32_t>(j / kSpBufs) & 1u;   // buffer use parity
-      const uint32_t tsp = tmem + lane_sel + tmem_sp(b) + 64u * h;   // this half's S columns
-      if (!mbar_wait_warp_sleep(&s.s_full[b], bph, abort, kSleepNs)) return false;
+      const int kc = d_kc(d), groups = (kc + 15) >> 4, b = j & 1;
+      const bool live = quarter * 32 < d_rows(d);        // warp-uniform
+      const uint32_t tsp = tmem + lane_sel + tmem_sp(g, b);
+      if (!wait_warp(&s.s_full[g][b], (j >> 1) & 1, abort)) return false;
       tc_fence_after();
-      // S is done, so the K/V load landed: zero V rows [kc, kc16) (whole 128-byte
-      // rows; they lie in one half, whose PV reads them)
-      if (kc < kc16 && (kc >> 6) == h) {
-        if (r < (kc16 - kc) * 8)
-          reinterpret_cast<uint4*>(s.v[d & kDStage])[kc * 8 + r] = make_uint4(0u, 0u, 0u, 0u);
+      if (kc & 15) {
+        // the last 16-key group reaches past the image: mask its S columns, and
+        // zero its V rows (S is done, so the chunk's load landed; whole 128-byte rows)
+        const int past = 16 * groups - kc;
+        if (live) mask_columns(tsp + static_cast<uint32_t>(kc), past);
+        if (r < past * 8)
+          reinterpret_cast<uint4*>(&s.v[d & kDStage][0][0] + g * 32 * d_blocks(d) * HD)[kc * 8 + r] = make_uint4(0u, 0u, 0u, 0u);
         fence_proxy_async_smem();
       }
       if (live) {
-        uint32_t s0[32], s1[32];
-        tmem_ld32(tsp, s0);
-        tmem_ld32(tsp + 32u, s1);
+        const int blocks = groups >> 1;                  // 32 columns each; then half a block
+        const uint32_t tail = tsp + 32u * static_cast<uint32_t>(blocks);
+        const bool first = (d & kDFirst) != 0;
+        // the maximum is formed by the loads themselves
+        float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+        uint32_t sv[KC];                                 // read again below, 32 at a time
+#pragma unroll
+        for (int i = 0; i < KC / 32; ++i)
+          if (i < blocks)
+            tmem_ld_max32(tsp + 32u * i, *reinterpret_cast<uint32_t(*)[32]>(&sv[32 * i]), mx[i]);
+        if (groups & 1) {
+          uint32_t a[16];
+          tmem_ld_max16(tail, a, mx[3]);
+        }
         tmem_ld_wait();
-        mask_tail(s0, kh);
-        mask_tail(s1, kh - 32);
-        const float mc = max32(s1, max32(s0, -INFINITY)) * scale_log2;
-        // reference maximum: set on the unit's first chunk, raised past 2^8
-        bool rescale = false;
+        const float mc = max3f(mx[0], mx[1], fmaxf(mx[2], mx[3])) * scale_log2;
         float alpha = 1.f;
-        if (d & kDUFirst) {
+        if (first) {
           m_ref = mc;
           l = 0.f;
-        } else {
-          const bool need = mc > m_ref + kRescaleLog2;
-          rescale = __any_sync(0xffffffffu, need) != 0;
-          if (need) {
-            alpha = ex2_approx(m_ref - mc);
-            l *= alpha;
-            m_ref = mc;
-          }
+        } else if (mc > m_ref + kRescaleLog2) {
+          alpha = ex2_approx(m_ref - mc);
+          l *= alpha;
+          m_ref = mc;
         }
-        // P over the first 32 of the half's own S columns, already read
-        exp32_pack(s0, scale_log2, -m_ref, l);
-        tmem_st16(tsp, lo16(s0));
-        if (kh > 32) {
-          exp32_pack(s1, scale_log2, -m_ref, l);
-          tmem_st16(tsp + 16u, lo16(s1));
-        }
-        if (rescale) {
-          // O_h holds the unit's earlier chunks once their PVs (step j - 1) are
-          // done: bring the row to the raised reference before this chunk's PV
-          const int pb = (j - 1) % kSpBufs;
-          if (!mbar_wait_warp_sleep(&s.p_free[pb], static_cast<uint32_t>((j - 1) / kSpBufs) & 1u,
-                                    abort, kSleepNs))
-            return false;
-          tc_fence_after();
+        // a chunk of -infinities alone (only from infinite inputs) weighs nothing
+        const float neg_m = m_ref == -INFINITY ? 0.f : -m_ref;
+        const uint64_t nm = f2_pack(neg_m, neg_m);
+        uint64_t l0 = f2_pack(l, 0.f), l1 = f2_pack(0.f, 0.f);
 #pragma unroll 1
-          for (int q = 0; q < 2; ++q) {
-            const uint32_t to = tmem + lane_sel + tmem_o(h, (d & kDUPar) ? 1 : 0) + 32u * q;
-            uint32_t o[32];
-            tmem_ld32(to, o);
+        for (int i = 0; i < blocks; ++i) {
+          uint32_t a[32], p[16];
+          tmem_ld32(tsp + 32u * i, a);
+          tmem_ld_wait();
+          exp_pack<32>(a, p, sc, nm, l0, l1);
+          tmem_st16(tsp + 16u * i, p);                   // over columns already read
+        }
+        if (groups & 1) {
+          uint32_t a[16], p[8];
+          tmem_ld16(tail, a);
+          tmem_ld_wait();
+          exp_pack<16>(a, p, sc, nm, l0, l1);
+          tmem_st8(tsp + 16u * blocks, p);
+        }
+        float s0, s1;
+        f2_unpack(f2_add(l0, l1), s0, s1);
+        l = s0 + s1;
+        if (__any_sync(0xffffffffu, alpha != 1.f)) {
+          // O holds the chunks before this one once their PV is done: bring it
+          // to the raised reference before this chunk's PV
+          if (!wait_warp(&s.p_free[g][b ^ 1], ((j - 1) >> 1) & 1, abort)) return false;
+          tc_fence_after();
+          const uint32_t to = tmem + lane_sel + tmem_o(g);
+#pragma unroll 1
+          for (int h = 0; h < 4; ++h) {
+            uint32_t o[16];
+            tmem_ld16(to + 16u * h, o);
             tmem_ld_wait();
 #pragma unroll
-            for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-            tmem_st16(to, lo16(o));
-            tmem_st16(to + 16u, *reinterpret_cast<const uint32_t(*)[16]>(&o[16]));
+            for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+            tmem_st16(to + 16u * h, o);
           }
         }
+        tmem_st_wait();
       }
-      tmem_st_wait();
-      if (d & (h == 0 ? kDLast0 : kDLast1)) {
-        s.lm[d_slot(d)][h][r] = make_float2(l, m_ref);
-        warp_arrive(&s.l_full[d_slot(d)][h]);
+      if (d & kDLast) s.lsum[g][u & 3][r] = l;
+      warp_arrive(&s.p_full[g][b]);
+      if (d & kDLast) {
+        if (lane == 0) mbar_arrive(&s.l_full[g][u & 3]);
+        ++u;
       }
-      warp_arrive(&s.p_full[b][h]);
       return true;
     };
     for (int j = 0;; ++j) {
       const int i = j % kDescRing;
-      if (!mbar_wait_warp_sleep(&s.sd_full[i], (j / kDescRing) & 1, abort, kSleepNs)) break;
+      if (!wait_warp(&s.sd_full[i], (j / kDescRing) & 1, abort)) break;
       const uint32_t d = s.sdesc[i];
       __syncwarp();
       if (lane == 0) mbar_arrive(&s.sd_empty[i]);
       if ((d & kDEnd) || !step(j, d)) break;
     }
-  } else if (warp >= kEpiWarp0) {
-    // ---------------- epilogue: merge the halves, O / row sum, four rows per store ----------------
+  } else {
+    // ---------------- epilogue: O / row sum ----------------
+    setmaxnreg_dec<kOtherRegs>();
     const int quarter = warp & 3;
     const int r = quarter * 32 + lane;
     const uint32_t lane_sel = static_cast<uint32_t>(quarter * 32) << 16;
-    uint4* const stage = s.ostage[warp - kEpiWarp0];
-    uint32_t opar = 0u;            // o_done phase parity, bit 2 * h + unit parity
-    uint32_t lpar = 0u;            // l_full phase parity, bit 2 * slot + h
+    const bool whole = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;   // 32-byte stores
+#pragma unroll 1
     for (int u = 0;; ++u) {
       const int i = u % kUnitRing;
       // one descriptor per unit, then an end marker
-      if (!mbar_wait_warp_sleep(&s.ud_full[i], (u / kUnitRing) & 1, abort, kSleepNs)) break;
+      if (!wait_warp(&s.ud_full[i], (u / kUnitRing) & 1, abort)) break;
       const uint32_t row0 = s.urow[i], hd = s.uhead[i];
       __syncwarp();
+      if (lane == 0) mbar_arrive(&s.ud_empty[i]);
       if (hd == 0xFFFFFFFFu) break;
-      const int rows = static_cast<int>((hd >> 16) & 0xFFu), head = static_cast<int>(hd & 0xFFFFu);
-      const uint32_t gm = (hd >> 24) & 3u;
+      const int rows = static_cast<int>(hd >> 16), head = static_cast<int>(hd & 0xFFFFu);
       bool ok = true;
-      for (int g = 0; g < 2 && ok; ++g) {
-        if (!(gm & (1u << g))) continue;
-        ok = mbar_wait_warp_sleep(&s.o_done[g][u & 1], (opar >> (2 * g + (u & 1))) & 1u, abort,
-                                  kSleepNs) &&
-             mbar_wait_warp_sleep(&s.l_full[i][g], (lpar >> (2 * i + g)) & 1u, abort, kSleepNs);
-        opar ^= 1u << (2 * g + (u & 1));
-        lpar ^= 1u << (2 * i + g);
-      }
-      if (!ok) break;
-      tc_fence_after();
-      const bool live = quarter * 32 < rows;
-      if (live) {
-        // weights of the two partial results in a common frame
-        // (only the halves the unit used are read: the other slot is stale)
-        float a0 = 0.f, a1 = 0.f;
-        if (gm == 3u) {
-          const float2 lm0 = s.lm[i][0][r], lm1 = s.lm[i][1][r];
-          const float mm = fmaxf(lm0.y, lm1.y);
-          a0 = ex2_approx(lm0.y - mm);
-          a1 = ex2_approx(lm1.y - mm);
-          const float inv = 1.0f / (a0 * lm0.x + a1 * lm1.x);
-          a0 *= inv;
-          a1 *= inv;
-        } else if (gm == 1u) {
-          a0 = 1.0f / s.lm[i][0][r].x;
-        } else {
-          a1 = 1.0f / s.lm[i][1][r].x;
-        }
+#pragma unroll 1
+      for (int g = 0; g < 2; ++g) {
+        if (!(ok = wait_warp(&s.l_full[g][u & 3], (u >> 2) & 1, abort))) break;
+        const bool live = quarter * 32 < rows && head + g < heads;   // warp-uniform
+        const float inv = live ? 1.0f / s.lsum[g][u & 3][r] : 1.f;
+        if (!(ok = wait_warp(&s.o_done[g], u & 1, abort))) break;
+        tc_fence_after();
+        uint16_t* const dst = out + static_cast<size_t>(row0 + r) * dim + (head + g) * HD;
 #pragma unroll 1
         for (int h = 0; h < 2; ++h) {
-          uint32_t oa[32], ob[32];
-          if (gm & 1u) tmem_ld32(tmem + lane_sel + tmem_o(0, u & 1) + 32u * h, oa);
-          if (gm & 2u) tmem_ld32(tmem + lane_sel + tmem_o(1, u & 1) + 32u * h, ob);
-          tmem_ld_wait();
-          if (h == 1) {
-            // all of O is in registers: the accumulators are free for the next unit
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) {
-              if (gm & 1u) mbar_arrive(&s.o_free[0][u & 1]);
-              if (gm & 2u) mbar_arrive(&s.o_free[1][u & 1]);
+          uint32_t o[32], w[16];
+          if (live) {
+            tmem_ld32(tmem + lane_sel + tmem_o(g) + 32u * h, o);
+            tmem_ld_wait();
+          }
+          if (h == 1) warp_arrive(&s.o_free[g]);
+          if (live && r < rows) {
+#pragma unroll
+            for (int e = 0; e < 16; ++e)
+              w[e] = pack_bf16x2(__uint_as_float(o[2 * e]) * inv,
+                                 __uint_as_float(o[2 * e + 1]) * inv);
+            uint32_t* const d = reinterpret_cast<uint32_t*>(dst + 32 * h);
+            if (whole) {
+              st_global_32(d, &w[0]);
+              st_global_32(d + 8, &w[8]);
+            } else {
+#pragma unroll
+              for (int c = 0; c < 4; ++c)
+                reinterpret_cast<uint4*>(d)[c] =
+                    make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
             }
           }
-          float v[32];
-          if (gm == 3u) {
-#pragma unroll
-            for (int e = 0; e < 32; ++e)
-              v[e] = fmaf(__uint_as_float(oa[e]), a0, __uint_as_float(ob[e]) * a1);
-          } else if (gm == 1u) {
-#pragma unroll
-            for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(oa[e]) * a0;
-          } else {
-#pragma unroll
-            for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(ob[e]) * a1;
-          }
-#pragma unroll
-          for (int c = 0; c < 4; ++c)
-            stage[lane * 8 + ((4 * h + c) ^ (lane & 7))] =
-                make_uint4(pack_bf16x2(v[c * 8 + 0], v[c * 8 + 1]),
-                           pack_bf16x2(v[c * 8 + 2], v[c * 8 + 3]),
-                           pack_bf16x2(v[c * 8 + 4], v[c * 8 + 5]),
-                           pack_bf16x2(v[c * 8 + 6], v[c * 8 + 7]));
         }
       }
-      // the unit's slot is free again (and O, if this warp's rows were dead)
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) {
-        if (!live) {
-          if (gm & 1u) mbar_arrive(&s.o_free[0][u & 1]);
-          if (gm & 2u) mbar_arrive(&s.o_free[1][u & 1]);
-        }
-        mbar_arrive(&s.ud_empty[i]);
-      }
-      if (live) {
-        __syncwarp();
-        const int c = lane & 7;
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          const int row = 4 * t + (lane >> 3);             // of this warp's 32
-          if (quarter * 32 + row < rows)
-            *reinterpret_cast<uint4*>(out + static_cast<size_t>(row0 + quarter * 32 + row) * dim +
-                                      head * HD + c * 8) = stage[row * 8 + (c ^ (row & 7))];
-        }
-        __syncwarp();
-      }
+      if (!ok) break;
     }
   }
 
@@ -553,56 +742,42 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (threadIdx.x == 0) {
       record_status(status, DORA_ERR_TIMEOUT);
       // let the last TMA load of every buffer land (earlier ones were consumed)
-      for (int c = max(0, s.q_issued - 2); c < s.q_issued; ++c)
-        mbar_wait_limited(&s.q_full[c & 1], (c >> 1) & 1, 100ull * 1000 * 1000);
+      for (int u = max(0, s.q_issued - 2); u < s.q_issued; ++u)
+        mbar_wait_limited(&s.q_full[u & 1], (u >> 1) & 1, 100ull * 1000 * 1000);
       for (int c = max(0, s.kv_issued - kStages); c < s.kv_issued; ++c)
         mbar_wait_limited(&s.kv_full[c % kStages], (c / kStages) & 1, 100ull * 1000 * 1000);
     }
     __syncthreads();
   }
-  if (warp == 1) {
+  if (warp == 3) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);
   }
 }
 
-}  // namespace split
 }  // namespace attn
 
-cudaError_t encode_qkv_maps(attn::QkvMaps* mp, const uint16_t* qkv, int32_t t_cap, int32_t heads) {
-  const uint64_t row = static_cast<uint64_t>(3) * heads * attn::HD;
-  CUtensorMap* maps[4] = {&mp->m128, &mp->m64, &mp->m32, &mp->m16};
-  for (int i = 0; i < 4; ++i)
-    if (encode_tmap_2d_bf16(maps[i], qkv, row, static_cast<uint64_t>(t_cap), row * 2, attn::HD,
-                            static_cast<uint32_t>(attn::KC >> i)) != 0)
-      return cudaErrorInvalidValue;
-  return cudaSuccess;
-}
-
-// Images of up to 256 tokens have at most two key chunks, whose loads the
-// two query tiles share: there one accumulator per query row (and three S/P
-// buffers) measured faster; longer images run the per-key-half kernel above.
 cudaError_t launch_varlen_attn(const uint16_t* qkv, const int32_t* cu, int32_t batch,
                                int32_t max_seqlen, int32_t t_cap, int32_t heads, float scale,
                                uint16_t* out, int32_t* status, cudaStream_t stream) {
   if (batch == 0 || t_cap == 0 || max_seqlen == 0) return cudaSuccess;
   attn::QkvMaps mp;
-  cudaError_t e = encode_qkv_maps(&mp, qkv, t_cap, heads);
+  for (int i = 0; i < attn::BQ / 32; ++i)
+    if (encode_tmap_heads(&mp.m[i], qkv, static_cast<uint64_t>(t_cap),
+                          static_cast<uint64_t>(3) * heads, 32u * (i + 1)) != 0)
+      return cudaErrorInvalidValue;
+  const size_t smem = sizeof(attn::Smem);
+  const cudaError_t e =
+      cudaFuncSetAttribute(attn::varlen_attn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  const long long ihs = static_cast<long long>(batch) * heads;
-  if (ihs > 0x7fffffffLL) return cudaErrorInvalidValue;
-  const float scale_log2 = scale * 1.4426950408889634f;
-  if (max_seqlen <= 2 * attn::KC)
-    return launch_varlen_attn_exchange(mp, cu, batch, max_seqlen, t_cap, heads, scale_log2, out,
-                                       status, stream);
-  const size_t smem = sizeof(attn::split::Smem);
-  e = cudaFuncSetAttribute(attn::split::varlen_attn_kernel,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (e != cudaSuccess) return e;
+  const long long units = static_cast<long long>(batch) * ((heads + 1) / 2) *
+                          ((max_seqlen + attn::BQ - 1) / attn::BQ);
+  if (units > 0x7fffffffLL) return cudaErrorInvalidValue;
   const long long cap = num_sms();
-  const int grid = static_cast<int>(ihs < cap ? ihs : cap);
-  return launch_pdl(attn::split::varlen_attn_kernel, dim3(grid), dim3(attn::kThreads), smem,
-                    stream, mp, cu, batch, max_seqlen, t_cap, heads, scale_log2, out, status);
+  const int grid = static_cast<int>(units < cap ? units : cap);
+  return launch_pdl(attn::varlen_attn_kernel, dim3(grid), dim3(attn::kThreads), smem, stream, mp,
+                    cu, batch, max_seqlen, t_cap, heads, scale * 1.4426950408889634f, out, status);
 }
 
 }  // namespace dora

@@ -129,6 +129,10 @@ cudaError_t launch_varlen_attn(const uint16_t* qkv, const int32_t* cu, int32_t b
 int encode_tmap_2d_bf16(void* map, const void* base, uint64_t inner, uint64_t outer,
                         uint64_t row_pitch_bytes, uint32_t box_inner, uint32_t box_outer,
                         int swizzle_bytes = 128);
+// Tensor map of a row-major bf16 [rows, heads * 64] matrix as [heads][rows][64],
+// with boxes of box_rows rows of two neighbouring heads (128-byte swizzle).
+int encode_tmap_heads(void* map, const void* base, uint64_t rows, uint64_t heads,
+                      uint32_t box_rows);
 
 int num_sms();
 

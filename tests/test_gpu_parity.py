@@ -814,6 +814,41 @@ def test_attention_range_split_over_many_images(mix):
     _check_attn(lens, heads, 24)
 
 
+@pytest.mark.parametrize("heads", [1, 3, 4])
+def test_attention_chunk_edges_with_odd_and_even_head_counts(heads):
+    """Lengths on both sides of the 16-, 32- and 96-key steps and of the
+    query tile, with a last head that has no partner (odd head counts) and an
+    output that is 16- but not 32-byte aligned."""
+    lens = np.array([15, 32, 47, 48, 49, 95, 96, 97, 112, 113, 160, 191, 192, 193, 288, 289])
+    _check_attn(lens, heads, 25)
+    cu = O.cu_from_counts(lens)
+    t = int(cu[-1])
+    qkv = S.f32_to_bf16_bits(np.random.default_rng(26).standard_normal((t, 3 * heads * 64)))
+    buf = torch.full((t * heads * 64 + 16,), 9.0, dtype=torch.bfloat16, device=dev())
+    off = 8 if buf.data_ptr() % 32 == 0 else 16
+    out = buf[off:off + t * heads * 64].view(t, heads * 64)
+    assert out.data_ptr() % 32 == 16
+    P.dora_varlen_attn(bf(qkv), i32(cu), int(lens.max()), heads, out)
+    torch.cuda.synchronize()
+    assert_close(f64(out), O.varlen_attention(qkv, cu, heads), "attn at a 16-byte boundary")
+    assert torch.all(buf[:off] == 9.0) and torch.all(buf[off + t * heads * 64:] == 9.0)
+
+
+def test_attention_first_chunk_of_minus_infinities():
+    """Logits of -inf (an infinite key component) in the whole first key
+    chunk weigh nothing; the later chunk's keys get the weight."""
+    lens, heads = np.array([150, 150]), 2
+    rng = np.random.default_rng(27)
+    cu = O.cu_from_counts(lens)
+    x = rng.standard_normal((int(cu[-1]), 3 * heads * 64))
+    x[:, 0:heads * 64:64] = np.abs(x[:, 0:heads * 64:64]) + 0.5          # q's first component
+    qkv = S.f32_to_bf16_bits(x)
+    qkv[cu[0]:cu[0] + 96, heads * 64:2 * heads * 64:64] = 0xFF80          # image 0's first 96 keys
+    out, st = _run_attn(qkv, cu, heads, 150)
+    assert st == 0
+    assert_close(f64(out), O.varlen_attention(qkv, cu, heads), "attn with -inf logits")
+
+
 def test_attention_matches_dense_when_unpruned():
     """k = 0: packed attention equals dense batched attention (torch SDPA on
     the same bf16 values, fp64) on the GPU path too."""
