@@ -47,6 +47,8 @@ __global__ void __launch_bounds__(kThreads)
                      int k_cap, int32_t* __restrict__ order, float* __restrict__ keys_out,
                      int32_t* status) {
   __shared__ uint32_t keys[kMaxVisual];
+  pdl_trigger();
+  pdl_wait();
   const int img = blockIdx.x;
   const int lo = cu[img], hi = cu[img + 1];
   int32_t* out = order + static_cast<size_t>(img) * k_cap;
@@ -126,6 +128,8 @@ __global__ void __launch_bounds__(kThreads)
   __shared__ float lt[kMaxVisual];        // L_t, then P_t
   __shared__ Lse part[kThreads / 32];
   __shared__ int bad;
+  pdl_trigger();
+  pdl_wait();
   const int img = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int lo = cu[img], hi = cu[img + 1];
   int n = hi - lo - 1;
@@ -250,6 +254,8 @@ __global__ void __launch_bounds__(kScanThreads)
   __shared__ int warp_fit[kScanThreads / 32];
   __shared__ long long carry;
   __shared__ int last_fit;
+  pdl_trigger();
+  pdl_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (cu_out != cu)
     for (int i = threadIdx.x; i <= batch; i += blockDim.x) cu_out[i] = cu[i];
@@ -313,6 +319,8 @@ __global__ void branch_rows_kernel(uint4* __restrict__ x, int32_t* __restrict__ 
                                    float2* __restrict__ mv, const int32_t* __restrict__ cu_out,
                                    int batch, const int32_t* __restrict__ src, int nb, int t_cap,
                                    int d8) {
+  pdl_trigger();
+  pdl_wait();
   const int warps = gridDim.x * (blockDim.x >> 5);
   const int lane = threadIdx.x & 31;
   const int r0 = cu_out[batch], r1 = min(cu_out[batch + nb], t_cap);
@@ -333,15 +341,204 @@ __global__ void branch_rows_kernel(uint4* __restrict__ x, int32_t* __restrict__ 
   }
 }
 
+// Branching up to kFusedBranches sequences in one launch: CTA (p, s) forms
+// sequence s's place itself (the lengths before it, summed by the block) and
+// copies part p of its rows, which are contiguous on both sides, so the copy is
+// one straight stream with four 16-byte loads a thread in flight.  HBM-bound.
+// Against the scan kernel followed by a warp per row (a binary search for the
+// row's sequence before each 1.5 KB copy): 256 sequences, 77 MB each way, 42.8 us
+// in two launches (device time) -> 22.8 us, 6.9 TB/s (part of it from L2).
+constexpr int kFusedBranches = 4096;
+constexpr int kBranchThreads = 256;
+constexpr int kBranchInFlight = 4;
+
+__device__ __forceinline__ long long branch_len(const int32_t* cu, int batch, const int32_t* src,
+                                                int t) {
+  const int b = src[t];
+  if (b < 0 || b >= batch) return 0;
+  const int len = cu[b + 1] - cu[b];
+  return len > 0 ? len : 0;
+}
+
+// Sum over the block; every thread gets it.
+__device__ __forceinline__ long long block_sum(long long v, long long* scratch) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = v;
+  __syncthreads();
+  long long t = 0;
+  for (int w = 0; w < kBranchThreads / 32; ++w) t += scratch[w];
+  return t;
+}
+
+__global__ void __launch_bounds__(kBranchThreads)
+    branch_kernel(uint4* x, int32_t* ids, float2* mv, const int32_t* cu, int batch,
+                  const int32_t* __restrict__ src, int nb, int t_cap, int d8, int32_t* cu_out,
+                  int32_t* len_out, int32_t* status) {
+  __shared__ long long scratch[kBranchThreads / 32];
+  __shared__ long long ends[kBranchThreads];
+  pdl_trigger();
+  pdl_wait();
+  const int sq = blockIdx.y, part = blockIdx.x;
+  const int base = cu[batch];
+  long long before = 0;
+  for (int t = threadIdx.x; t < sq; t += kBranchThreads) before += branch_len(cu, batch, src, t);
+  const long long start = base + block_sum(before, scratch);
+  const long long len = branch_len(cu, batch, src, sq), end = start + len;
+  const bool fits = end <= t_cap;
+  if (part == 0) {
+    if (sq == 0 && cu_out != cu)
+      for (int i = threadIdx.x; i <= batch; i += kBranchThreads) cu_out[i] = cu[i];
+    const int b = src[sq];
+    if (threadIdx.x == 0 && (b < 0 || b >= batch)) record_status(status, DORA_ERR_DEVICE_BAD_COUNT);
+    long long at = end;
+    if (!fits) {
+      // the first sequence that does not fit in t_cap, and every one after it,
+      // gets length 0 (its end is the last end that fits); the ends only grow
+      const int per = (nb + kBranchThreads - 1) / kBranchThreads;
+      const int t0 = min(nb, static_cast<int>(threadIdx.x) * per), t1 = min(nb, t0 + per);
+      long long mine = 0;
+      for (int t = t0; t < t1; ++t) mine += branch_len(cu, batch, src, t);
+      __syncthreads();
+      ends[threadIdx.x] = mine;
+      __syncthreads();
+      long long e = base, last = base < t_cap ? base : t_cap;
+      for (int u = 0; u < static_cast<int>(threadIdx.x); ++u) e += ends[u];
+      for (int t = t0; t < t1; ++t) {
+        e += branch_len(cu, batch, src, t);
+        if (e <= t_cap) last = e;
+      }
+      __syncthreads();
+      ends[threadIdx.x] = last;
+      __syncthreads();
+      for (int u = 0; u < kBranchThreads; ++u) last = ends[u] > last ? ends[u] : last;
+      at = last;
+      if (threadIdx.x == 0 && len > 0) record_status(status, DORA_ERR_DEVICE_SEQLEN);
+    }
+    if (threadIdx.x == 0) {
+      cu_out[batch + 1 + sq] = static_cast<int32_t>(at);
+      if (len_out != nullptr) len_out[sq] = fits ? static_cast<int32_t>(len) : 0;
+    }
+  }
+  if (!fits || len == 0) return;
+  const size_t from = static_cast<size_t>(cu[src[sq]]), to = static_cast<size_t>(start);
+  if (part == static_cast<int>(gridDim.x) - 1)
+    for (int r = threadIdx.x; r < static_cast<int>(len); r += kBranchThreads) {
+      if (ids != nullptr) ids[to + r] = ids[from + r];
+      if (mv != nullptr) mv[to + r] = mv[from + r];
+    }
+  const uint4* xs = x + from * d8;
+  uint4* xd = x + to * d8;
+  const long long total = len * d8;
+  const long long c1 = total * (part + 1) / gridDim.x;
+  long long c = total * part / gridDim.x + threadIdx.x;
+  for (; c + (kBranchInFlight - 1) * kBranchThreads < c1; c += kBranchInFlight * kBranchThreads) {
+    uint4 v[kBranchInFlight];
+#pragma unroll
+    for (int e = 0; e < kBranchInFlight; ++e) v[e] = xs[c + e * kBranchThreads];
+#pragma unroll
+    for (int e = 0; e < kBranchInFlight; ++e) xd[c + e * kBranchThreads] = v[e];
+  }
+  for (; c < c1; c += kBranchThreads) xd[c] = xs[c];
+}
+
 // ---------------------------------------------------------------------------
-// Fidelity cost: one warp per shadow, fp32, two passes over the true classes.
+// Fidelity cost: one warp per shadow, fp32, over the true classes.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float bf(uint16_t v) { return __uint_as_float(static_cast<uint32_t>(v) << 16); }
 
+__device__ __forceinline__ float warp_max(float v) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
+  return v;
+}
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  return v;
+}
+
+// Rows of up to kHeldClasses classes, 16-byte aligned: both rows are read once,
+// 16 bytes at a time, into registers (the maximum, the sum and the divergence
+// all come from there).  Latency-bound: 768 rows of 1000 classes 15.5 us with
+// 2-byte loads read twice and a running log-sum-exp per element -> 6.1 us.
+constexpr int kHeldChunks = 4;                       // 8 classes a lane each
+constexpr int kHeldClasses = 32 * 8 * kHeldChunks;
+constexpr int kHeldThreads = 128;
+
+__global__ void __launch_bounds__(kHeldThreads)
+    kd_cost_held_kernel(const uint4* __restrict__ zn, const uint4* __restrict__ z,
+                        const int32_t* __restrict__ map, int shadows, int batch, int classes,
+                        int ld8, float inv_tau, float tau2, float* __restrict__ cost,
+                        int32_t* status) {
+  pdl_trigger();
+  pdl_wait();
+  const int sh = (blockIdx.x * kHeldThreads + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (sh >= shadows) return;
+  const int img = map != nullptr ? map[sh] : sh;
+  if (img < 0 || img >= batch) {
+    if (lane == 0) {
+      record_status(status, DORA_ERR_DEVICE_BAD_COUNT);
+      cost[sh] = NAN;
+    }
+    return;
+  }
+  uint4 qa[kHeldChunks], qb[kHeldChunks];
+#pragma unroll
+  for (int i = 0; i < kHeldChunks; ++i) {
+    const int c8 = lane + 32 * i;
+    if (8 * c8 < classes) {
+      qb[i] = z[static_cast<size_t>(sh) * ld8 + c8];
+      qa[i] = zn[static_cast<size_t>(img) * ld8 + c8];
+    }
+  }
+  float a[8 * kHeldChunks], b[8 * kHeldChunks];
+  float ma = -INFINITY, mb = -INFINITY;
+#pragma unroll
+  for (int i = 0; i < kHeldChunks; ++i) {
+    const uint32_t wa[4] = {qa[i].x, qa[i].y, qa[i].z, qa[i].w};
+    const uint32_t wb[4] = {qb[i].x, qb[i].y, qb[i].z, qb[i].w};
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const bool in = 8 * (lane + 32 * i) + e < classes;
+      const uint32_t va = (e & 1) ? wa[e >> 1] & 0xFFFF0000u : wa[e >> 1] << 16;
+      const uint32_t vb = (e & 1) ? wb[e >> 1] & 0xFFFF0000u : wb[e >> 1] << 16;
+      a[8 * i + e] = in ? __uint_as_float(va) * inv_tau : -INFINITY;
+      b[8 * i + e] = in ? __uint_as_float(vb) * inv_tau : -INFINITY;
+      ma = fmaxf(ma, a[8 * i + e]);
+      mb = fmaxf(mb, b[8 * i + e]);
+    }
+  }
+  ma = warp_max(ma);
+  mb = warp_max(mb);
+  float sa = 0.f, sb = 0.f;
+#pragma unroll
+  for (int e = 0; e < 8 * kHeldChunks; ++e) {
+    sa += __expf(a[e] - ma);
+    sb += __expf(b[e] - mb);
+  }
+  const float za = ma + __logf(warp_sum(sa)), zb = mb + __logf(warp_sum(sb));
+  float kl = 0.f;
+#pragma unroll
+  for (int i = 0; i < kHeldChunks; ++i)
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      if (8 * (lane + 32 * i) + e < classes) {
+        const float lpa = a[8 * i + e] - za, lpb = b[8 * i + e] - zb;
+        kl += __expf(lpa) * (lpa - lpb);
+      }
+  kl = warp_sum(kl);
+  if (lane == 0) cost[sh] = tau2 * kl;
+}
+
+// Any other row: two passes over the classes, a running log-sum-exp.
 __global__ void kd_cost_kernel(const uint16_t* __restrict__ zn, const uint16_t* __restrict__ z,
                                const int32_t* __restrict__ map, int shadows, int batch,
                                int classes, int ld, float inv_tau, float tau2,
                                float* __restrict__ cost, int32_t* status) {
+  pdl_trigger();
+  pdl_wait();
   const int sh = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (sh >= shadows) return;
   const int img = map != nullptr ? map[sh] : sh;
@@ -386,6 +583,8 @@ __global__ void step_rewards_kernel(const float* __restrict__ cost,
                                     const int32_t* __restrict__ blocks, int n_blocks, int batch,
                                     int depth, int n0, float a, float* __restrict__ reward,
                                     float* __restrict__ ret) {
+  pdl_trigger();
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= batch) return;
   const float inv = 25.f / (static_cast<float>(depth) * static_cast<float>(n0));
@@ -415,6 +614,7 @@ int device_or_error() {
   return DORA_OK;
 }
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+int launched(cudaError_t e) { return e == cudaSuccess ? DORA_OK : DORA_ERR_CUDA; }
 }  // namespace
 
 extern "C" {
@@ -429,9 +629,9 @@ int dora_pl_sample(const float* scores, const float* gumbel, const int32_t* cu, 
   const int e = device_or_error();
   if (e != DORA_OK) return e;
   if (batch == 0) return DORA_OK;
-  train::pl_sample_kernel<<<batch, train::kThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
-      scores, gumbel, cu, t_cap, k, k_cap, order, keys_out, status);
-  return cudaGetLastError() == cudaSuccess ? DORA_OK : DORA_ERR_CUDA;
+  return launched(launch_pdl(train::pl_sample_kernel, dim3(batch), dim3(train::kThreads), 0,
+                             reinterpret_cast<cudaStream_t>(stream), scores, gumbel, cu, t_cap, k,
+                             k_cap, order, keys_out, status));
 }
 
 int dora_pl_logprob(const float* scores, const int32_t* cu, int32_t batch, int32_t t_cap,
@@ -444,9 +644,9 @@ int dora_pl_logprob(const float* scores, const int32_t* cu, int32_t batch, int32
   const int e = device_or_error();
   if (e != DORA_OK) return e;
   if (batch == 0) return DORA_OK;
-  train::pl_logprob_kernel<<<batch, train::kThreads, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
-      scores, cu, t_cap, k, order, k_cap, logp, grad, dlogp, status);
-  return cudaGetLastError() == cudaSuccess ? DORA_OK : DORA_ERR_CUDA;
+  return launched(launch_pdl(train::pl_logprob_kernel, dim3(batch), dim3(train::kThreads), 0,
+                             reinterpret_cast<cudaStream_t>(stream), scores, cu, t_cap, k, order,
+                             k_cap, logp, grad, dlogp, status));
 }
 
 int dora_branch(dora_bf16* x, int32_t* ids, float* x_moments, const int32_t* cu, int32_t batch,
@@ -461,29 +661,43 @@ int dora_branch(dora_bf16* x, int32_t* ids, float* x_moments, const int32_t* cu,
   const int e = device_or_error();
   if (e != DORA_OK) return e;
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
-  train::branch_cu_kernel<<<1, train::kScanThreads, 0, stream>>>(cu, batch, src, n_branch, t_cap,
-                                                                  cu_out, len_out, status);
-  if (cudaGetLastError() != cudaSuccess) return DORA_ERR_CUDA;
-  if (n_branch == 0) return DORA_OK;
-  train::branch_rows_kernel<<<152 * 8, 256, 0, stream>>>(
-      reinterpret_cast<uint4*>(x), ids, reinterpret_cast<float2*>(x_moments), cu_out, batch, src,
-      n_branch, t_cap, dim / 8);
-  return cudaGetLastError() == cudaSuccess ? DORA_OK : DORA_ERR_CUDA;
+  if (n_branch > 0 && n_branch <= train::kFusedBranches) {
+    // about six CTAs a SM in all; a sequence's rows in at most 16 parts
+    const int parts = n_branch >= 912 ? 1 : (912 / n_branch < 16 ? 912 / n_branch : 16);
+    return launched(launch_pdl(train::branch_kernel, dim3(parts, n_branch),
+                               dim3(train::kBranchThreads), 0, stream,
+                               reinterpret_cast<uint4*>(x), ids,
+                               reinterpret_cast<float2*>(x_moments), cu, batch, src, n_branch,
+                               t_cap, dim / 8, cu_out, len_out, status));
+  }
+  // more sequences than every CTA should sum over (or none): one scan, then a warp per row
+  int rc = launched(launch_pdl(train::branch_cu_kernel, dim3(1), dim3(train::kScanThreads), 0,
+                               stream, cu, batch, src, n_branch, t_cap, cu_out, len_out, status));
+  if (rc != DORA_OK || n_branch == 0) return rc;
+  return launched(launch_pdl(train::branch_rows_kernel, dim3(152 * 8), dim3(256), 0, stream,
+                             reinterpret_cast<uint4*>(x), ids,
+                             reinterpret_cast<float2*>(x_moments), cu_out, batch, src, n_branch,
+                             t_cap, dim / 8));
 }
 
 int dora_kd_cost(const dora_bf16* z_native, const dora_bf16* z, const int32_t* shadow_image,
                  int32_t shadows, int32_t batch, int32_t classes, int32_t ld, float tau,
-                 float* cost, int32_t* status, dora_stream_t stream) {
+                 float* cost, int32_t* status, dora_stream_t stream_) {
   if (shadows < 0 || batch < 1 || classes < 1 || ld < classes || !(tau > 0.f))
     return DORA_ERR_INVALID_ARG;
   if (z_native == nullptr || z == nullptr || cost == nullptr) return DORA_ERR_INVALID_ARG;
   const int e = device_or_error();
   if (e != DORA_OK) return e;
   if (shadows == 0) return DORA_OK;
-  const int blocks = (shadows * 32 + 255) / 256;
-  train::kd_cost_kernel<<<blocks, 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
-      z_native, z, shadow_image, shadows, batch, classes, ld, 1.f / tau, tau * tau, cost, status);
-  return cudaGetLastError() == cudaSuccess ? DORA_OK : DORA_ERR_CUDA;
+  cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
+  if (classes <= train::kHeldClasses && ld % 8 == 0 && aligned16(z_native) && aligned16(z))
+    return launched(launch_pdl(
+        train::kd_cost_held_kernel, dim3((shadows + 3) / 4), dim3(train::kHeldThreads), 0, stream,
+        reinterpret_cast<const uint4*>(z_native), reinterpret_cast<const uint4*>(z), shadow_image,
+        shadows, batch, classes, ld / 8, 1.f / tau, tau * tau, cost, status));
+  return launched(launch_pdl(train::kd_cost_kernel, dim3((shadows * 32 + 255) / 256), dim3(256), 0,
+                             stream, z_native, z, shadow_image, shadows, batch, classes, ld,
+                             1.f / tau, tau * tau, cost, status));
 }
 
 int dora_step_rewards(const float* cost, const int32_t* removals, const int32_t* blocks,
@@ -495,10 +709,9 @@ int dora_step_rewards(const float* cost, const int32_t* removals, const int32_t*
     return DORA_ERR_INVALID_ARG;
   const int e = device_or_error();
   if (e != DORA_OK) return e;
-  train::step_rewards_kernel<<<(batch + 255) / 256, 256, 0,
-                               reinterpret_cast<cudaStream_t>(stream)>>>(
-      cost, removals, blocks, n_blocks, batch, depth, n0, a, reward, ret);
-  return cudaGetLastError() == cudaSuccess ? DORA_OK : DORA_ERR_CUDA;
+  return launched(launch_pdl(train::step_rewards_kernel, dim3((batch + 255) / 256), dim3(256), 0,
+                             reinterpret_cast<cudaStream_t>(stream), cost, removals, blocks,
+                             n_blocks, batch, depth, n0, a, reward, ret));
 }
 
 }  // extern "C"

@@ -436,6 +436,59 @@ def test_branch_scan_across_chunks_and_overflow():
     assert int(st.item()) == (O.DORA_ERR_DEVICE_SEQLEN if (lens[src][~fits] > 0).any() else 0)
 
 
+@pytest.mark.parametrize("nb", [1, 3, 255, 257, 4096, 4097])
+def test_branch_on_both_sides_of_the_one_launch_limit(nb):
+    """Up to 4096 appended sequences in one launch (every CTA summing the
+    lengths before its sequence, its rows in up to 16 parts), more by the
+    scan; row counts on both sides of the copy's 1024-piece strides; bad and
+    empty sources among them."""
+    rng = np.random.default_rng(16)
+    lens = rng.integers(0, 4, 64)
+    lens[:3] = [43, 0, 44]                                # 43 x 24 pieces > 1024 >= 42 x 24
+    cu = O.cu_from_counts(lens)
+    src = rng.integers(0, 64, nb).astype(np.int32)
+    src[-1] = 0
+    if nb > 2:
+        src[1] = 64                                       # out of range: flagged, no rows
+    n_of = np.where(src < 64, lens[np.minimum(src, 63)], 0)
+    want = np.concatenate([cu, cu[-1] + np.cumsum(n_of)])
+    d, t_cap = 192, int(want[-1]) + 1
+    x = S.f32_to_bf16_bits(rng.standard_normal((t_cap, d)))
+    ids = rng.integers(0, 1000, t_cap).astype(np.int32)
+    xt, it = bf(x), i32(ids)
+    cu_out = torch.zeros(65 + nb, dtype=torch.int32, device=dev())
+    lens_out = torch.zeros(nb, dtype=torch.int32, device=dev())
+    st = _status()
+    P.dora_branch(xt, i32(cu), i32(src), cu_out, ids=it, len_out=lens_out, status=st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == (5 if nb > 2 else 0)
+    assert np.array_equal(cu_out.cpu().numpy(), want)
+    assert np.array_equal(lens_out.cpu().numpy(), n_of)
+    rows = np.concatenate([np.arange(cu[s], cu[s + 1]) for s in src if s < 64]).astype(np.int64)
+    assert np.array_equal(bits(xt)[int(cu[-1]):int(want[-1])], x[rows])
+    assert np.array_equal(it.cpu().numpy()[int(cu[-1]):int(want[-1])], ids[rows])
+
+
+@pytest.mark.parametrize("classes,ld", [(1, 8), (7, 8), (8, 8), (257, 264), (1000, 1024),
+                                        (1023, 1024), (1024, 1024), (1025, 1032), (1000, 1004)])
+def test_kd_cost_held_and_streamed_rows(classes, ld):
+    """Rows held in registers (up to 1024 classes, 16-byte rows) and streamed
+    (more classes, or a row pitch that is no multiple of eight), the padding
+    ignored in both."""
+    rng = np.random.default_rng(17)
+    zn, z = (rng.standard_normal((n, ld)).astype(np.float32) * 3 for n in (3, 6))
+    z[:, classes:] = 60.0
+    zn_b, z_b = S.f32_to_bf16_bits(zn), S.f32_to_bf16_bits(z)
+    cost = torch.zeros(6, dtype=torch.float32, device=dev())
+    img = np.arange(6) % 3
+    P.dora_kd_cost(bf(zn_b), bf(z_b), cost, classes, shadow_image=i32(img), tau=3.0)
+    torch.cuda.synchronize()
+    got = cost.cpu().numpy().astype(np.float64)
+    for s in range(6):
+        ref = O.kd_cost(O.bf16_to_f64(zn_b)[img[s], :classes], O.bf16_to_f64(z_b)[s, :classes], 3.0)
+        assert abs(got[s] - ref) <= 1e-4 * (1 + ref), (s, got[s], ref)
+
+
 def test_pl_sample_and_logprob_at_the_largest_image():
     """2048 visual tokens (the kernels' shared-memory limit), k up to 2048."""
     cu = O.cu_from_counts([2049, 2049, 300])
