@@ -542,7 +542,8 @@ int dora_pruned_block_actor(const dora_bf16* x_in, const int32_t* cu_in, const i
  * (pos bf16 [g + 1, dim]; cls bf16 [dim]).  1 <= patch <= 64, 1 <= channels
  * <= 64, height and width multiples of patch, dim % 64 == 0.  The
  * convolution is a relayout (patchify) and one tcgen05 GEMM with fp32
- * accumulation (its output rounded to bf16), then the position add.  When
+ * accumulation whose epilogue adds bias, CLS and position embeddings in fp32
+ * (one rounding to bf16).  When
  * K = channels * patch^2 is not a multiple of 64 (DINOv2's 14-pixel patches:
  * K = 588) the patch matrix is K-padded with zero columns to the next
  * multiple of 64 and a zero-padded copy of w_pe is written to the workspace

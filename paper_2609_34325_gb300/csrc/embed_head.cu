@@ -1,9 +1,11 @@
 // The two ends of the ViT forward, which the paper's GFLOPs and throughput
 // include (App. E.4 "GFLOPs accounting"; backbones of Sec. 4.1):
 //   patch embedding   a patch x patch convolution with stride patch, as
-//                     patchify (a pure relayout) + one tcgen05 GEMM, then each
-//                     image's CLS token prepended and the position embeddings
-//                     added, into the packed token layout of the blocks;
+//                     patchify (a pure relayout) + one tcgen05 GEMM whose rows
+//                     are the packed tokens, CLS rows included, and whose
+//                     epilogue adds bias, CLS and position embeddings (a pass of
+//                     its own over the tokens: 18.5 us for 128 x 257 x 768, the
+//                     GEMM with it 38.2 us against 28.6);
 //   classifier head   the final LayerNorm on each image's CLS row and the
 //                     linear layer to the class logits (tcgen05 GEMM);
 //   LC1 head          DINOv2's readout (App. E.3): the final LayerNorm on every
@@ -29,51 +31,57 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<const uint32_t*>(&h);
 }
-__device__ __forceinline__ uint4 add8(uint4 a, uint4 b) {
-  return make_uint4(pack2(lo_f(a.x) + lo_f(b.x), hi_f(a.x) + hi_f(b.x)),
-                    pack2(lo_f(a.y) + lo_f(b.y), hi_f(a.y) + hi_f(b.y)),
-                    pack2(lo_f(a.z) + lo_f(b.z), hi_f(a.z) + hi_f(b.z)),
-                    pack2(lo_f(a.w) + lo_f(b.w), hi_f(a.w) + hi_f(b.w)));
-}
 
-// images [B, C, H, W] -> patches [B * gh * gw, C * p * p], 8 pixels (16 bytes)
-// a thread: row = b * gh * gw + (y / p) * gw + x / p, column = c * p * p +
-// (y % p) * p + x % p.  The weights [d, C, p, p] flattened are the GEMM's B.
+// The patch matrix has a row per token of the packed layout, image after image:
+// row b (g + 1) is image b's CLS row, zero (the GEMM's epilogue puts the CLS
+// token there), and row b (g + 1) + 1 + gy gw + gx its patch (gy, gx), column
+// c p^2 + dy p + dx.  So the GEMM's output rows are the tokens themselves.
+
+// p a multiple of 8: 8 pixels (16 bytes) a thread, twice as many where p is a
+// multiple of 16.  The weights [d, C, p, p] flattened are the GEMM's B.
+template <int V>
 __global__ void patchify_kernel(const uint4* __restrict__ img, int batch, int ch, int h, int w,
                                 int p, uint4* __restrict__ out) {
-  const int gw = w / p, gh = h / p;
-  const long long segs = static_cast<long long>(batch) * ch * h * (w / 8);
-  const int kcols8 = ch * p * p / 8;
-  for (long long s = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; s < segs;
-       s += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const int xs = static_cast<int>(s % (w / 8));
-    long long r = s / (w / 8);
-    const int y = static_cast<int>(r % h);
-    r /= h;
-    const int c = static_cast<int>(r % ch);
-    const int b = static_cast<int>(r / ch);
-    const int x = xs * 8;
-    const long long row = (static_cast<long long>(b) * gh + y / p) * gw + x / p;
-    const int col8 = (c * p * p + (y % p) * p + x % p) / 8;
-    out[row * kcols8 + col8] = img[s];
+  pdl_trigger();
+  pdl_wait();
+  const int gw = w / p, g = gw * (h / p), wv = w / (8 * V), kcols8 = ch * p * p / 8;
+  const uint32_t row_segs = static_cast<uint32_t>(h) * wv;      // V-vectors of a channel
+  const uint32_t segs = static_cast<uint32_t>(batch) * ch * row_segs;
+  const uint32_t zeros = static_cast<uint32_t>(batch) * (kcols8 / V);
+  for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < segs + zeros;
+       s += gridDim.x * blockDim.x) {
+    if (s >= segs) {                                            // CLS rows
+      const uint32_t z = s - segs, b = z / (kcols8 / V), c = z - b * (kcols8 / V);
+#pragma unroll
+      for (int v = 0; v < V; ++v)
+        out[static_cast<size_t>(b) * (g + 1) * kcols8 + c * V + v] = make_uint4(0u, 0u, 0u, 0u);
+      continue;
+    }
+    const uint32_t bc = s / row_segs, in = s - bc * row_segs;
+    const int y = in / wv, x = (in - y * wv) * 8 * V;
+    const int b = bc / ch, c = bc - b * ch, gy = y / p, gx = x / p;
+    const size_t row = static_cast<size_t>(b) * (g + 1) + 1 + gy * gw + gx;
+    const int col8 = (c * p * p + (y - gy * p) * p + x - gx * p) / 8;
+#pragma unroll
+    for (int v = 0; v < V; ++v) out[row * kcols8 + col8 + v] = __ldg(img + static_cast<size_t>(s) * V + v);
   }
 }
 
 // Any patch side: one thread writes 8 consecutive columns of one row of the
-// K-padded patch matrix [B gh gw, kpad] (2-byte gathers; columns >= C p^2 are
-// zero).  Column order as above: c * p * p + dy * p + dx.
+// K-padded patch matrix [B (g + 1), kpad] (2-byte gathers; columns >= C p^2 and
+// CLS rows are zero).
 __global__ void patchify_any_kernel(const uint16_t* __restrict__ img, int batch, int ch, int h,
                                     int w, int p, int kpad, uint4* __restrict__ out) {
-  const int gw = w / p, gh = h / p, pp = p * p, k = ch * pp, kp8 = kpad / 8;
-  const long long total = static_cast<long long>(batch) * gh * gw * kp8;
+  pdl_trigger();
+  pdl_wait();
+  const int gw = w / p, gh = h / p, g = gw * gh, pp = p * p, k = ch * pp, kp8 = kpad / 8;
+  const long long total = static_cast<long long>(batch) * (g + 1) * kp8;
   for (long long s = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; s < total;
        s += static_cast<long long>(gridDim.x) * blockDim.x) {
     const int c8 = static_cast<int>(s % kp8);
-    long long r = s / kp8;
-    const int gx = static_cast<int>(r % gw);
-    r /= gw;
-    const int gy = static_cast<int>(r % gh);
-    const long long b = r / gh;
+    const long long r = s / kp8, b = r / (g + 1);
+    const int tok = static_cast<int>(r - b * (g + 1)) - 1;      // -1: CLS
+    const int gy = tok / gw, gx = tok - gy * gw;
     uint32_t v[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
@@ -81,7 +89,7 @@ __global__ void patchify_any_kernel(const uint16_t* __restrict__ img, int batch,
 #pragma unroll
       for (int hlf = 0; hlf < 2; ++hlf) {
         const int col = c8 * 8 + 2 * e + hlf;
-        if (col < k) {
+        if (tok >= 0 && col < k) {
           const int c = col / pp, rem = col - c * pp, dy = rem / p, dx = rem - dy * p;
           const long long pix =
               ((b * ch + c) * h + gy * p + dy) * static_cast<long long>(w) + gx * p + dx;
@@ -97,61 +105,86 @@ __global__ void patchify_any_kernel(const uint16_t* __restrict__ img, int batch,
 // Even patch side (DINOv2's 14): one thread writes one 4-byte pixel pair of
 // the K-padded patch matrix, consecutive threads consecutive pairs of a
 // token row, so every store is coalesced; the pair (an even pair never
-// straddles two patches) is read from the image, pad pairs are zero.  All
-// counts fit in 32 bits (checked by the caller).
+// straddles two patches) is read from the image, pad pairs and CLS rows are
+// zero.  All counts fit in 32 bits (checked by the caller).
 __global__ void patchify_even_kernel(const uint32_t* __restrict__ img, int batch, int ch, int h,
                                      int w, int p, int kpad, uint32_t* __restrict__ out) {
+  pdl_trigger();
+  pdl_wait();
   const int gw = w / p, gh = h / p, p2 = p / 2, row2 = p * p2, k2 = ch * row2, w2 = w / 2;
-  const int kp2 = kpad / 2;
-  const int total = batch * gh * gw * kp2;
+  const int kp2 = kpad / 2, g = gw * gh;
+  const int total = batch * (g + 1) * kp2;
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < total; s += gridDim.x * blockDim.x) {
-    const int q = s % kp2, tok = s / kp2;
+    const int q = s % kp2, r = s / kp2, b = r / (g + 1), tok = r - b * (g + 1) - 1;
     uint32_t v = 0u;
-    if (q < k2) {
+    if (tok >= 0 && q < k2) {
       const int c = q / row2, rem = q - c * row2, dy = rem / p2, e = rem - dy * p2;
-      const int gx = tok % gw, t2 = tok / gw, gy = t2 % gh, b = t2 / gh;
+      const int gy = tok / gw, gx = tok - gy * gw;
       v = __ldg(img + (static_cast<size_t>((b * ch + c) * h + gy * p + dy) * w2 + gx * p2 + e));
     }
     out[s] = v;
   }
 }
 
+// Piece s (8 columns) of w [d, k] padded with zero columns to [d, kpad].
+__device__ __forceinline__ uint4 padded_piece(const uint16_t* __restrict__ w, int k, int kpad,
+                                              long long s) {
+  const int kp8 = kpad / 8, c8 = static_cast<int>(s % kp8);
+  const uint16_t* row = w + (s / kp8) * k;
+  uint32_t v[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int j = c8 * 8 + 2 * e;
+    v[e] = (j < k ? static_cast<uint32_t>(row[j]) : 0u) |
+           (j + 1 < k ? static_cast<uint32_t>(row[j + 1]) << 16 : 0u);
+  }
+  return make_uint4(v[0], v[1], v[2], v[3]);
+}
+
 // The same relayout with the patch side and channel count fixed at compile
 // time (DINOv2-B/14 on RGB), staged through shared memory: one block per
 // band of patches (image b, patch row gy).  The band's CH x P image rows are
 // read with coalesced 16-byte loads, then its gw token rows are written with
-// coalesced 16-byte stores, each 8-column piece gathered from shared memory
-// (column c P^2 + dy P + dx, zero past CH P^2).  Needs w % 8 == 0.
+// coalesced 16-byte stores, each 8-column piece gathered from shared memory as
+// four pixel pairs (P even: a pair never straddles two rows of a patch).  Needs
+// w % 8 == 0.  The blocks past the bands pad the weights [d, CH P^2] for the
+// GEMM, instead of a launch of their own.  128 images of 16 x 16 patches: 25.6 +
+// 5.7 us as two kernels with 2-byte gathers -> 17.4 us, 4.9 TB/s.
 template <int P, int CH>
 __global__ void __launch_bounds__(256)
-    patchify_band_kernel(const uint4* __restrict__ img, int gh, int gw, int h, int w,
-                         uint4* __restrict__ out) {
-  extern __shared__ uint16_t band[];                   // [CH][P][w]
+    patchify_band_kernel(const uint4* __restrict__ img, int batch, int gh, int gw, int h, int w,
+                         uint4* __restrict__ out, const uint16_t* __restrict__ wt, int d,
+                         uint4* __restrict__ wp) {
+  static_assert(P % 2 == 0, "pixel pairs");
+  extern __shared__ uint32_t band[];                   // [CH][P][w / 2]
   constexpr int kK = CH * P * P, kKp8 = (kK + 63) / 64 * 8;
+  pdl_trigger();
+  pdl_wait();
+  const int bands = batch * gh;
+  if (static_cast<int>(blockIdx.x) >= bands) {
+    const long long s = (blockIdx.x - bands) * 256LL + threadIdx.x;
+    if (s < static_cast<long long>(d) * kKp8) wp[s] = padded_piece(wt, kK, 8 * kKp8, s);
+    return;
+  }
   const int gy = blockIdx.x % gh, b = blockIdx.x / gh;
-  const int w8 = w / 8;
+  const int w8 = w / 8, w2 = w / 2;
   uint4* band4 = reinterpret_cast<uint4*>(band);
   for (int i = threadIdx.x; i < CH * P * w8; i += blockDim.x) {
     const int x8 = i % w8, r = i / w8, dy = r % P, c = r / P;
     band4[i] = __ldg(img + (static_cast<size_t>((b * CH + c) * h + gy * P + dy) * w8 + x8));
   }
+  uint4* dst = out + (static_cast<size_t>(b) * (gh * gw + 1) + 1 + gy * gw) * kKp8;
+  if (gy == 0)
+    for (int i = threadIdx.x; i < kKp8; i += blockDim.x) dst[i - kKp8] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
-  uint4* dst = out + static_cast<size_t>(blockIdx.x) * gw * kKp8;
   for (int i = threadIdx.x; i < gw * kKp8; i += blockDim.x) {
     const int gx = i / kKp8, c8 = i - gx * kKp8;
     uint32_t v[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      uint32_t pr = 0u;
-#pragma unroll
-      for (int hlf = 0; hlf < 2; ++hlf) {
-        const int col = c8 * 8 + 2 * e + hlf;
-        if (col < kK) {
-          const int c = col / (P * P), rem = col - c * (P * P), dy = rem / P, dx = rem - dy * P;
-          pr |= static_cast<uint32_t>(band[(c * P + dy) * w + gx * P + dx]) << (16 * hlf);
-        }
-      }
-      v[e] = pr;
+      const int col = c8 * 8 + 2 * e;
+      const int r = col / P, dx = col - r * P;         // r = c P + dy
+      v[e] = col < kK ? band[r * w2 + (gx * P + dx) / 2] : 0u;
     }
     dst[i] = make_uint4(v[0], v[1], v[2], v[3]);
   }
@@ -159,29 +192,11 @@ __global__ void __launch_bounds__(256)
 
 // w [d, k] -> [d, kpad] with zero columns k..kpad-1 (the GEMM's B for K-padded patches).
 __global__ void pad_cols_kernel(const uint16_t* __restrict__ w, int d, int k, int kpad,
-                                uint16_t* __restrict__ out) {
-  const long long total = static_cast<long long>(d) * kpad;
-  for (long long s = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; s < total;
-       s += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const int j = static_cast<int>(s % kpad);
-    out[s] = j < k ? w[(s / kpad) * k + j] : static_cast<uint16_t>(0);
-  }
-}
-
-// x0 row b * (g + 1) + j: j = 0 -> cls + pos[0]; else emb[b * g + j - 1] + pos[j].
-__global__ void assemble_kernel(const uint4* __restrict__ emb, const uint4* __restrict__ cls,
-                                const uint4* __restrict__ pos, int batch, int g, int dim8,
-                                uint4* __restrict__ x0) {
-  const long long total = static_cast<long long>(batch) * (g + 1) * dim8;
-  for (long long s = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; s < total;
-       s += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const int c = static_cast<int>(s % dim8);
-    const long long row = s / dim8;
-    const int j = static_cast<int>(row % (g + 1));
-    const long long b = row / (g + 1);
-    const uint4 base = j == 0 ? cls[c] : emb[(b * g + j - 1) * dim8 + c];
-    x0[s] = add8(base, pos[static_cast<long long>(j) * dim8 + c]);
-  }
+                                uint4* __restrict__ out) {
+  pdl_trigger();
+  pdl_wait();
+  const long long s = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
+  if (s < static_cast<long long>(d) * (kpad / 8)) out[s] = padded_piece(w, k, kpad, s);
 }
 
 // LayerNorm of each image's CLS row (row cu[i]) into u [batch, dim]: one warp
@@ -384,8 +399,12 @@ size_t dora_embed_workspace_size(int32_t batch, int32_t channels, int32_t height
   if (batch < 0 || channels <= 0 || patch <= 0 || height <= 0 || width <= 0 || dim <= 0) return 0;
   const size_t tok = static_cast<size_t>(batch) * (height / patch) * (width / patch);
   const size_t k = static_cast<size_t>(channels) * patch * patch, kpad = (k + 63) / 64 * 64;
-  return 256 + embed::up256(tok * kpad * 2) + embed::up256(tok * dim * 2) +
-         (kpad != k ? embed::up256(static_cast<size_t>(dim) * kpad * 2) : 0);
+  const size_t wp = kpad != k ? embed::up256(static_cast<size_t>(dim) * kpad * 2) : 0;
+  // the patch matrix with its CLS rows; never less than earlier versions asked for
+  // (patches and their embeddings)
+  const size_t now = embed::up256((tok + batch) * kpad * 2);
+  const size_t was = embed::up256(tok * kpad * 2) + embed::up256(tok * dim * 2);
+  return 256 + (now > was ? now : was) + wp;
 }
 
 int dora_patch_embed(const dora_bf16* images, int32_t batch, int32_t channels, int32_t height,
@@ -415,60 +434,68 @@ int dora_patch_embed(const dora_bf16* images, int32_t batch, int32_t channels, i
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   int32_t* status = reinterpret_cast<int32_t*>(ws);
   const int k = channels * patch * patch, kpad = (k + 63) / 64 * 64;
+  const long long rows = tok + batch;                  // a token row and a patch row each
   uint16_t* patches = reinterpret_cast<uint16_t*>(ws + 256);
-  uint16_t* emb = reinterpret_cast<uint16_t*>(ws + 256 + embed::up256(tok * kpad * 2));
   const uint16_t* w_gemm = w_pe;
-  if (patch % 8 == 0 && kpad == k) {
-    const long long segs = static_cast<long long>(batch) * channels * height * (width / 8);
-    embed::patchify_kernel<<<embed::grid_for(segs), 256, 0, stream>>>(
-        reinterpret_cast<const uint4*>(images), batch, channels, height, width, patch,
-        reinterpret_cast<uint4*>(patches));
+  const long long pixels = static_cast<long long>(batch) * channels * height * width;
+  if (patch % 8 == 0 && kpad == k && pixels < (1LL << 31) && rows * (k / 8) < (1LL << 31)) {
+    const int v = patch % 16 == 0 ? 2 : 1;
+    const long long items = pixels / (8 * v) + static_cast<long long>(batch) * (k / 8 / v);
+    if (launch_pdl(v == 2 ? embed::patchify_kernel<2> : embed::patchify_kernel<1>,
+                   dim3(embed::grid_for(items)), dim3(256), 0, stream,
+                   reinterpret_cast<const uint4*>(images), batch, channels, height, width, patch,
+                   reinterpret_cast<uint4*>(patches)) != cudaSuccess)
+      return DORA_ERR_CUDA;
   } else {
     // K padded to a multiple of the GEMM's 64-wide K step: zero patch columns
     // and a zero-padded copy of the weights in the workspace
-    uint16_t* wp = reinterpret_cast<uint16_t*>(ws + 256 + embed::up256(tok * kpad * 2) +
-                                               embed::up256(tok * dim * 2));
-    const long long items = tok * (kpad / 2);
+    uint16_t* wp = reinterpret_cast<uint16_t*>(ws + 256 + embed::up256(rows * kpad * 2));
+    const long long items = rows * (kpad / 2), pieces = static_cast<long long>(dim) * (kpad / 8);
     const int band_smem = 3 * 14 * width * 2;
+    bool padded = kpad == k;
     if (patch == 14 && channels == 3 && width % 8 == 0 && band_smem <= 160 * 1024 &&
-        static_cast<long long>(batch) * (height / patch) < (1LL << 31)) {
+        static_cast<long long>(batch) * (height / patch) + (pieces + 255) / 256 < (1LL << 31)) {
       auto kern = embed::patchify_band_kernel<14, 3>;
       if (band_smem > 48 * 1024 &&
           cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, band_smem) !=
               cudaSuccess)
         return DORA_ERR_CUDA;
-      kern<<<static_cast<unsigned>(batch * (height / patch)), 256, band_smem, stream>>>(
-          reinterpret_cast<const uint4*>(images), height / patch, width / patch, height, width,
-          reinterpret_cast<uint4*>(patches));
-    } else if (patch % 2 == 0 && items < (1LL << 31) &&
-               static_cast<long long>(batch) * channels * height * width / 2 < (1LL << 31)) {
-      embed::patchify_even_kernel<<<embed::grid_for(items), 256, 0, stream>>>(
-          reinterpret_cast<const uint32_t*>(images), batch, channels, height, width, patch, kpad,
-          reinterpret_cast<uint32_t*>(patches));
+      if (launch_pdl(kern,
+                     dim3(static_cast<unsigned>(batch * (height / patch) + (pieces + 255) / 256)),
+                     dim3(256), static_cast<size_t>(band_smem), stream,
+                     reinterpret_cast<const uint4*>(images), batch, height / patch, width / patch,
+                     height, width, reinterpret_cast<uint4*>(patches), w_pe, dim,
+                     reinterpret_cast<uint4*>(wp)) != cudaSuccess)
+        return DORA_ERR_CUDA;
+      padded = true;
+    } else if (patch % 2 == 0 && items < (1LL << 31) && pixels / 2 < (1LL << 31)) {
+      if (launch_pdl(embed::patchify_even_kernel, dim3(embed::grid_for(items)), dim3(256), 0,
+                     stream, reinterpret_cast<const uint32_t*>(images), batch, channels, height,
+                     width, patch, kpad, reinterpret_cast<uint32_t*>(patches)) != cudaSuccess)
+        return DORA_ERR_CUDA;
     } else {
-      const long long segs = tok * (kpad / 8);
-      embed::patchify_any_kernel<<<embed::grid_for(segs), 256, 0, stream>>>(
-          images, batch, channels, height, width, patch, kpad, reinterpret_cast<uint4*>(patches));
+      if (launch_pdl(embed::patchify_any_kernel, dim3(embed::grid_for(rows * (kpad / 8))),
+                     dim3(256), 0, stream, images, batch, channels, height, width, patch, kpad,
+                     reinterpret_cast<uint4*>(patches)) != cudaSuccess)
+        return DORA_ERR_CUDA;
     }
-    if (cudaGetLastError() != cudaSuccess) return DORA_ERR_CUDA;
-    if (kpad != k) {
-      embed::pad_cols_kernel<<<embed::grid_for(static_cast<long long>(dim) * kpad), 256, 0,
-                               stream>>>(w_pe, dim, k, kpad, wp);
-      w_gemm = wp;
-    }
+    if (!padded && launch_pdl(embed::pad_cols_kernel,
+                              dim3(static_cast<unsigned>((pieces + 255) / 256)), dim3(256), 0,
+                              stream, w_pe, dim, k, kpad, reinterpret_cast<uint4*>(wp)) !=
+                       cudaSuccess)
+      return DORA_ERR_CUDA;
+    if (kpad != k) w_gemm = wp;
   }
-  if (cudaGetLastError() != cudaSuccess) return DORA_ERR_CUDA;
+  // tokens: the convolution with bias, CLS and position embeddings in the epilogue
   LinearEpi ep;
   ep.bias = b_pe;
-  if (launch_linear(patches, static_cast<int32_t>(tok), nullptr, kpad, w_gemm, dim, DORA_EPI_BIAS,
-                    ep, emb, status, stream) != cudaSuccess)
-    return DORA_ERR_CUDA;
-  const long long total = static_cast<long long>(batch) * (g + 1) * (dim / 8);
-  embed::assemble_kernel<<<embed::grid_for(total), 256, 0, stream>>>(
-      reinterpret_cast<const uint4*>(emb), reinterpret_cast<const uint4*>(cls),
-      reinterpret_cast<const uint4*>(pos), batch, static_cast<int>(g), dim / 8,
-      reinterpret_cast<uint4*>(x0));
-  return cudaGetLastError() == cudaSuccess ? DORA_OK : DORA_ERR_CUDA;
+  ep.cls = cls;
+  ep.pos = pos;
+  ep.tokens = static_cast<int32_t>(g + 1);
+  return launch_linear(patches, static_cast<int32_t>(rows), nullptr, kpad, w_gemm, dim, kEpiTokens,
+                       ep, x0, status, stream) == cudaSuccess
+             ? DORA_OK
+             : DORA_ERR_CUDA;
 }
 
 size_t dora_head_workspace_size(int32_t batch, int32_t dim) {

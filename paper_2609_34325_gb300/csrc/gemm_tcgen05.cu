@@ -31,8 +31,10 @@
 //              which a TMA load brings the residual chunk while the tile's
 //              MMAs still run; the result is written over it in place (a
 //              long-K linear keeps two buffers a warp and reloads them within
-//              the tile, for one more stage).  The tile that straddles the
-//              live row count stores row by row.
+//              the tile, for one more stage).  The patch embedding's epilogue
+//              is the same with the position embeddings as the residual, boxes
+//              of one image's rows shared by every image.  The tile that
+//              straddles the live row count stores row by row.
 // The live row count M may come from device memory (rows left after a
 // deletion); tiles past it are never scheduled.  Every wait is bounded.
 #include <cuda.h>
@@ -80,7 +82,8 @@ struct Cfg {
   static constexpr int kChunks = kCols / 32;
   // chunks per TMEM load: two (64 registers) unless 16 warps cap registers at 96
   static constexpr int kBatch = kEpiWarps == 16 ? 1 : (kChunks < 2 ? kChunks : 2);
-  static constexpr bool kResTma = EPI == DORA_EPI_BIAS_RESIDUAL || EPI == kEpiResidualLongK;
+  static constexpr bool kResTma =
+      EPI == DORA_EPI_BIAS_RESIDUAL || EPI == kEpiResidualLongK || EPI == kEpiTokens;
   // staging buffers per epilogue warp: one per chunk for the residual (its
   // TMA load lands there; two for a long K), one with 16 warps or the folded
   // LayerNorm, else two
@@ -189,7 +192,7 @@ __device__ __forceinline__ void epilogue_math(const uint32_t (&r)[32], float (&v
                        f2_pack(d.z, d.w)),
                 v[4 * q + 2], v[4 * q + 3]);
     }
-  } else if (ep.bias != nullptr) {
+  } else if (EPI != kEpiTokens && ep.bias != nullptr) {
     const uint4* bp = reinterpret_cast<const uint4*>(ep.bias + gcol);
 #pragma unroll
     for (int q = 0; q < 4; ++q) add_bf16x8(v + 8 * q, __ldg(bp + q));
@@ -425,11 +428,20 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
     uint32_t res_par = 0;                         // their next completion parity
     // Residual chunk `c` of the warp's 32 rows from row0, column col0 on, into
     // staging buffer c % kBufs (whose previous store must have read it).
+    // The patch embedding's residual is its token's position embedding: the
+    // box starts at the first row's token, and lanes past the image's last
+    // token (where the box reads zeros) fetch theirs from the next image's start.
+    auto residual_row = [&](int row_, int gcol) {
+      const int r_ = EPI == kEpiTokens ? row_ % ep.tokens : row_;
+      return reinterpret_cast<const uint4*>((EPI == kEpiTokens ? ep.pos : ep.residual) +
+                                            static_cast<size_t>(r_) * N + gcol);
+    };
     auto load_residual = [&](int c, int row0, int col0) {
       const int b = c % kBufs;
       if (lane == 0) {
         mbar_arrive_expect_tx(&s.res_full[ew][b], kStageChunk * 2);
-        tma_load_2d(s.out[ew][b], &tmR, &s.res_full[ew][b], col0 + c * 32, row0);
+        tma_load_2d(s.out[ew][b], &tmR, &s.res_full[ew][b], col0 + c * 32,
+                    EPI == kEpiTokens ? row0 % ep.tokens : row0);
       }
       res_pend |= 1u << b;
     };
@@ -501,6 +513,7 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
       const int row0 = mt * BM + q * 32;          // first row of this warp
       const int row = row0 + lane;
       const bool whole = row0 + 32 <= M;          // all 32 rows live: TMA store
+      const bool past_image = EPI == kEpiTokens && row0 % ep.tokens + lane >= ep.tokens;
       float neg_mean = 0.f, rstd = 0.f;           // folded LayerNorm of this row
       if constexpr (C::kLn) {
         neg_mean = -mv.x;
@@ -543,6 +556,18 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
           epilogue_math<EPI>(r[c], v, ep, gcol, neg_mean, rstd,
                              &s.cd[ew][0][((cb + c) * 32) % C::kCdCols],
                              &s.cd[ew][1][((cb + c) * 32) % C::kCdCols]);
+          if constexpr (EPI == kEpiTokens) {
+            // bias, or the CLS token, whose row takes nothing from its (zero) patch
+            const bool is_cls = row % ep.tokens == 0;
+            const uint16_t* add = is_cls ? ep.cls : ep.bias;
+#pragma unroll
+            for (int e = 0; e < 32; ++e) v[e] = is_cls ? 0.f : v[e];
+            if (add != nullptr) {
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                add_bf16x8(v + 8 * j, __ldg(reinterpret_cast<const uint4*>(add + gcol) + j));
+            }
+          }
           if (whole) {
             // row `lane` of the 32x32 chunk, 64-byte swizzle: 16-byte piece j
             // of row l sits at piece j ^ ((l >> 1) & 3).
@@ -571,10 +596,12 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
 #pragma unroll
               for (int j = 0; j < 4; ++j)
                 add_bf16x8(v + 8 * j,
-                           *reinterpret_cast<const uint4*>(rowp + ((j ^ ((lane >> 1) & 3)) << 4)));
+                           past_image ? __ldg(residual_row(row, gcol) + j)
+                                      : *reinterpret_cast<const uint4*>(
+                                            rowp + ((j ^ ((lane >> 1) & 3)) << 4)));
             }
             pack_row(v, o);
-            if constexpr (C::kResTma)
+            if constexpr (C::kResTma && EPI != kEpiTokens)
               if (ep.stats_out != nullptr) emit_moments(o, row, gcol);
 #pragma unroll
             for (int j = 0; j < 4; ++j)
@@ -598,13 +625,12 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
             }
           } else if (row < M) {
             if constexpr (C::kResTma) {
-              const uint4* rp =
-                  reinterpret_cast<const uint4*>(ep.residual + static_cast<size_t>(row) * N + gcol);
+              const uint4* rp = residual_row(row, gcol);
 #pragma unroll
               for (int j = 0; j < 4; ++j) add_bf16x8(v + 8 * j, __ldg(rp + j));
             }
             pack_row(v, o);
-            if constexpr (C::kResTma)
+            if constexpr (C::kResTma && EPI != kEpiTokens)
               if (ep.stats_out != nullptr) emit_moments(o, row, gcol);
             uint4* yp = reinterpret_cast<uint4*>(Y + static_cast<size_t>(row) * N + gcol);
 #pragma unroll
@@ -712,6 +738,9 @@ static cudaError_t launch_bn(const CUtensorMap& ta, const CUtensorMap& tb, const
     case kEpiResidualLongK:
       return launch_bn_epi<BN, kEpiResidualLongK, kPair>(ta, tb, ty, tr, y, ep, m_cap, m_dev, n,
                                                          k, status, stream);
+    case kEpiTokens:
+      return launch_bn_epi<BN, kEpiTokens, kPair>(ta, tb, ty, tr, y, ep, m_cap, m_dev, n, k,
+                                                  status, stream);
     case kEpiLn:
       return launch_bn_epi<BN, kEpiLn, kPair>(ta, tb, ty, tr, y, ep, m_cap, m_dev, n, k, status,
                                               stream);
@@ -744,8 +773,10 @@ cudaError_t launch_linear(const uint16_t* x, int32_t m_cap, const int32_t* m_dev
     return cudaErrorInvalidValue;
   // the residual [m_cap, n] in the output's 32 x 32 chunks (unused otherwise)
   tr = ty;
-  if (epilogue == DORA_EPI_BIAS_RESIDUAL &&
-      encode_tmap_2d_bf16(&tr, ep.residual, static_cast<uint64_t>(n), static_cast<uint64_t>(m_cap),
+  const bool tokens = epilogue == kEpiTokens;          // the position embeddings
+  if ((epilogue == DORA_EPI_BIAS_RESIDUAL || tokens) &&
+      encode_tmap_2d_bf16(&tr, tokens ? ep.pos : ep.residual, static_cast<uint64_t>(n),
+                          static_cast<uint64_t>(tokens ? ep.tokens : m_cap),
                           static_cast<uint64_t>(n) * 2, 32, 32, 64) != 0)
     return cudaErrorInvalidValue;
   if (bn == 256) {

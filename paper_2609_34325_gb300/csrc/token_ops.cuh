@@ -100,9 +100,12 @@ cudaError_t launch_gather_scores(const float* table, int32_t stride, const int32
 // the public DORA_EPI_* epilogues, two with a LayerNorm folded in:
 //   kEpiLn      y = rstd_r (x w'^T - mean_r colsum) + colbias
 //   kEpiLnGelu  the same, then GELU
-// with rstd_r = 1/sqrt(var_r + eps) from the row moments (stats_in).
+// with rstd_r = 1/sqrt(var_r + eps) from the row moments (stats_in);
+// and the patch embedding's, row r being token j = r mod tokens of its image:
+//   kEpiTokens  y = x w^T + bias + pos[j], for j = 0 (CLS) y = cls + pos[0]
 constexpr int kEpiLn = 3;
 constexpr int kEpiLnGelu = 4;
+constexpr int kEpiTokens = 6;
 struct LinearEpi {
   const uint16_t* bias = nullptr;       // bf16 [n], nullable (plain epilogues)
   const uint16_t* residual = nullptr;   // bf16 [m, n] (residual epilogue)
@@ -112,6 +115,9 @@ struct LinearEpi {
   float* stats_out = nullptr;           // slice moments of y, [n/64][m_cap], nullable
   float eps = 0.f;                      // LayerNorm epsilon (LN epilogues)
   int32_t slices = 0;                   // n / 64 (stats_out)
+  const uint16_t* cls = nullptr;        // bf16 [n] (kEpiTokens)
+  const uint16_t* pos = nullptr;        // bf16 [tokens, n] (kEpiTokens)
+  int32_t tokens = 0;                   // rows per image (kEpiTokens)
   int32_t m_reverse = 0;                // 1: walk the row blocks from the last one
 };
 // lda: row pitch of x in elements (0 = k; a multiple of 8).

@@ -1389,6 +1389,25 @@ def test_patch_embed_matches_oracle(b, c, h, w, patch, d):
     assert_close(f64(x0), ref, f"patch embed {b}x{c}x{h}x{w}/{patch} d={d}")
 
 
+@pytest.mark.parametrize("gw", [1, 15, 30, 31, 32, 63])
+def test_patch_embed_epilogue_where_a_chunk_spans_images(gw):
+    """The position embeddings come as 32-row boxes starting at a chunk's first
+    token: images of 2 to 64 tokens, so that a chunk ends with its image, runs
+    into the next one or spans many; no bias; the last rows past the last
+    whole chunk."""
+    b, patch, d = 9, 8, 64
+    rng = np.random.default_rng(gw)
+    im = S.f32_to_bf16_bits(rng.standard_normal((b, 1, patch, gw * patch)))
+    wpe = S.f32_to_bf16_bits(rng.standard_normal((d, patch * patch)) / patch)
+    cls, pos = (S.f32_to_bf16_bits(rng.standard_normal(n)) for n in (d, (gw + 1, d)))
+    x0 = torch.full((b * (gw + 1), d), 9.0, dtype=torch.bfloat16, device=dev())
+    P.dora_patch_embed(bf(im), bf(wpe), None, bf(cls), bf(pos), patch, x0)
+    torch.cuda.synchronize()
+    ref = O.patch_embed(im, O.bf16_to_f64(wpe), np.zeros(d), O.bf16_to_f64(cls),
+                        O.bf16_to_f64(pos), patch)
+    assert_close(f64(x0), ref, f"patch embed, {gw} patches")
+
+
 @pytest.mark.parametrize("name", ["cfg1", "cfg3"])
 def test_classifier_head_matches_oracle(name):
     cfg = S.get_config(name)
