@@ -12,10 +12,10 @@
 //             written W_1 Z_j + b_1 + (k / N_l) W_1 W_k: the first term is one
 //             tcgen05 GEMM over all tokens, W_1 W_k is made once per set of
 //             weights, and the rest runs per token.
-// The attention kernel works on heads of 64 lanes.  The encoder's heads of 32
-// are zero-padded to 64: the padded QKV rows and W_o columns are zero, so
-// every score, softmax weight and head output equals that of the 32-wide head
-// (the softmax scale stays 1/sqrt(32)).
+// The attention kernel has an instance for heads of 32 (softmax scale
+// 1/sqrt(32)).  On heads zero-padded to 64 the QKV linear wrote twice the bytes
+// and both MMAs did twice the work: 256 x 197 tokens, QKV 29.7 -> 16.5 us,
+// attention 33 -> 30.8, output projection 14.7 -> 14.0.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -31,7 +31,6 @@ namespace actor {
 constexpr int W = 128;          // encoder width
 constexpr int HEADS = 4;
 constexpr int HD = 32;          // encoder head width
-constexpr int HDP = 64;         // padded head width
 constexpr int FF = 256;         // feed-forward width
 constexpr int GH = 64;          // gate hidden units
 constexpr int GE = 16;          // gate block embedding
@@ -61,34 +60,6 @@ __device__ __forceinline__ float warp_sum(float v) {
 // ---------------------------------------------------------------------------
 // preparation (once per set of weights)
 // ---------------------------------------------------------------------------
-// Padded QKV [768, 128]: row part * 256 + head * 64 + j takes folded row
-// part * 128 + head * 32 + j for j < 32 and is zero otherwise (so are its c, d).
-__global__ void pad_qkv_kernel(const uint16_t* __restrict__ wf, const float* __restrict__ cf,
-                               const float* __restrict__ df, uint16_t* __restrict__ wp,
-                               float* __restrict__ cp, float* __restrict__ dp) {
-  const int p = blockIdx.x;
-  const int part = p / (HEADS * HDP), head = (p / HDP) % HEADS, j = p % HDP;
-  const bool live = j < HD;
-  const int src = part * W + head * HD + j;
-  for (int c = threadIdx.x; c < W; c += blockDim.x)
-    wp[static_cast<size_t>(p) * W + c] = live ? wf[static_cast<size_t>(src) * W + c] : 0;
-  if (threadIdx.x == 0) {
-    cp[p] = live ? cf[src] : 0.f;
-    dp[p] = live ? df[src] : 0.f;
-  }
-}
-
-// Padded W_o [128, 256]: column head * 64 + j takes column head * 32 + j for
-// j < 32 and is zero otherwise.
-__global__ void pad_wo_kernel(const uint16_t* __restrict__ wo, uint16_t* __restrict__ wp) {
-  const int r = blockIdx.x;
-  for (int c = threadIdx.x; c < HEADS * HDP; c += blockDim.x) {
-    const int head = c / HDP, j = c % HDP;
-    wp[static_cast<size_t>(r) * HEADS * HDP + c] =
-        j < HD ? wo[static_cast<size_t>(r) * W + head * HD + j] : 0;
-  }
-}
-
 // The selector's W_1 W_k (fp32 [64]).
 __global__ void sel_wk_kernel(const uint16_t* __restrict__ w1, const uint16_t* __restrict__ w_k,
                               float* __restrict__ out) {
@@ -162,6 +133,8 @@ __global__ void __launch_bounds__(256) gate_kernel(
   __shared__ float z[kMaxDim + GE + 3];
   __shared__ float part[4][GH];
   extern __shared__ __align__(16) uint4 wsm[];          // W_1^T when it fits (else empty)
+  pdl_trigger();
+  pdl_wait();
   const int i = blockIdx.x, t = threadIdx.x;
   const int lo = cu[i], hi = cu[i + 1];
   const int n = (lo < 0 || hi > t_cap) ? -1 : hi - lo - 1;   // visual tokens
@@ -229,6 +202,8 @@ __global__ void __launch_bounds__(128) budget_kernel(
     float* __restrict__ scores) {
   __shared__ float u[W], hb[W], logit[kMaxBudgets];
   extern __shared__ __align__(16) uint4 bsm[];          // W_1^T [128, 128], W_2^T [128, M]
+  pdl_trigger();
+  pdl_wait();
   const int i = blockIdx.x, t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int lo = cu[i], hi = cu[i + 1];
   const int n = (lo < 0 || hi > t_cap) ? -1 : hi - lo - 1;
@@ -268,14 +243,29 @@ __global__ void __launch_bounds__(128) budget_kernel(
   __syncthreads();
   for (int m = t; m < m_out; m += blockDim.x) logit[m] = dot_t(w2s, m_out, m, hb, 0, W) + ld(bb2, m);
   __syncthreads();
-  if (t == 0) {
-    int best = -1;
-    float bv = 0.f;
-    for (int m = 0; m < m_out; ++m)
-      if (2 * (m + 1) <= n - 4 && (best < 0 || logit[m] > bv)) {
+  if (warp == 0) {
+    // the first of the highest among the feasible (2 (m + 1) <= n - 4); a NaN
+    // counts only in the first place, where nothing is higher than it
+    const int feasible = min(n >= 6 ? (n - 4) / 2 : 0, m_out);
+    int best = feasible;
+    float bv = -INFINITY;
+    for (int m = lane; m < feasible; m += 32)
+      if (logit[m] > bv || (best == feasible && logit[m] == bv)) {
         best = m;
         bv = logit[m];
       }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+      const int om = __shfl_xor_sync(0xffffffffu, best, o);
+      if (ov > bv || (ov == bv && om < best)) {
+        best = om;
+        bv = ov;
+      }
+    }
+    if (feasible == 0) best = -1;
+    else if (best == feasible || logit[0] != logit[0]) best = 0;
+    if (lane != 0) return;
     const int bud = best < 0 ? 0 : 2 * (best + 1);
     const int g = (glogit[i] >= 0.f && bud > 0) ? 1 : 0;
     const int kk = g ? bud : 0;
@@ -300,6 +290,8 @@ __global__ void __launch_bounds__(256) selector_kernel(
     const uint16_t* __restrict__ sw2, const uint16_t* __restrict__ sb2,
     float* __restrict__ scores) {
   __shared__ float sck[SH], sw2s[SH];
+  pdl_trigger();
+  pdl_wait();
   const int i = blockIdx.x, t = threadIdx.x;
   const int lo = cu[i], hi = cu[i + 1];
   const int n = (lo < 0 || hi > t_cap) ? -1 : hi - lo - 1;
@@ -335,21 +327,16 @@ __global__ void __launch_bounds__(256) selector_kernel(
 size_t up256(size_t v) { return (v + 255) & ~static_cast<size_t>(255); }
 
 struct Prep {
-  size_t bias_in, wqkv_f, cqkv_f, dqkv_f, wqkv_p, cqkv_p, dqkv_p, wo_p, wfc1, cfc1, dfc1, sel_wk,
-      gate_w1t, bud_w1t, bud_w2t, total;
+  size_t bias_in, wqkv, cqkv, dqkv, wfc1, cfc1, dfc1, sel_wk, gate_w1t, bud_w1t, bud_w2t, total;
 };
 
 Prep prep_layout(const dora_actor_weights* w) {
   Prep P{};
   size_t off = 0;
   P.bias_in = off; off += up256(static_cast<size_t>(w->depth) * W * 2);
-  P.wqkv_f = off;  off += up256(3 * W * W * 2);
-  P.cqkv_f = off;  off += up256(3 * W * 4);
-  P.dqkv_f = off;  off += up256(3 * W * 4);
-  P.wqkv_p = off;  off += up256(3 * HEADS * HDP * W * 2);
-  P.cqkv_p = off;  off += up256(3 * HEADS * HDP * 4);
-  P.dqkv_p = off;  off += up256(3 * HEADS * HDP * 4);
-  P.wo_p = off;    off += up256(W * HEADS * HDP * 2);
+  P.wqkv = off;    off += up256(3 * W * W * 2);
+  P.cqkv = off;    off += up256(3 * W * 4);
+  P.dqkv = off;    off += up256(3 * W * 4);
   P.wfc1 = off;    off += up256(FF * W * 2);
   P.cfc1 = off;    off += up256(FF * 4);
   P.dfc1 = off;    off += up256(FF * 4);
@@ -372,8 +359,8 @@ Ws ws_layout(int32_t t_cap, int32_t batch, const dora_actor_weights* w) {
   L.status = off; off += 256;
   L.x = off;      off += up256(t * W * 2);
   L.mv = off;     off += up256(t * 8);
-  L.qkv = off;    off += up256(t * 3 * HEADS * HDP * 2);
-  L.o = off;      off += up256(t * HEADS * HDP * 2);
+  L.qkv = off;    off += up256(t * 3 * W * 2);
+  L.o = off;      off += up256(t * W * 2);
   L.z1 = off;     off += up256(t * W * 2);
   L.sm = off;     off += up256(t * 2 * 8);
   L.f = off;      off += up256(t * FF * 2);
@@ -405,16 +392,10 @@ bool weights_ok(const dora_actor_weights* w) {
 cudaError_t prepare(const dora_actor_weights* w, uint8_t* prep, cudaStream_t stream) {
   const Prep P = prep_layout(w);
   cudaError_t e = launch_fold_ln(w->enc_w_qkv, 3 * W, W, w->enc_ln1_w, w->enc_ln1_b,
-                                 w->enc_b_qkv, reinterpret_cast<uint16_t*>(prep + P.wqkv_f),
-                                 reinterpret_cast<float*>(prep + P.cqkv_f),
-                                 reinterpret_cast<float*>(prep + P.dqkv_f), stream);
+                                 w->enc_b_qkv, reinterpret_cast<uint16_t*>(prep + P.wqkv),
+                                 reinterpret_cast<float*>(prep + P.cqkv),
+                                 reinterpret_cast<float*>(prep + P.dqkv), stream);
   if (e != cudaSuccess) return e;
-  pad_qkv_kernel<<<3 * HEADS * HDP, 128, 0, stream>>>(
-      reinterpret_cast<const uint16_t*>(prep + P.wqkv_f),
-      reinterpret_cast<const float*>(prep + P.cqkv_f),
-      reinterpret_cast<const float*>(prep + P.dqkv_f), reinterpret_cast<uint16_t*>(prep + P.wqkv_p),
-      reinterpret_cast<float*>(prep + P.cqkv_p), reinterpret_cast<float*>(prep + P.dqkv_p));
-  pad_wo_kernel<<<W, 256, 0, stream>>>(w->enc_w_o, reinterpret_cast<uint16_t*>(prep + P.wo_p));
   bias_in_kernel<<<w->depth, W, 0, stream>>>(w->enc_b_in, w->enc_emb,
                                              reinterpret_cast<uint16_t*>(prep + P.bias_in));
   sel_wk_kernel<<<1, SH, 0, stream>>>(w->sel_w1, w->sel_w_k, reinterpret_cast<float*>(prep + P.sel_wk));
@@ -526,16 +507,16 @@ int dora_actor(const dora_bf16* qkv, const int32_t* cu, int32_t batch, int32_t m
       cudaFuncSetAttribute(budget_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            static_cast<int>(bud_smem)) != cudaSuccess)
     return DORA_ERR_CUDA;
-  gate_kernel<<<batch, 256, gate_smem, stream>>>(
-      qkv, d, cu, t_cap, block, w->depth, w->n0, rho, interventions,
-      reinterpret_cast<const uint16_t*>(prep + P.gate_w1t), w->gate_b1, w->gate_w2, w->gate_b2,
-      w->gate_emb, w->enc_w_h, x, glogit, p_gate);
-  if (cudaGetLastError() != cudaSuccess) return DORA_ERR_CUDA;
+  if (launch_pdl(gate_kernel, dim3(batch), dim3(256), gate_smem, stream, qkv, d, cu, t_cap, block,
+                 w->depth, w->n0, rho, interventions,
+                 reinterpret_cast<const uint16_t*>(prep + P.gate_w1t), w->gate_b1, w->gate_w2,
+                 w->gate_b2, w->gate_emb, w->enc_w_h, x, glogit, p_gate) != cudaSuccess)
+    return DORA_ERR_CUDA;
   // Z1 = X + W_o Attention(LayerNorm1(X)) + b_o
   LinearEpi e_q;
   e_q.stats_in = mv;
-  e_q.colsum = reinterpret_cast<const float*>(prep + P.cqkv_p);
-  e_q.colbias = reinterpret_cast<const float*>(prep + P.dqkv_p);
+  e_q.colsum = reinterpret_cast<const float*>(prep + P.cqkv);
+  e_q.colbias = reinterpret_cast<const float*>(prep + P.dqkv);
   e_q.eps = w->eps;
   LinearEpi e_o;
   e_o.bias = w->enc_b_o;
@@ -543,12 +524,12 @@ int dora_actor(const dora_bf16* qkv, const int32_t* cu, int32_t batch, int32_t m
   e_o.stats_out = sm;
   e_o.slices = W / kSliceCols;
   if (launch_row_stats(x, t_cap, rows, W, mv, stream) != cudaSuccess ||
-      launch_linear(x, t_cap, rows, W, reinterpret_cast<const uint16_t*>(prep + P.wqkv_p),
-                    3 * HEADS * HDP, kEpiLn, e_q, qkv_e, status, stream) != cudaSuccess ||
+      launch_linear(x, t_cap, rows, W, reinterpret_cast<const uint16_t*>(prep + P.wqkv),
+                    3 * W, kEpiLn, e_q, qkv_e, status, stream) != cudaSuccess ||
       launch_varlen_attn(qkv_e, cu, batch, max_seqlen, t_cap, HEADS, 0.17677669529663688f, o_e,
-                         status, stream) != cudaSuccess ||
-      launch_linear(o_e, t_cap, rows, HEADS * HDP, reinterpret_cast<const uint16_t*>(prep + P.wo_p),
-                    W, DORA_EPI_BIAS_RESIDUAL, e_o, z1, status, stream) != cudaSuccess ||
+                         status, stream, HD) != cudaSuccess ||
+      launch_linear(o_e, t_cap, rows, W, w->enc_w_o, W, DORA_EPI_BIAS_RESIDUAL, e_o, z1, status,
+                    stream) != cudaSuccess ||
       launch_merge_moments(sm, t_cap, rows, W / kSliceCols, mv, stream) != cudaSuccess)
     return DORA_ERR_CUDA;
   // Z = Z1 + W_2 GELU(W_1 LayerNorm2(Z1) + b_1) + b_2
@@ -572,16 +553,17 @@ int dora_actor(const dora_bf16* qkv, const int32_t* cu, int32_t batch, int32_t m
   if (launch_linear(z, t_cap, rows, W, w->sel_w1, SH, DORA_EPI_BIAS, e_s, s1, status, stream) !=
       cudaSuccess)
     return DORA_ERR_CUDA;
-  budget_kernel<<<batch, 128, bud_smem, stream>>>(
-      z, cu, t_cap, w->n0, w->eps, w->bud_ln_w, w->bud_ln_b,
-      reinterpret_cast<const uint16_t*>(prep + P.bud_w1t), w->bud_b1,
-      reinterpret_cast<const uint16_t*>(prep + P.bud_w2t), w->bud_b2, glogit, interventions, gate,
-      budget, k, keep_counts, rho_next,
-      interventions_next, scores);
-  selector_kernel<<<batch, 256, 0, stream>>>(s1, cu, t_cap, budget,
-                                             reinterpret_cast<const float*>(prep + P.sel_wk),
-                                             w->sel_w2, w->sel_b2, scores);
-  return cudaGetLastError() == cudaSuccess ? DORA_OK : DORA_ERR_CUDA;
+  if (launch_pdl(budget_kernel, dim3(batch), dim3(128), bud_smem, stream, z, cu, t_cap, w->n0,
+                 w->eps, w->bud_ln_w, w->bud_ln_b,
+                 reinterpret_cast<const uint16_t*>(prep + P.bud_w1t), w->bud_b1,
+                 reinterpret_cast<const uint16_t*>(prep + P.bud_w2t), w->bud_b2, glogit,
+                 interventions, gate, budget, k, keep_counts, rho_next, interventions_next,
+                 scores) != cudaSuccess ||
+      launch_pdl(selector_kernel, dim3(batch), dim3(256), 0, stream, s1, cu, t_cap, budget,
+                 reinterpret_cast<const float*>(prep + P.sel_wk), w->sel_w2, w->sel_b2,
+                 scores) != cudaSuccess)
+    return DORA_ERR_CUDA;
+  return DORA_OK;
 }
 
 }  // extern "C"

@@ -96,16 +96,17 @@ int encode_tmap_2d_bf16(void* map, const void* base, uint64_t inner, uint64_t ou
 }
 
 int encode_tmap_heads(void* map, const void* base, uint64_t rows, uint64_t heads,
-                      uint32_t box_rows) {
+                      uint32_t head_dim, uint32_t box_rows) {
   const auto encode = encode_fn();
   if (encode == nullptr) return -1;
-  cuuint64_t dims[3] = {64, rows, heads};
-  cuuint64_t strides[2] = {heads * 128, 128};
-  cuuint32_t box[3] = {64, box_rows, 2};
+  cuuint64_t dims[3] = {head_dim, rows, heads};
+  cuuint64_t strides[2] = {heads * head_dim * 2, head_dim * 2};
+  cuuint32_t box[3] = {head_dim, box_rows, 2};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = encode(reinterpret_cast<CUtensorMap*>(map), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
                       const_cast<void*>(base), dims, strides, box, estr,
-                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                      CU_TENSOR_MAP_INTERLEAVE_NONE,
+                      head_dim == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                       CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? 0 : static_cast<int>(r);
 }

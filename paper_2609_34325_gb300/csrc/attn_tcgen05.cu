@@ -59,8 +59,6 @@ namespace attn {
 
 constexpr int BQ = 128;         // query rows per unit
 constexpr int KC = 96;          // keys per step, at most
-constexpr int HD = 64;
-constexpr int kStages = 3;      // K/V chunk ring, two heads' chunks each
 constexpr int kDescRing = 8;    // step descriptors in flight
 constexpr int kUnitRing = 4;    // unit descriptors in flight
 constexpr int kThreads = 512;   // 16 warps, 128 registers a thread at launch
@@ -94,9 +92,12 @@ __device__ __forceinline__ int d_kc(uint32_t d) { return static_cast<int>((d >> 
 __device__ __forceinline__ int d_blocks(uint32_t d) { return (d_kc(d) + 31) >> 5; }
 __device__ __forceinline__ int d_rows(uint32_t d) { return static_cast<int>((d >> 16) & 0xFFu); }
 
+// HD: head width, 64 or 32 (rows of 128 or 64 bytes, swizzled as wide).
+template <int HD>
 struct Smem {
-  uint16_t q[2][2][BQ * HD];    // 16 KB each: by unit parity and group
-  uint16_t k[kStages][2][KC * HD];   // 12 KB each: by stage and group
+  static constexpr int kStages = HD == 64 ? 3 : 6;   // K/V chunk ring, two heads' chunks each
+  uint16_t q[2][2][BQ * HD];    // 16 KB each (HD 64): by unit parity and group
+  uint16_t k[kStages][2][KC * HD];   // 12 KB each (HD 64): by stage and group
   uint16_t v[kStages][2][KC * HD];
   float lsum[2][4][BQ];         // row sums, by group and unit mod 4
   uint64_t q_full[2];
@@ -122,7 +123,13 @@ struct Smem {
   int img_begin, unit_begin, img_end, unit_end;   // the CTA's units
   int q_issued, kv_issued;
 };
-static_assert(sizeof(Smem) <= 227 * 1024, "shared memory");
+static_assert(sizeof(Smem<64>) <= 227 * 1024 && sizeof(Smem<32>) <= 227 * 1024, "shared memory");
+
+// Descriptor of a tile of HD-wide rows as TMA wrote it, swizzled over 8 rows.
+template <int HD>
+__device__ __forceinline__ uint64_t tile_desc(uint32_t saddr, uint32_t lbo) {
+  return HD == 64 ? sdesc_sw128(saddr, lbo, 1024) : sdesc_sw64(saddr, lbo, 512);
+}
 
 // The map's box from row y of heads z and z + 1, one behind the other in dst.
 __device__ __forceinline__ void tma_load_heads(void* dst, const CUtensorMap* map, uint64_t* bar,
@@ -348,6 +355,7 @@ __device__ __forceinline__ void exp_pack(const uint32_t (&a)[N], uint32_t (&p)[N
   }
 }
 
+template <int HD>
 __global__ void __launch_bounds__(kThreads, 1)
     varlen_attn_kernel(const __grid_constant__ QkvMaps mp, const int32_t* __restrict__ cu,
                        int batch, int max_seqlen, int t_cap, int heads, float scale_log2,
@@ -359,7 +367,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (threadIdx.x == 0) record_status(status, DORA_ERR_UNSUPPORTED);
     return;
   }
-  Smem& s = *reinterpret_cast<Smem*>(smem_raw);
+  Smem<HD>& s = *reinterpret_cast<Smem<HD>*>(smem_raw);
+  constexpr int kStages = Smem<HD>::kStages;
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int dim = heads * HD;
@@ -519,13 +528,12 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int g = 0; g < 2; ++g) {
             if (j >= 2 && !(ok = wait_one(&s.p_free[g][b], ((j >> 1) - 1) & 1, abort))) break;
             tc_fence_after();
-            const uint64_t qd = sdesc_sw128(smem_u32(&s.q[qb][0][0] + g * q_step), 16, 1024);
-            const uint64_t kd = sdesc_sw128(smem_u32(&s.k[stg][0][0] + g * k_step), 16, 1024);
+            const uint64_t qd = tile_desc<HD>(smem_u32(&s.q[qb][0][0] + g * q_step), 16);
+            const uint64_t kd = tile_desc<HD>(smem_u32(&s.k[stg][0][0] + g * k_step), 16);
             const uint32_t dt = tmem + tmem_sp(g, b);
-            mma_bf16_ss(dt, qd, kd, id_s, 0u);
-            mma_bf16_ss(dt, qd + 2, kd + 2, id_s, 1u);
-            mma_bf16_ss(dt, qd + 4, kd + 4, id_s, 1u);
-            mma_bf16_ss(dt, qd + 6, kd + 6, id_s, 1u);
+#pragma unroll
+            for (int k = 0; k < HD / 16; ++k)
+              mma_bf16_ss(dt, qd + 2 * k, kd + 2 * k, id_s, k > 0 ? 1u : 0u);
             mma_commit(&s.s_full[g][b]);
           }
           if (d & kDLast) {
@@ -551,7 +559,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (d & kDEnd) break;
           const int nk = (d_kc(d) + 15) >> 4, stg = static_cast<int>(d & kDStage);
           const uint64_t vd =
-              sdesc_sw128(smem_u32(&s.v[stg][0][0] + g * 32 * d_blocks(d) * HD), 1024, 1024);
+              tile_desc<HD>(smem_u32(&s.v[stg][0][0] + g * 32 * d_blocks(d) * HD), 16 * HD);
           const uint32_t ot = tmem + tmem_o(g), at = tmem + tmem_sp(g, b);
           constexpr uint32_t id_o = idesc_bf16(BQ, HD, true);
           if ((d & kDFirst) && up > 0 && !wait_one(&s.o_free[g], (up - 1) & 1, abort)) break;
@@ -559,8 +567,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           tc_fence_after();
           mma_bf16_ts(ot, at, vd, id_o, (d & kDFirst) ? 0u : 1u);
 #pragma unroll
-          for (int kk = 1; kk < KC / 16; ++kk)   // 16 keys: 2048 bytes of V, 8 P columns
-            if (kk < nk) mma_bf16_ts(ot, at + 8u * kk, vd + 128u * kk, id_o, 1u);
+          for (int kk = 1; kk < KC / 16; ++kk)   // 16 keys: 2 HD 16-byte pieces of V, 8 P columns
+            if (kk < nk) mma_bf16_ts(ot, at + 8u * kk, vd + 2u * HD * kk, id_o, 1u);
           mma_commit(&s.p_free[g][b]);
           if (d & kDLast) {
             mma_commit(&s.o_done[g]);
@@ -590,11 +598,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc_fence_after();
       if (kc & 15) {
         // the last 16-key group reaches past the image: mask its S columns, and
-        // zero its V rows (S is done, so the chunk's load landed; whole 128-byte rows)
+        // zero its V rows (S is done, so the chunk's load landed; whole rows)
         const int past = 16 * groups - kc;
         if (live) mask_columns(tsp + static_cast<uint32_t>(kc), past);
-        if (r < past * 8)
-          reinterpret_cast<uint4*>(&s.v[d & kDStage][0][0] + g * 32 * d_blocks(d) * HD)[kc * 8 + r] = make_uint4(0u, 0u, 0u, 0u);
+        constexpr int kRow16 = HD / 8;                   // 16-byte pieces of a row
+        if (r < past * kRow16)
+          reinterpret_cast<uint4*>(&s.v[d & kDStage][0][0] +
+                                   g * 32 * d_blocks(d) * HD)[kc * kRow16 + r] =
+              make_uint4(0u, 0u, 0u, 0u);
         fence_proxy_async_smem();
       }
       if (live) {
@@ -652,7 +663,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           tc_fence_after();
           const uint32_t to = tmem + lane_sel + tmem_o(g);
 #pragma unroll 1
-          for (int h = 0; h < 4; ++h) {
+          for (int h = 0; h < HD / 16; ++h) {
             uint32_t o[16];
             tmem_ld16(to + 16u * h, o);
             tmem_ld_wait();
@@ -706,13 +717,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc_fence_after();
         uint16_t* const dst = out + static_cast<size_t>(row0 + r) * dim + (head + g) * HD;
 #pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < HD / 32; ++h) {
           uint32_t o[32], w[16];
           if (live) {
             tmem_ld32(tmem + lane_sel + tmem_o(g) + 32u * h, o);
             tmem_ld_wait();
           }
-          if (h == 1) warp_arrive(&s.o_free[g]);
+          if (h == HD / 32 - 1) warp_arrive(&s.o_free[g]);
           if (live && r < rows) {
 #pragma unroll
             for (int e = 0; e < 16; ++e)
@@ -757,27 +768,40 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 }  // namespace attn
 
-cudaError_t launch_varlen_attn(const uint16_t* qkv, const int32_t* cu, int32_t batch,
-                               int32_t max_seqlen, int32_t t_cap, int32_t heads, float scale,
-                               uint16_t* out, int32_t* status, cudaStream_t stream) {
-  if (batch == 0 || t_cap == 0 || max_seqlen == 0) return cudaSuccess;
-  attn::QkvMaps mp;
-  for (int i = 0; i < attn::BQ / 32; ++i)
+namespace attn {
+template <int HD>
+static cudaError_t launch(const uint16_t* qkv, const int32_t* cu, int32_t batch,
+                          int32_t max_seqlen, int32_t t_cap, int32_t heads, float scale,
+                          uint16_t* out, int32_t* status, cudaStream_t stream) {
+  QkvMaps mp;
+  for (int i = 0; i < BQ / 32; ++i)
     if (encode_tmap_heads(&mp.m[i], qkv, static_cast<uint64_t>(t_cap),
-                          static_cast<uint64_t>(3) * heads, 32u * (i + 1)) != 0)
+                          static_cast<uint64_t>(3) * heads, HD, 32u * (i + 1)) != 0)
       return cudaErrorInvalidValue;
-  const size_t smem = sizeof(attn::Smem);
+  const size_t smem = sizeof(Smem<HD>);
   const cudaError_t e =
-      cudaFuncSetAttribute(attn::varlen_attn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      cudaFuncSetAttribute(varlen_attn_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  const long long units = static_cast<long long>(batch) * ((heads + 1) / 2) *
-                          ((max_seqlen + attn::BQ - 1) / attn::BQ);
+  const long long units =
+      static_cast<long long>(batch) * ((heads + 1) / 2) * ((max_seqlen + BQ - 1) / BQ);
   if (units > 0x7fffffffLL) return cudaErrorInvalidValue;
   const long long cap = num_sms();
   const int grid = static_cast<int>(units < cap ? units : cap);
-  return launch_pdl(attn::varlen_attn_kernel, dim3(grid), dim3(attn::kThreads), smem, stream, mp,
-                    cu, batch, max_seqlen, t_cap, heads, scale * 1.4426950408889634f, out, status);
+  return launch_pdl(varlen_attn_kernel<HD>, dim3(grid), dim3(kThreads), smem, stream, mp, cu,
+                    batch, max_seqlen, t_cap, heads, scale * 1.4426950408889634f, out, status);
+}
+}  // namespace attn
+
+cudaError_t launch_varlen_attn(const uint16_t* qkv, const int32_t* cu, int32_t batch,
+                               int32_t max_seqlen, int32_t t_cap, int32_t heads, float scale,
+                               uint16_t* out, int32_t* status, cudaStream_t stream,
+                               int32_t head_dim) {
+  if (batch == 0 || t_cap == 0 || max_seqlen == 0) return cudaSuccess;
+  return head_dim == 32 ? attn::launch<32>(qkv, cu, batch, max_seqlen, t_cap, heads, scale, out,
+                                           status, stream)
+                        : attn::launch<64>(qkv, cu, batch, max_seqlen, t_cap, heads, scale, out,
+                                           status, stream);
 }
 
 }  // namespace dora

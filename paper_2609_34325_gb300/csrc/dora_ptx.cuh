@@ -365,6 +365,17 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr, uint32_t lbo, ui
   return d;
 }
 
+// The same with the 64-byte swizzle (rows of 64 bytes, swizzle mode 4).
+__device__ __forceinline__ uint64_t sdesc_sw64(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+  uint64_t d = 0;
+  d |= static_cast<uint64_t>((saddr >> 4) & 0x3FFFu);
+  d |= static_cast<uint64_t>((lbo >> 4) & 0x3FFFu) << 16;
+  d |= static_cast<uint64_t>((sbo >> 4) & 0x3FFFu) << 32;
+  d |= 1ull << 46;
+  d |= 4ull << 61;
+  return d;
+}
+
 // Instruction descriptor of kind::f16 with bf16 A/B, fp32 accumulator, A
 // K-major, B K-major (b_mn_major = false) or MN-major.
 __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n, bool b_mn_major) {

@@ -125,20 +125,22 @@ cudaError_t launch_linear(const uint16_t* x, int32_t m_cap, const int32_t* m_dev
                           const uint16_t* w, int32_t n, int32_t epilogue, const LinearEpi& ep,
                           uint16_t* y, int32_t* status, cudaStream_t stream, int32_t lda = 0);
 
-// tcgen05 varlen attention.
+// tcgen05 varlen attention; head_dim 64, or 32 (the actor's heads).
 cudaError_t launch_varlen_attn(const uint16_t* qkv, const int32_t* cu, int32_t batch,
                                int32_t max_seqlen, int32_t t_cap, int32_t heads, float scale,
-                               uint16_t* out, int32_t* status, cudaStream_t stream);
+                               uint16_t* out, int32_t* status, cudaStream_t stream,
+                               int32_t head_dim = 64);
 
 // Tensor-map encoding through the driver entry point (no libcuda link).
 // swizzle_bytes: 128 (default) or 64 (CU_TENSOR_MAP_SWIZZLE_128B / _64B).
 int encode_tmap_2d_bf16(void* map, const void* base, uint64_t inner, uint64_t outer,
                         uint64_t row_pitch_bytes, uint32_t box_inner, uint32_t box_outer,
                         int swizzle_bytes = 128);
-// Tensor map of a row-major bf16 [rows, heads * 64] matrix as [heads][rows][64],
-// with boxes of box_rows rows of two neighbouring heads (128-byte swizzle).
+// Tensor map of a row-major bf16 [rows, heads * head_dim] matrix (head_dim 64 or
+// 32) as [heads][rows][head_dim], with boxes of box_rows rows of two neighbouring
+// heads, swizzled as wide as a head's row.
 int encode_tmap_heads(void* map, const void* base, uint64_t rows, uint64_t heads,
-                      uint32_t box_rows);
+                      uint32_t head_dim, uint32_t box_rows);
 
 int num_sms();
 

@@ -1280,6 +1280,27 @@ def test_actor_matches_oracle(name, block, seed):
     _check_actor(cfg, cu, qkv, rho, e_prev, wa, got, block, images)
 
 
+@pytest.mark.parametrize("high", [[], [0], [1], [33, 70], [31, 32], [95], [40, 200]])
+def test_actor_budget_ties_over_the_lanes(high):
+    """The budget head's argmax over a warp's lanes: with a zero last layer the
+    logits are the biases, so the first of the highest feasible ones wins
+    whichever lane holds it, and images too short for a high one fall back."""
+    cfg = S.get_config("cfg1", batch=6)
+    lens = np.array([197, 197, 150, 80, 12, 5])
+    cu, qkv, rho, e_prev, wa, aw = _actor_case(cfg, 31, lens=lens)
+    m = O.budget_grid(cfg.n_vis0).size
+    bias = np.zeros(m)
+    bias[[h for h in high if h < m]] = 2.0
+    t = dict(aw.tensors)
+    t["bud_w2"] = torch.zeros_like(t["bud_w2"])
+    t["bud_b2"] = bf(S.f32_to_bf16_bits(bias))
+    aw = P.ActorWeights(t, aw.dim, aw.depth, aw.n0, aw.eps).prepare()
+    got = _run_actor(cfg, cu, qkv, rho, e_prev, aw, 0, cfg.n_tokens)
+    for i, n in enumerate(lens - 1):
+        feasible = bias[:max(0, (n - 4) // 2)]
+        assert got["budget"][i] == (2 * (int(np.argmax(feasible)) + 1) if feasible.size else 0)
+
+
 def test_actor_edges_short_images_and_gate_bias():
     """Images too short for any budget (N_l < 6) keep everything; an empty
     image is skipped; a strongly positive or negative gate bias opens or
