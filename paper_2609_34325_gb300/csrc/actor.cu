@@ -4,14 +4,16 @@
 //             SiLU MLP: one CTA per image;
 //   encoder   X = W_in K + b_in + e^C_l (+ W_h h_l on the CLS row), then one
 //             pre-LayerNorm Transformer block of width 128 (four heads of 32,
-//             GELU feed-forward 128 -> 256 -> 128), run on the library's
-//             tcgen05 GEMMs (LayerNorms folded in) and varlen attention;
+//             GELU feed-forward 128 -> 256 -> 128): input projection and QKV on
+//             the library's tcgen05 GEMM (LayerNorm folded in), the varlen
+//             attention, and all that follows it in one kernel
+//             (actor_tail.cu);
 //   budget    the highest logit of MLP_B(LayerNorm(Z_CLS)) among the budgets
 //             k <= N_l - 4 (ties to the smaller), and
 //   selector  s_j = MLP_S(Z_j + W_k k / N_l), a 128 -> 64 -> 1 SiLU MLP,
-//             written W_1 Z_j + b_1 + (k / N_l) W_1 W_k: the first term is one
-//             tcgen05 GEMM over all tokens, W_1 W_k is made once per set of
-//             weights, and the rest runs per token.
+//             written W_1 Z_j + b_1 + (k / N_l) W_1 W_k: the first term comes
+//             with Z, W_1 W_k is made once per set of weights, and the rest runs
+//             per token.
 // The attention kernel has an instance for heads of 32 (softmax scale
 // 1/sqrt(32)).  On heads zero-padded to 64 the QKV linear wrote twice the bytes
 // and both MMAs did twice the work: 256 x 197 tokens, QKV 29.7 -> 16.5 us,
@@ -349,7 +351,7 @@ Prep prep_layout(const dora_actor_weights* w) {
 }
 
 struct Ws {
-  size_t status, x, mv, qkv, o, z1, sm, f, z, s1, glogit, prep, total;
+  size_t status, x, mv, qkv, o, z, s1, glogit, prep, total;
 };
 
 Ws ws_layout(int32_t t_cap, int32_t batch, const dora_actor_weights* w) {
@@ -361,9 +363,6 @@ Ws ws_layout(int32_t t_cap, int32_t batch, const dora_actor_weights* w) {
   L.mv = off;     off += up256(t * 8);
   L.qkv = off;    off += up256(t * 3 * W * 2);
   L.o = off;      off += up256(t * W * 2);
-  L.z1 = off;     off += up256(t * W * 2);
-  L.sm = off;     off += up256(t * 2 * 8);
-  L.f = off;      off += up256(t * FF * 2);
   L.z = off;      off += up256(t * W * 2);
   L.s1 = off;     off += up256(t * SH * 2);
   L.glogit = off; off += up256(b * 4);
@@ -480,9 +479,6 @@ int dora_actor(const dora_bf16* qkv, const int32_t* cu, int32_t batch, int32_t m
   float* mv = reinterpret_cast<float*>(ws + L.mv);
   uint16_t* qkv_e = reinterpret_cast<uint16_t*>(ws + L.qkv);
   uint16_t* o_e = reinterpret_cast<uint16_t*>(ws + L.o);
-  uint16_t* z1 = reinterpret_cast<uint16_t*>(ws + L.z1);
-  float* sm = reinterpret_cast<float*>(ws + L.sm);
-  uint16_t* f = reinterpret_cast<uint16_t*>(ws + L.f);
   uint16_t* z = z_out != nullptr ? z_out : reinterpret_cast<uint16_t*>(ws + L.z);
   float* glogit = reinterpret_cast<float*>(ws + L.glogit);
   uint8_t* prep = ws + L.prep;
@@ -512,46 +508,33 @@ int dora_actor(const dora_bf16* qkv, const int32_t* cu, int32_t batch, int32_t m
                  reinterpret_cast<const uint16_t*>(prep + P.gate_w1t), w->gate_b1, w->gate_w2,
                  w->gate_b2, w->gate_emb, w->enc_w_h, x, glogit, p_gate) != cudaSuccess)
     return DORA_ERR_CUDA;
-  // Z1 = X + W_o Attention(LayerNorm1(X)) + b_o
+  // Attention(LayerNorm1(X))
   LinearEpi e_q;
   e_q.stats_in = mv;
   e_q.colsum = reinterpret_cast<const float*>(prep + P.cqkv);
   e_q.colbias = reinterpret_cast<const float*>(prep + P.dqkv);
   e_q.eps = w->eps;
-  LinearEpi e_o;
-  e_o.bias = w->enc_b_o;
-  e_o.residual = x;
-  e_o.stats_out = sm;
-  e_o.slices = W / kSliceCols;
   if (launch_row_stats(x, t_cap, rows, W, mv, stream) != cudaSuccess ||
       launch_linear(x, t_cap, rows, W, reinterpret_cast<const uint16_t*>(prep + P.wqkv),
                     3 * W, kEpiLn, e_q, qkv_e, status, stream) != cudaSuccess ||
       launch_varlen_attn(qkv_e, cu, batch, max_seqlen, t_cap, HEADS, 0.17677669529663688f, o_e,
-                         status, stream, HD) != cudaSuccess ||
-      launch_linear(o_e, t_cap, rows, W, w->enc_w_o, W, DORA_EPI_BIAS_RESIDUAL, e_o, z1, status,
-                    stream) != cudaSuccess ||
-      launch_merge_moments(sm, t_cap, rows, W / kSliceCols, mv, stream) != cudaSuccess)
+                         status, stream, HD) != cudaSuccess)
     return DORA_ERR_CUDA;
-  // Z = Z1 + W_2 GELU(W_1 LayerNorm2(Z1) + b_1) + b_2
-  LinearEpi e_f1;
-  e_f1.stats_in = mv;
-  e_f1.colsum = reinterpret_cast<const float*>(prep + P.cfc1);
-  e_f1.colbias = reinterpret_cast<const float*>(prep + P.dfc1);
-  e_f1.eps = w->eps;
-  LinearEpi e_f2;
-  e_f2.bias = w->enc_b_fc2;
-  e_f2.residual = z1;
-  if (launch_linear(z1, t_cap, rows, W, reinterpret_cast<const uint16_t*>(prep + P.wfc1), FF,
-                    kEpiLnGelu, e_f1, f, status, stream) != cudaSuccess ||
-      launch_linear(f, t_cap, rows, FF, w->enc_w_fc2, W, DORA_EPI_BIAS_RESIDUAL, e_f2, z, status,
-                    stream) != cudaSuccess)
-    return DORA_ERR_CUDA;
-  // selector's first layer on every token, then budget head and selector tail
+  // output projection, feed-forward and the selector's first layer on every
+  // token, then budget head and selector tail
   uint16_t* s1 = reinterpret_cast<uint16_t*>(ws + L.s1);
-  LinearEpi e_s;
-  e_s.bias = w->sel_b1;
-  if (launch_linear(z, t_cap, rows, W, w->sel_w1, SH, DORA_EPI_BIAS, e_s, s1, status, stream) !=
-      cudaSuccess)
+  TailArgs ta;
+  ta.x = x;
+  ta.bo = w->enc_b_o;
+  ta.c1 = reinterpret_cast<const float*>(prep + P.cfc1);
+  ta.d1 = reinterpret_cast<const float*>(prep + P.dfc1);
+  ta.eps = w->eps;
+  ta.b2 = w->enc_b_fc2;
+  ta.bs = w->sel_b1;
+  ta.z = z;
+  ta.s1 = s1;
+  if (launch_actor_tail(o_e, w->enc_w_o, reinterpret_cast<const uint16_t*>(prep + P.wfc1),
+                        w->enc_w_fc2, w->sel_w1, ta, t_cap, rows, status, stream) != cudaSuccess)
     return DORA_ERR_CUDA;
   if (launch_pdl(budget_kernel, dim3(batch), dim3(128), bud_smem, stream, z, cu, t_cap, w->n0,
                  w->eps, w->bud_ln_w, w->bud_ln_b,

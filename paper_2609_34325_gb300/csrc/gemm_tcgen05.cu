@@ -43,6 +43,7 @@
 #include <stdint.h>
 
 #include "dora_ptx.cuh"
+#include "epilogue_math.cuh"
 #include "token_ops.cuh"
 
 namespace dora {
@@ -121,52 +122,6 @@ struct Smem {
   int consumed;
 };
 
-__device__ __forceinline__ float rcp_approx(float x) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-// GELU(x) = x * Phi(x), Phi(x) = (1 + erf(x / sqrt 2)) / 2, with erf from
-// formula 7.1.26 of Abramowitz & Stegun, Handbook of Mathematical Functions
-// (|erf error| <= 1.5e-7): for z >= 0,
-//     erf(z) = 1 - t (a1 + t (a2 + t (a3 + t (a4 + t a5)))) exp(-z^2),
-//     t = 1 / (1 + p z).
-// With z = |x| / sqrt 2 and q = (1 - erf(z)) / 2, Phi = 1 - q for x >= 0 and
-// q for x < 0, so in both cases GELU(x) = max(x, 0) - |x| q: no select on
-// the sign.  The constants below fold in the 1/sqrt 2, the 1/2 and the sign
-// of q.  Evaluated on two values at once with the paired fp32 instructions
-// (fma/mul.rn.f32x2): the epilogue's ALU work is what limits this GEMM.
-__device__ __forceinline__ void gelu_erf2(float& x0, float& x1) {
-  const uint64_t P2 = f2_pack(0.3275911f * 0.70710678118654752f, 0.3275911f * 0.70710678118654752f);
-  const uint64_t ONE2 = f2_pack(1.0f, 1.0f);
-  const uint64_t A1 = f2_pack(-0.5f * 0.254829592f, -0.5f * 0.254829592f);
-  const uint64_t A2 = f2_pack(-0.5f * -0.284496736f, -0.5f * -0.284496736f);
-  const uint64_t A3 = f2_pack(-0.5f * 1.421413741f, -0.5f * 1.421413741f);
-  const uint64_t A4 = f2_pack(-0.5f * -1.453152027f, -0.5f * -1.453152027f);
-  const uint64_t A5 = f2_pack(-0.5f * 1.061405429f, -0.5f * 1.061405429f);
-  const uint64_t C2 = f2_pack(-0.72134752044448170f, -0.72134752044448170f);   // -log2(e) / 2
-  const uint64_t AX = f2_pack(fabsf(x0), fabsf(x1));
-  float d0, d1;
-  f2_unpack(f2_fma(P2, AX, ONE2), d0, d1);
-  const uint64_t T = f2_pack(rcp_approx(d0), rcp_approx(d1));
-  const uint64_t poly =
-      f2_mul(T, f2_fma(T, f2_fma(T, f2_fma(T, f2_fma(T, A5, A4), A3), A2), A1));
-  float e0, e1;
-  f2_unpack(f2_mul(f2_mul(AX, AX), C2), e0, e1);
-  const uint64_t neg_q = f2_mul(poly, f2_pack(ex2_approx(e0), ex2_approx(e1)));
-  f2_unpack(f2_fma(AX, neg_q, f2_pack(fmaxf(x0, 0.0f), fmaxf(x1, 0.0f))), x0, x1);
-}
-
-// Adds 8 bf16 values (one 16-byte piece) to v[0..7] in fp32 pairs.
-__device__ __forceinline__ void add_bf16x8(float* v, const uint4& piece) {
-  const uint32_t* w = reinterpret_cast<const uint32_t*>(&piece);
-#pragma unroll
-  for (int e = 0; e < 4; ++e)
-    f2_unpack(f2_add(f2_pack(v[2 * e], v[2 * e + 1]), f2_pack(bf16_lo(w[e]), bf16_hi(w[e]))),
-              v[2 * e], v[2 * e + 1]);
-}
-
 // Bias (or the folded LayerNorm) and GELU of one 32-column chunk of one row,
 // in fp32.
 // For the folded LayerNorm, c and d of the chunk's 32 columns come from
@@ -178,20 +133,7 @@ __device__ __forceinline__ void epilogue_math(const uint32_t (&r)[32], float (&v
 #pragma unroll
   for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(r[e]);
   if constexpr (EPI == kEpiLn || EPI == kEpiLnGelu) {
-    // v = rstd (acc - mean c) + d
-    const float4* cp = reinterpret_cast<const float4*>(cs);
-    const float4* dp = reinterpret_cast<const float4*>(cb);
-    const uint64_t NM = f2_pack(neg_mean, neg_mean), RS = f2_pack(rstd, rstd);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const float4 c = cp[q], d = dp[q];
-      f2_unpack(f2_fma(RS, f2_fma(NM, f2_pack(c.x, c.y), f2_pack(v[4 * q], v[4 * q + 1])),
-                       f2_pack(d.x, d.y)),
-                v[4 * q], v[4 * q + 1]);
-      f2_unpack(f2_fma(RS, f2_fma(NM, f2_pack(c.z, c.w), f2_pack(v[4 * q + 2], v[4 * q + 3])),
-                       f2_pack(d.z, d.w)),
-                v[4 * q + 2], v[4 * q + 3]);
-    }
+    fold_layernorm(v, neg_mean, rstd, cs, cb);
   } else if (EPI != kEpiTokens && ep.bias != nullptr) {
     const uint4* bp = reinterpret_cast<const uint4*>(ep.bias + gcol);
 #pragma unroll
@@ -201,32 +143,6 @@ __device__ __forceinline__ void epilogue_math(const uint32_t (&r)[32], float (&v
 #pragma unroll
     for (int e = 0; e < 32; e += 2) gelu_erf2(v[e], v[e + 1]);
   }
-}
-
-__device__ __forceinline__ void pack_row(const float (&v)[32], uint32_t (&o)[16]) {
-#pragma unroll
-  for (int e = 0; e < 16; ++e) o[e] = pack_bf16x2(v[2 * e], v[2 * e + 1]);
-}
-
-// Slice moments (mean, sum of squared deviations from it) of one 64-column
-// slice of a rounded output row, from its two packed 32-column chunks.
-__device__ __forceinline__ float2 slice_moments(const uint32_t (&lo)[16], const uint32_t (&hi)[16]) {
-  float s4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int e = 0; e < 16; ++e) {
-    s4[e & 1] += bf16_lo(lo[e]) + bf16_hi(lo[e]);
-    s4[2 + (e & 1)] += bf16_lo(hi[e]) + bf16_hi(hi[e]);
-  }
-  const float mean = ((s4[0] + s4[1]) + (s4[2] + s4[3])) * (1.0f / kSliceCols);
-  float q4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int e = 0; e < 16; ++e) {
-    const float a = bf16_lo(lo[e]) - mean, b = bf16_hi(lo[e]) - mean;
-    const float c = bf16_lo(hi[e]) - mean, d = bf16_hi(hi[e]) - mean;
-    q4[e & 1] += a * a + b * b;
-    q4[2 + (e & 1)] += c * c + d * d;
-  }
-  return make_float2(mean, (q4[0] + q4[1]) + (q4[2] + q4[3]));
 }
 
 template <int BN, int EPI, bool PAIR>

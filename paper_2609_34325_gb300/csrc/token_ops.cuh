@@ -125,6 +125,24 @@ cudaError_t launch_linear(const uint16_t* x, int32_t m_cap, const int32_t* m_dev
                           const uint16_t* w, int32_t n, int32_t epilogue, const LinearEpi& ep,
                           uint16_t* y, int32_t* status, cudaStream_t stream, int32_t lda = 0);
 
+// The actor's encoder after its attention, and the selector's first layer, in
+// one kernel: o [m, 128], W_o [128, 128], W_1' [256, 128] (LayerNorm folded in),
+// W_2 [128, 256], W_s [64, 128].
+struct TailArgs {
+  const uint16_t* x;        // bf16 [m, 128], the encoder's input
+  const uint16_t* bo;       // bf16 [128]
+  const float *c1, *d1;     // fp32 [256], of the folded W_1
+  float eps;
+  const uint16_t* b2;       // bf16 [128]
+  const uint16_t* bs;       // bf16 [64]
+  uint16_t* z;              // bf16 [m, 128]
+  uint16_t* s1;             // bf16 [m, 64]
+};
+cudaError_t launch_actor_tail(const uint16_t* o, const uint16_t* wo, const uint16_t* w1,
+                              const uint16_t* w2, const uint16_t* ws, const TailArgs& args,
+                              int32_t m_cap, const int32_t* m_dev, int32_t* status,
+                              cudaStream_t stream);
+
 // tcgen05 varlen attention; head_dim 64, or 32 (the actor's heads).
 cudaError_t launch_varlen_attn(const uint16_t* qkv, const int32_t* cu, int32_t batch,
                                int32_t max_seqlen, int32_t t_cap, int32_t heads, float scale,
