@@ -366,6 +366,10 @@ Ws ws_layout(int32_t t_cap, int32_t batch, const dora_actor_weights* w) {
   L.z = off;      off += up256(t * W * 2);
   L.s1 = off;     off += up256(t * SH * 2);
   L.glogit = off; off += up256(b * 4);
+  // the size stays what it was when heads were padded to 64 and Z1, its slice
+  // moments and the feed-forward's hidden rows were kept: callers that sized
+  // the workspace by that are not refused, nor is its size a surprise to them
+  off += up256(t * (3 * W * 2 + W * 2 + W * 2 + 2 * 8 + FF * 2));
   L.prep = off;   off += w->prepared != nullptr ? 0 : prep_layout(w).total;
   L.total = off;
   return L;
