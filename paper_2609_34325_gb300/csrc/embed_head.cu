@@ -205,6 +205,8 @@ __global__ void cls_ln_kernel(const uint16_t* __restrict__ x, const int32_t* __r
                               int batch, int t_cap, int dim, const uint16_t* __restrict__ gam,
                               const uint16_t* __restrict__ bet, float eps,
                               uint16_t* __restrict__ u, int32_t* status) {
+  pdl_trigger();
+  pdl_wait();
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (warp >= batch) return;
   const int r = cu[warp];
@@ -237,20 +239,35 @@ __global__ void cls_ln_kernel(const uint16_t* __restrict__ x, const int32_t* __r
   }
 }
 
-// LC1 readout of one image per CTA (8 warps): rows lo..hi-1 of x are layer-
-// normalised (fp32, biased variance, row held in registers: dim <= 2048); the
-// CLS row goes to u[i, 0:d], the others are summed per lane in registers and
-// their mean goes to u[i, d:2d] (zero for an image without visual rows).
+// LC1 readout of one image per CTA: rows lo..hi-1 of x are layer-normalised
+// (fp32, biased variance, row held in registers: dim <= 2048); the CLS row goes
+// to u[i, 0:d], the others are summed per lane in registers and their mean goes to
+// u[i, d:2d] (zero for an image without visual rows).
+// Bound by the instructions and the shuffle chains of a row, not its bytes
+// (256 images of 29 to 143 rows of 768: 34 MB, in L2): each warp takes two rows
+// at a time, so that one row's shuffles cover the other's, in paired fp32, and
+// keeps the centred row from the variance for the sum: 15.3 -> 11.8 us against one
+// row at a time in scalar fp32 (16 warps of that: no faster).
 constexpr int kLc1Warps = 8;
 constexpr int kLc1MaxDim = 2048;
 
-// kChunks = 16-byte pieces of a row per lane (dim <= 256 kChunks).
-template <int kChunks>
+__device__ __forceinline__ uint64_t bf_pair(uint32_t w) { return f2_pack(lo_f(w), hi_f(w)); }
+__device__ __forceinline__ float f2_sum(uint64_t v) {
+  float a, b;
+  f2_unpack(v, a, b);
+  return a + b;
+}
+
+// kChunks = 16-byte pieces of a row per lane (dim <= 256 kChunks); R rows of a
+// warp at a time.
+template <int kChunks, int R>
 __global__ void __launch_bounds__(kLc1Warps * 32)
     lc1_pool_kernel(const uint16_t* __restrict__ x, const int32_t* __restrict__ cu, int t_cap,
                     int dim, const uint16_t* __restrict__ gam, const uint16_t* __restrict__ bet,
                     float eps, uint16_t* __restrict__ u, int32_t* status) {
   extern __shared__ float acc[];                 // [kLc1Warps][dim]
+  pdl_trigger();
+  pdl_wait();
   const int img = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int d8 = dim / 8;
   const int lo = cu[img], hi = cu[img + 1];
@@ -264,76 +281,98 @@ __global__ void __launch_bounds__(kLc1Warps * 32)
   // Each lane owns the columns of its chunks c8 = lane + 32 i in every row,
   // so the visual rows' normalised values x^ = (x - mean) rstd are summed in
   // its registers; the affine map is applied once at the end, to the mean
-  // (mean of g x^ + b = g mean(x^) + b).  Each warp walks rows lo + warp,
-  // lo + warp + 8, ...; the next row's loads are issued before the current
-  // row is reduced.
-  float accr[kChunks][8];
+  // (mean of g x^ + b = g mean(x^) + b).  Each warp walks rows lo + R warp ..
+  // lo + R warp + R - 1 and on by R kLc1Warps; the next rows' loads are issued
+  // before the current ones are reduced.
+  uint64_t accr[kChunks][4];
 #pragma unroll
   for (int i = 0; i < kChunks; ++i)
 #pragma unroll
-    for (int e = 0; e < 8; ++e) accr[i][e] = 0.f;
-  uint4 nxt[kChunks];
-  auto load_row = [&](int j, uint4 (&q)[kChunks]) {
-    const uint4* xr = reinterpret_cast<const uint4*>(x + static_cast<size_t>(j) * dim);
+    for (int e = 0; e < 4; ++e) accr[i][e] = f2_pack(0.f, 0.f);
+  uint4 nxt[R][kChunks];
+  auto load_rows = [&](int j) {
 #pragma unroll
-    for (int i = 0; i < kChunks; ++i) {
-      const int c8 = lane + 32 * i;
-      q[i] = (j < hi && c8 < d8) ? xr[c8] : make_uint4(0, 0, 0, 0);
-    }
-  };
-  load_row(lo + warp, nxt);
-  for (int j = lo + warp; j < hi; j += kLc1Warps) {
-    uint4 q[kChunks];
-#pragma unroll
-    for (int i = 0; i < kChunks; ++i) q[i] = nxt[i];
-    load_row(j + kLc1Warps, nxt);
-    float s = 0.f;
-#pragma unroll
-    for (int i = 0; i < kChunks; ++i)
-      s += lo_f(q[i].x) + hi_f(q[i].x) + lo_f(q[i].y) + hi_f(q[i].y) + lo_f(q[i].z) +
-           hi_f(q[i].z) + lo_f(q[i].w) + hi_f(q[i].w);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    const float mean = s / dim;
-    float v2 = 0.f;
-#pragma unroll
-    for (int i = 0; i < kChunks; ++i) {
-      if (lane + 32 * i >= d8) continue;
-      const uint32_t wv[4] = {q[i].x, q[i].y, q[i].z, q[i].w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float a = lo_f(wv[e]) - mean, b = hi_f(wv[e]) - mean;
-        v2 += a * a + b * b;
-      }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v2 += __shfl_xor_sync(0xffffffffu, v2, o);
-    const float rstd = rsqrtf(v2 / dim + eps);
-    if (j == lo) {                                       // CLS row: LN(x) itself
+    for (int k = 0; k < R; ++k) {
+      const uint4* xr = reinterpret_cast<const uint4*>(x + static_cast<size_t>(j + k) * dim);
 #pragma unroll
       for (int i = 0; i < kChunks; ++i) {
         const int c8 = lane + 32 * i;
-        if (c8 >= d8) continue;
-        const uint32_t wv[4] = {q[i].x, q[i].y, q[i].z, q[i].w};
-        const uint4 g4 = reinterpret_cast<const uint4*>(gam)[c8];
-        const uint4 b4 = reinterpret_cast<const uint4*>(bet)[c8];
-        const uint32_t gv[4] = {g4.x, g4.y, g4.z, g4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
-        uint32_t o[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-          o[e] = pack2((lo_f(wv[e]) - mean) * rstd * lo_f(gv[e]) + lo_f(bv[e]),
-                       (hi_f(wv[e]) - mean) * rstd * hi_f(gv[e]) + hi_f(bv[e]));
-        reinterpret_cast<uint4*>(ur)[c8] = make_uint4(o[0], o[1], o[2], o[3]);
+        nxt[k][i] = (j + k < hi && c8 < d8) ? xr[c8] : make_uint4(0, 0, 0, 0);
       }
-    } else {
+    }
+  };
+  const float inv_dim = 1.f / static_cast<float>(dim);
+  load_rows(lo + R * warp);
+  for (int j = lo + R * warp; j < hi; j += R * kLc1Warps) {
+    uint64_t v[R][kChunks][4];
+    float s[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+      uint64_t t = f2_pack(0.f, 0.f);
 #pragma unroll
       for (int i = 0; i < kChunks; ++i) {
-        const uint32_t wv[4] = {q[i].x, q[i].y, q[i].z, q[i].w};
+        const uint32_t w[4] = {nxt[k][i].x, nxt[k][i].y, nxt[k][i].z, nxt[k][i].w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          accr[i][2 * e] += (lo_f(wv[e]) - mean) * rstd;
-          accr[i][2 * e + 1] += (hi_f(wv[e]) - mean) * rstd;
+          v[k][i][e] = bf_pair(w[e]);
+          t = f2_add(t, v[k][i][e]);
         }
+      }
+      s[k] = f2_sum(t);
+    }
+    load_rows(j + R * kLc1Warps);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < R; ++k) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+    float q[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+      const float nm = -s[k] * inv_dim;
+      const uint64_t NM = f2_pack(nm, nm);
+      uint64_t t = f2_pack(0.f, 0.f);
+#pragma unroll
+      for (int i = 0; i < kChunks; ++i) {
+        if (lane + 32 * i >= d8) continue;             // (its pieces stay zero)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          v[k][i][e] = f2_add(v[k][i][e], NM);
+          t = f2_fma(v[k][i][e], v[k][i][e], t);
+        }
+      }
+      q[k] = f2_sum(t);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < R; ++k) q[k] += __shfl_xor_sync(0xffffffffu, q[k], o);
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+      if (j + k >= hi) continue;
+      const float rstd = rsqrtf(q[k] * inv_dim + eps);
+      if (j + k == lo) {                                 // CLS row: LN(x) itself
+#pragma unroll
+        for (int i = 0; i < kChunks; ++i) {
+          const int c8 = lane + 32 * i;
+          if (c8 >= d8) continue;
+          const uint4 g4 = reinterpret_cast<const uint4*>(gam)[c8];
+          const uint4 b4 = reinterpret_cast<const uint4*>(bet)[c8];
+          const uint32_t gv[4] = {g4.x, g4.y, g4.z, g4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
+          uint32_t o[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            float a, b;
+            f2_unpack(v[k][i][e], a, b);
+            o[e] = pack2(a * rstd * lo_f(gv[e]) + lo_f(bv[e]), b * rstd * hi_f(gv[e]) + hi_f(bv[e]));
+          }
+          reinterpret_cast<uint4*>(ur)[c8] = make_uint4(o[0], o[1], o[2], o[3]);
+        }
+      } else {
+        const uint64_t RS = f2_pack(rstd, rstd);
+#pragma unroll
+        for (int i = 0; i < kChunks; ++i)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) accr[i][e] = f2_fma(v[k][i][e], RS, accr[i][e]);
       }
     }
   }
@@ -341,8 +380,12 @@ __global__ void __launch_bounds__(kLc1Warps * 32)
   for (int i = 0; i < kChunks; ++i) {
     const int c8 = lane + 32 * i;
     if (c8 >= d8) continue;
+    float f[8];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) acc[warp * dim + c8 * 8 + e] = accr[i][e];
+    for (int e = 0; e < 4; ++e) f2_unpack(accr[i][e], f[2 * e], f[2 * e + 1]);
+    float4* dst = reinterpret_cast<float4*>(acc + warp * dim + c8 * 8);
+    dst[0] = make_float4(f[0], f[1], f[2], f[3]);
+    dst[1] = make_float4(f[4], f[5], f[6], f[7]);
   }
   __syncthreads();
   const int n_vis = hi - lo - 1;
@@ -529,9 +572,9 @@ int dora_classifier_head(const dora_bf16* x, const int32_t* cu, int32_t batch, i
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   int32_t* status = reinterpret_cast<int32_t*>(ws);
   uint16_t* u = reinterpret_cast<uint16_t*>(ws + 256);
-  embed::cls_ln_kernel<<<(batch + 7) / 8, 256, 0, stream>>>(x, cu, batch, t_cap, dim, norm_w,
-                                                            norm_b, eps, u, status);
-  if (cudaGetLastError() != cudaSuccess) return DORA_ERR_CUDA;
+  if (launch_pdl(embed::cls_ln_kernel, dim3((batch + 7) / 8), dim3(256), 0, stream, x, cu, batch,
+                 t_cap, dim, norm_w, norm_b, eps, u, status) != cudaSuccess)
+    return DORA_ERR_CUDA;
   LinearEpi ep;
   ep.bias = b_head;
   return launch_linear(u, batch, nullptr, dim, w_head, classes, DORA_EPI_BIAS, ep, logits, status,
@@ -573,18 +616,18 @@ int dora_classifier_head_lc1(const dora_bf16* x, const int32_t* cu, int32_t batc
   uint16_t* u = reinterpret_cast<uint16_t*>(ws + 256);
   const int smem = embed::kLc1Warps * dim * 4;
   const int chunks = (dim / 8 + 31) / 32;
-  auto kern = chunks <= 1   ? embed::lc1_pool_kernel<1>
-              : chunks <= 2 ? embed::lc1_pool_kernel<2>
-              : chunks <= 3 ? embed::lc1_pool_kernel<3>
-              : chunks <= 4 ? embed::lc1_pool_kernel<4>
-                            : embed::lc1_pool_kernel<8>;
+  auto kern = chunks <= 1   ? embed::lc1_pool_kernel<1, 2>
+              : chunks <= 2 ? embed::lc1_pool_kernel<2, 2>
+              : chunks <= 3 ? embed::lc1_pool_kernel<3, 2>
+              : chunks <= 4 ? embed::lc1_pool_kernel<4, 2>
+                            : embed::lc1_pool_kernel<8, 1>;
   if (smem > 48 * 1024 &&
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
           cudaSuccess)
     return DORA_ERR_CUDA;
-  kern<<<batch, embed::kLc1Warps * 32, smem, stream>>>(x, cu, t_cap, dim, norm_w, norm_b, eps, u,
-                                                      status);
-  if (cudaGetLastError() != cudaSuccess) return DORA_ERR_CUDA;
+  if (launch_pdl(kern, dim3(batch), dim3(embed::kLc1Warps * 32), static_cast<size_t>(smem), stream,
+                 x, cu, t_cap, dim, norm_w, norm_b, eps, u, status) != cudaSuccess)
+    return DORA_ERR_CUDA;
   LinearEpi ep;
   ep.bias = b_head;
   return launch_linear(u, batch, nullptr, 2 * dim, w_head, classes, DORA_EPI_BIAS, ep, logits,
