@@ -35,6 +35,8 @@ STATUS_NAMES = {0: "DORA_OK", 1: "DORA_ERR_INVALID_ARG", 2: "DORA_ERR_UNSUPPORTE
                 6: "DORA_ERR_DEVICE_SEQLEN", 7: "DORA_ERR_SCRATCH_TOO_SMALL"}
 NOALLOC_SCRATCH_BYTES = 32 << 20
 
+_Tensor = torch.Tensor
+_BF16, _F32, _I32, _U8 = torch.bfloat16, torch.float32, torch.int32, torch.uint8
 _vp, _i32, _f32, _sz = ctypes.c_void_p, ctypes.c_int32, ctypes.c_float, ctypes.c_size_t
 _SIGS = {
     "dora_status_string": (ctypes.c_char_p, [ctypes.c_int]),
@@ -141,9 +143,18 @@ def _ptr(t):
     return t.data_ptr()
 
 
+# The current stream's handle as torch's own launchers read it: 0.3 us against
+# 3 us for a torch.cuda.Stream object, a tenth of a small call's host time.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None and _raw_device is not None and torch.cuda.is_initialized():
+        return _raw_stream(_raw_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _req(t, dtype, name, optional=False):
@@ -157,6 +168,17 @@ def _req(t, dtype, name, optional=False):
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise TypeError(f"{name} must be contiguous")
+
+
+def _arg(t, dtype, name):
+    """_req, and the tensor's device pointer: one look at a good tensor."""
+    if not (isinstance(t, _Tensor) and t.dtype is dtype and t.is_cuda and t.is_contiguous()):
+        _req(t, dtype, name)
+    return t.data_ptr()
+
+
+def _opt(t, dtype, name):
+    return None if t is None else _arg(t, dtype, name)
 
 
 def _check(code, name):
@@ -400,14 +422,12 @@ def dora_varlen_attn(qkv, cu_seqlens, max_seqlen, heads, out, head_dim=64, softm
 
 
 def dora_gather_scores(table, ids, cu, scores, status=None, stream=None):
-    _req(table, torch.float32, "table")
-    _req(scores, torch.float32, "scores")
-    _req(ids, torch.int32, "ids")
-    _req(cu, torch.int32, "cu")
-    _req(status, torch.int32, "status", optional=True)
-    _check(load_library().dora_gather_scores(_ptr(table), table.shape[-1], _ptr(ids), _ptr(cu),
-                                             cu.numel() - 1, _ptr(scores), _ptr(status),
-                                             _stream(stream)), "dora_gather_scores")
+    code = load_library().dora_gather_scores(
+        _arg(table, _F32, "table"), table.shape[-1], _arg(ids, _I32, "ids"), _arg(cu, _I32, "cu"),
+        cu.numel() - 1, _arg(scores, _F32, "scores"), _opt(status, _I32, "status"),
+        _stream(stream))
+    if code:
+        _check(code, "dora_gather_scores")
 
 
 class BlockWeights:
@@ -477,26 +497,21 @@ def dora_pruned_block(x_in, cu_in, weights: BlockWeights, max_seqlen, x_out, wor
     """One block of Eq. 1 (dora_pruned_block).  x_in_moments / x_out_moments
     (fp32 [t_cap, 2], optional) carry the row moments from block to block so
     that the next block skips its pass over x_in."""
-    _req(x_in, torch.bfloat16, "x_in")
-    _req(x_out, torch.bfloat16, "x_out")
-    _req(cu_in, torch.int32, "cu_in")
-    _req(workspace, torch.uint8, "workspace")
-    for n, t in (("ids_in", ids_in), ("keep_counts", keep_counts), ("cu_out", cu_out),
-                 ("ids_out", ids_out), ("kept_idx", kept_idx)):
-        _req(t, torch.int32, n, optional=True)
-    _req(scores, torch.float32, "scores", optional=True)
-    _req(x_in_moments, torch.float32, "x_in_moments", optional=True)
-    _req(x_out_moments, torch.float32, "x_out_moments", optional=True)
-    t_cap = x_in.shape[0]
+    x, cu, out = _arg(x_in, _BF16, "x_in"), _arg(cu_in, _I32, "cu_in"), _arg(x_out, _BF16, "x_out")
+    ws, t_cap = _arg(workspace, _U8, "workspace"), x_in.size(0)
+    mv_in = _opt(x_in_moments, _F32, "x_in_moments")
+    mv_out = _opt(x_out_moments, _F32, "x_out_moments")
     for t in (x_in_moments, x_out_moments):
         if t is not None and t.numel() < 2 * t_cap:
             raise ValueError("row moments must hold [t_cap, 2] floats")
-    _check(load_library().dora_pruned_block(
-        _ptr(x_in), _ptr(cu_in), _ptr(ids_in), cu_in.numel() - 1, int(max_seqlen), t_cap,
-        ctypes.byref(weights.c), _ptr(scores), _ptr(keep_counts), _ptr(x_out), _ptr(cu_out),
-        _ptr(ids_out), _ptr(kept_idx), _ptr(x_in_moments), _ptr(x_out_moments),
-        _ptr(workspace), workspace.numel(), _stream(stream)),
-        "dora_pruned_block")
+    code = load_library().dora_pruned_block(
+        x, cu, _opt(ids_in, _I32, "ids_in"), cu_in.numel() - 1, int(max_seqlen), t_cap,
+        ctypes.byref(weights.c), _opt(scores, _F32, "scores"),
+        _opt(keep_counts, _I32, "keep_counts"), out, _opt(cu_out, _I32, "cu_out"),
+        _opt(ids_out, _I32, "ids_out"), _opt(kept_idx, _I32, "kept_idx"), mv_in, mv_out, ws,
+        workspace.numel(), _stream(stream))
+    if code:
+        _check(code, "dora_pruned_block")
 
 
 def dora_pruned_block_noalloc(x_in, cu_in, weights: BlockWeights, max_seqlen, x_out,
@@ -600,30 +615,22 @@ def dora_actor(qkv, cu, weights: ActorWeights, block, max_seqlen, rho, intervent
                interventions_next=None, z_out=None, stream=None):
     """The deterministic actor at one block (dora_actor): gate, budget, k,
     keep counts and deletion scores for every image of the packed batch."""
-    _req(qkv, torch.bfloat16, "qkv")
-    _req(cu, torch.int32, "cu")
-    _req(workspace, torch.uint8, "workspace")
-    for n, t, dt, opt in (("rho", rho, torch.float32, False),
-                          ("interventions", interventions, torch.int32, False),
-                          ("gate", gate, torch.int32, False), ("budget", budget, torch.int32, False),
-                          ("k", k, torch.int32, False), ("keep_counts", keep_counts, torch.int32, False),
-                          ("scores", scores, torch.float32, False),
-                          ("p_gate", p_gate, torch.float32, True),
-                          ("rho_next", rho_next, torch.float32, True),
-                          ("interventions_next", interventions_next, torch.int32, True),
-                          ("z_out", z_out, torch.bfloat16, True)):
-        _req(t, dt, n, optional=opt)
-    t_cap = qkv.shape[0]
-    batch = cu.numel() - 1
-    if qkv.shape[1] != 3 * weights.dim or scores.numel() < t_cap:
+    q, c, ws = _arg(qkv, _BF16, "qkv"), _arg(cu, _I32, "cu"), _arg(workspace, _U8, "workspace")
+    sc, z = _arg(scores, _F32, "scores"), _opt(z_out, _BF16, "z_out")
+    t_cap = qkv.size(0)
+    if qkv.size(1) != 3 * weights.dim or scores.numel() < t_cap:
         raise ValueError("qkv must be [t_cap, 3 dim] and scores hold t_cap floats")
     if z_out is not None and tuple(z_out.shape) != (t_cap, 128):
         raise ValueError("z_out must be [t_cap, 128]")
-    _check(load_library().dora_actor(
-        _ptr(qkv), _ptr(cu), batch, int(max_seqlen), t_cap, int(block), ctypes.byref(weights.c),
-        _ptr(rho), _ptr(interventions), _ptr(p_gate), _ptr(gate), _ptr(budget), _ptr(k),
-        _ptr(keep_counts), _ptr(scores), _ptr(rho_next), _ptr(interventions_next), _ptr(z_out),
-        _ptr(workspace), workspace.numel(), _stream(stream)), "dora_actor")
+    code = load_library().dora_actor(
+        q, c, cu.numel() - 1, int(max_seqlen), t_cap, int(block), ctypes.byref(weights.c),
+        _arg(rho, _F32, "rho"), _arg(interventions, _I32, "interventions"),
+        _opt(p_gate, _F32, "p_gate"), _arg(gate, _I32, "gate"), _arg(budget, _I32, "budget"),
+        _arg(k, _I32, "k"), _arg(keep_counts, _I32, "keep_counts"), sc,
+        _opt(rho_next, _F32, "rho_next"), _opt(interventions_next, _I32, "interventions_next"), z,
+        ws, workspace.numel(), _stream(stream))
+    if code:
+        _check(code, "dora_actor")
 
 
 def dora_pruned_block_actor(x_in, cu_in, weights: BlockWeights, max_seqlen, x_out, workspace,
@@ -634,31 +641,22 @@ def dora_pruned_block_actor(x_in, cu_in, weights: BlockWeights, max_seqlen, x_ou
                             stream=None):
     """dora_pruned_block with the actor deciding the deletion at this block
     (its scores; its keep counts unless ``keep_counts`` is given)."""
-    _req(x_in, torch.bfloat16, "x_in")
-    _req(x_out, torch.bfloat16, "x_out")
-    for n, t in (("cu_in", cu_in), ("ids_in", ids_in), ("cu_out", cu_out), ("ids_out", ids_out),
-                 ("interventions", interventions), ("gate", gate), ("budget", budget), ("k", k),
-                 ("actor_keep", actor_keep)):
-        _req(t, torch.int32, n)
-    for n, t in (("keep_counts", keep_counts), ("kept_idx", kept_idx),
-                 ("interventions_next", interventions_next)):
-        _req(t, torch.int32, n, optional=True)
-    _req(rho, torch.float32, "rho")
-    _req(scores, torch.float32, "scores")
-    for n, t in (("rho_next", rho_next), ("x_in_moments", x_in_moments),
-                 ("x_out_moments", x_out_moments)):
-        _req(t, torch.float32, n, optional=True)
-    _req(workspace, torch.uint8, "workspace")
-    _req(actor_workspace, torch.uint8, "actor_workspace")
-    t_cap = x_in.shape[0]
-    _check(load_library().dora_pruned_block_actor(
-        _ptr(x_in), _ptr(cu_in), _ptr(ids_in), cu_in.numel() - 1, int(max_seqlen), t_cap,
-        ctypes.byref(weights.c), _ptr(x_out), _ptr(cu_out), _ptr(ids_out), _ptr(kept_idx),
-        _ptr(x_in_moments), _ptr(x_out_moments), _ptr(workspace), workspace.numel(),
-        ctypes.byref(actor.c), int(block), _ptr(rho), _ptr(interventions), _ptr(keep_counts),
-        _ptr(gate), _ptr(budget), _ptr(k), _ptr(actor_keep), _ptr(scores), _ptr(rho_next),
-        _ptr(interventions_next), _ptr(actor_workspace), actor_workspace.numel(),
-        _stream(stream)), "dora_pruned_block_actor")
+    ws = _arg(workspace, _U8, "workspace")
+    aws = _arg(actor_workspace, _U8, "actor_workspace")
+    code = load_library().dora_pruned_block_actor(
+        _arg(x_in, _BF16, "x_in"), _arg(cu_in, _I32, "cu_in"), _arg(ids_in, _I32, "ids_in"),
+        cu_in.numel() - 1, int(max_seqlen), x_in.size(0), ctypes.byref(weights.c),
+        _arg(x_out, _BF16, "x_out"), _arg(cu_out, _I32, "cu_out"), _arg(ids_out, _I32, "ids_out"),
+        _opt(kept_idx, _I32, "kept_idx"), _opt(x_in_moments, _F32, "x_in_moments"),
+        _opt(x_out_moments, _F32, "x_out_moments"), ws, workspace.numel(), ctypes.byref(actor.c),
+        int(block), _arg(rho, _F32, "rho"), _arg(interventions, _I32, "interventions"),
+        _opt(keep_counts, _I32, "keep_counts"), _arg(gate, _I32, "gate"),
+        _arg(budget, _I32, "budget"), _arg(k, _I32, "k"), _arg(actor_keep, _I32, "actor_keep"),
+        _arg(scores, _F32, "scores"), _opt(rho_next, _F32, "rho_next"),
+        _opt(interventions_next, _I32, "interventions_next"), aws, actor_workspace.numel(),
+        _stream(stream))
+    if code:
+        _check(code, "dora_pruned_block_actor")
 
 
 # ---------------------------------------------------------------------------
@@ -779,40 +777,32 @@ def dora_classifier_head(x, cu, norm_w, norm_b, eps, w_head, b_head, logits, wor
 def dora_pl_sample(scores, gumbel, cu, k, order, keys_out=None, status=None, stream=None):
     """Gumbel-top-k removal sequences: order int32 [B, k_cap] (-1 past k_i);
     keys_out (fp32, row-aligned) receives the perturbed keys s + g."""
-    _req(scores, torch.float32, "scores")
-    _req(gumbel, torch.float32, "gumbel")
-    _req(cu, torch.int32, "cu")
-    _req(k, torch.int32, "k")
-    _req(order, torch.int32, "order")
-    _req(keys_out, torch.float32, "keys_out", optional=True)
-    b = cu.numel() - 1
-    if order.dim() != 2 or order.shape[0] != b or k.numel() != b:
+    s, g, c = _arg(scores, _F32, "scores"), _arg(gumbel, _F32, "gumbel"), _arg(cu, _I32, "cu")
+    kp, o, b = _arg(k, _I32, "k"), _arg(order, _I32, "order"), cu.numel() - 1
+    keys = _opt(keys_out, _F32, "keys_out")
+    if order.dim() != 2 or order.size(0) != b or k.numel() != b:
         raise ValueError("order must be [B, k_cap] and k [B]")
-    _check(load_library().dora_pl_sample(_ptr(scores), _ptr(gumbel), _ptr(cu), b, scores.numel(),
-                                         _ptr(k), order.shape[1], _ptr(order), _ptr(keys_out),
-                                         _ptr(status), _stream(stream)), "dora_pl_sample")
+    code = load_library().dora_pl_sample(s, g, c, b, scores.numel(), kp, order.size(1), o, keys,
+                                         _ptr(status), _stream(stream))
+    if code:
+        _check(code, "dora_pl_sample")
     return order
 
 
 def dora_pl_logprob(scores, cu, k, order, logp, grad=None, dlogp=None, status=None, stream=None):
     """Plackett-Luce log-probabilities logp [B] and, optionally, their gradient
     with respect to the row-aligned scores (times dlogp)."""
-    _req(scores, torch.float32, "scores")
-    _req(cu, torch.int32, "cu")
-    _req(k, torch.int32, "k")
-    _req(order, torch.int32, "order")
-    _req(logp, torch.float32, "logp")
-    _req(grad, torch.float32, "grad", optional=True)
-    _req(dlogp, torch.float32, "dlogp", optional=True)
-    b = cu.numel() - 1
-    if order.dim() != 2 or order.shape[0] != b or logp.numel() != b:
+    s, c, kp = _arg(scores, _F32, "scores"), _arg(cu, _I32, "cu"), _arg(k, _I32, "k")
+    o, lp, b = _arg(order, _I32, "order"), _arg(logp, _F32, "logp"), cu.numel() - 1
+    gp, up = _opt(grad, _F32, "grad"), _opt(dlogp, _F32, "dlogp")
+    if order.dim() != 2 or order.size(0) != b or logp.numel() != b:
         raise ValueError("order must be [B, k_cap] and logp [B]")
     if grad is not None and grad.numel() != scores.numel():
         raise ValueError("grad must match scores")
-    _check(load_library().dora_pl_logprob(_ptr(scores), _ptr(cu), b, scores.numel(), _ptr(k),
-                                          _ptr(order), order.shape[1], _ptr(logp), _ptr(grad),
-                                          _ptr(dlogp), _ptr(status), _stream(stream)),
-           "dora_pl_logprob")
+    code = load_library().dora_pl_logprob(s, c, b, scores.numel(), kp, o, order.size(1), lp, gp,
+                                          up, _ptr(status), _stream(stream))
+    if code:
+        _check(code, "dora_pl_logprob")
     return logp
 
 
@@ -820,20 +810,17 @@ def dora_branch(x, cu, src, cu_out, ids=None, x_moments=None, len_out=None, stat
                 stream=None):
     """Append copies of sequences src (device int32) after row cu[-1] of x,
     in place; cu_out [B + 1 + len(src)]."""
-    _req(x, torch.bfloat16, "x")
-    _req(cu, torch.int32, "cu")
-    _req(src, torch.int32, "src")
-    _req(cu_out, torch.int32, "cu_out")
-    _req(ids, torch.int32, "ids", optional=True)
-    _req(x_moments, torch.float32, "x_moments", optional=True)
-    _req(len_out, torch.int32, "len_out", optional=True)
-    b, nb = cu.numel() - 1, src.numel()
+    xp, c, sp = _arg(x, _BF16, "x"), _arg(cu, _I32, "cu"), _arg(src, _I32, "src")
+    co, b, nb = _arg(cu_out, _I32, "cu_out"), cu.numel() - 1, src.numel()
     if cu_out.numel() < b + 1 + nb:
         raise ValueError("cu_out needs B + 1 + len(src) entries")
     t_cap, d = x.shape
-    _check(load_library().dora_branch(_ptr(x), _ptr(ids), _ptr(x_moments), _ptr(cu), b, t_cap, d,
-                                      _ptr(src), nb, _ptr(cu_out), _ptr(len_out), _ptr(status),
-                                      _stream(stream)), "dora_branch")
+    code = load_library().dora_branch(xp, _opt(ids, _I32, "ids"),
+                                      _opt(x_moments, _F32, "x_moments"), c, b, t_cap, d, sp, nb,
+                                      co, _opt(len_out, _I32, "len_out"), _ptr(status),
+                                      _stream(stream))
+    if code:
+        _check(code, "dora_branch")
     return cu_out
 
 
@@ -841,15 +828,14 @@ def dora_kd_cost(z_native, z, cost, classes, shadow_image=None, tau=3.0, status=
                  stream=None):
     """Fidelity costs [S]: tau^2 KL(softmax(z_native[img] / tau) || softmax(z[s] / tau))
     over the first `classes` logits of each row."""
-    _req(z_native, torch.bfloat16, "z_native")
-    _req(z, torch.bfloat16, "z")
-    _req(cost, torch.float32, "cost")
-    _req(shadow_image, torch.int32, "shadow_image", optional=True)
-    if z.shape[1] != z_native.shape[1] or cost.numel() != z.shape[0]:
+    zn, zp, c = _arg(z_native, _BF16, "z_native"), _arg(z, _BF16, "z"), _arg(cost, _F32, "cost")
+    si, n, ld = _opt(shadow_image, _I32, "shadow_image"), z.size(0), z.size(1)
+    if ld != z_native.size(1) or cost.numel() != n:
         raise ValueError("z and z_native need the same row pitch; cost one entry per row of z")
-    _check(load_library().dora_kd_cost(_ptr(z_native), _ptr(z), _ptr(shadow_image), z.shape[0],
-                                       z_native.shape[0], int(classes), z.shape[1], float(tau),
-                                       _ptr(cost), _ptr(status), _stream(stream)), "dora_kd_cost")
+    code = load_library().dora_kd_cost(zn, zp, si, n, z_native.size(0), int(classes), ld,
+                                       float(tau), c, _ptr(status), _stream(stream))
+    if code:
+        _check(code, "dora_kd_cost")
     return cost
 
 
@@ -857,16 +843,15 @@ def dora_step_rewards(cost, removals, blocks, depth, n0, a, reward, ret=None, st
     """Local rewards [P, B] (and episode sums [B]) from a batched shadow
     forward's fidelity costs (rollout, Native, shadows) and the removal
     counts [P, B] at the pruning blocks (device int32 [P])."""
-    _req(cost, torch.float32, "cost")
-    _req(removals, torch.int32, "removals")
-    _req(blocks, torch.int32, "blocks")
-    _req(reward, torch.float32, "reward")
-    _req(ret, torch.float32, "ret", optional=True)
+    c, rm = _arg(cost, _F32, "cost"), _arg(removals, _I32, "removals")
+    bl, rw = _arg(blocks, _I32, "blocks"), _arg(reward, _F32, "reward")
+    rt = _opt(ret, _F32, "ret")
     p, b = removals.shape
     if blocks.numel() != p or tuple(reward.shape) != (p, b) or cost.numel() < (p + 1) * b:
         raise ValueError("removals and reward must be [P, B], blocks [P], cost >= (P + 1) B")
-    _check(load_library().dora_step_rewards(_ptr(cost), _ptr(removals), _ptr(blocks), p, b,
-                                            int(depth), int(n0), float(a), _ptr(reward),
-                                            _ptr(ret), _stream(stream)), "dora_step_rewards")
+    code = load_library().dora_step_rewards(c, rm, bl, p, b, int(depth), int(n0), float(a), rw, rt,
+                                            _stream(stream))
+    if code:
+        _check(code, "dora_step_rewards")
     return reward
 
