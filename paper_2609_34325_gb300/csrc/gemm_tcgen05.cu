@@ -9,14 +9,18 @@
 // rows; the residual epilogue writes the 64-column slice moments they are
 // merged from.
 //
-// Design (one persistent CTA per SM, CTAs paired in clusters of two):
-//   The two CTAs of a cluster work on vertically adjacent output tiles
-//   (M-tiles 2p and 2p+1 of the same N-tile), so they need the same W tile.
+// Design (one persistent CTA per SM, CTAs working in pairs):
+//   The two CTAs of a pair work on vertically adjacent output tiles (M-tiles
+//   2p and 2p+1 of the same N-tile), so they need the same W tile.  With
+//   256-wide tiles a pair is a cluster; narrower tiles need nothing from the
+//   neighbour but its L2 reads, and launching them without clusters takes
+//   0.5-0.7 us off each (two cluster barriers and the cluster's scheduling):
+//   197 x 192 to 576 columns 4.5 -> 4.0 us, 768 to 192 6.2 -> 5.5.
 //   warp 0     TMA producer: the CTA's own 128x64 X tile and its part of the
 //              BNx64 W tile, per stage of a shared-memory ring (128-byte
 //              swizzle).  256-wide tiles run as a CTA pair (below), each CTA
 //              loading half of W; narrower tiles load the whole W tile in each
-//              CTA (both CTAs of a cluster read the same W tile, so the second
+//              CTA (both CTAs of a pair read the same W tile, so the second
 //              read is an L2 hit).
 //   warp 1     MMA issuer: one thread issues tcgen05.mma (M=128, N=BN, K=16,
 //              or M=256 across the pair) into one of two TMEM accumulators
@@ -172,10 +176,11 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
   const int lane = threadIdx.x & 31;
   // Work is a list of tile pairs: pair p covers M-tiles 2*(p / n_tiles) and
   // 2*(p / n_tiles) + 1 of N-tile p % n_tiles (row pairs counted from the
-  // last with ep.m_reverse); CTA `rank` of cluster c takes the M-tile
+  // last with ep.m_reverse); CTA `rank` of CTA pair c takes the M-tile
   // 2*(p / n_tiles) + rank of pairs c, c + clusters, ...
-  // Both CTAs of a cluster walk the same pairs in lockstep.
-  const int rank = static_cast<int>(cluster_ctarank());
+  // Both CTAs of a cluster (pair mode) walk the same pairs in lockstep.
+  const int rank =
+      kPair ? static_cast<int>(cluster_ctarank()) : static_cast<int>(blockIdx.x % kCluster);
   const int cid = blockIdx.x / kCluster;
   const int n_clusters = gridDim.x / kCluster;
   const int n_tiles = (N + BN - 1) / BN;
@@ -214,7 +219,9 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
     else tmem_alloc(&s.tmem_base, kTmemCols);
   }
   tc_fence_before();
-  cluster_sync();              // peers' barriers are initialised before any remote signal
+  // peers' barriers are initialised before any remote signal
+  if constexpr (kPair) cluster_sync();
+  else __syncthreads();
   tc_fence_after();
   // the set-up above overlaps the previous kernel; global memory waits for it
   pdl_wait();
@@ -594,7 +601,8 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
     if constexpr (kPair) tmem_dealloc_pair(tmem, kTmemCols);
     else tmem_dealloc(tmem, kTmemCols);
   }
-  cluster_sync();              // no CTA leaves while its peer may still signal it
+  // no CTA leaves while its peer may still signal it
+  if constexpr (kPair) cluster_sync();
 }
 
 template <int BN, int EPI, bool PAIR>
@@ -610,17 +618,17 @@ static cudaError_t launch_bn_epi(const CUtensorMap& ta, const CUtensorMap& tb,
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = kCluster;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = kCluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.blockDim = dim3(Cfg<BN, EPI, PAIR>::kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.attrs = attr + 1;
+  cfg.numAttrs = PAIR ? 1 : 0;
   // as many co-resident clusters as fit, capped by the tile pairs of m_cap
   static int max_clusters[64] = {0};   // per instantiation and device
   int dev = 0;
@@ -628,16 +636,21 @@ static cudaError_t launch_bn_epi(const CUtensorMap& ta, const CUtensorMap& tb,
   if (dev < 0 || dev >= 64) dev = 0;
   if (max_clusters[dev] == 0) {
     cfg.gridDim = dim3(kCluster * (num_sms() / kCluster));
-    int c = 0;
-    e = cudaOccupancyMaxActiveClusters(&c, kern, &cfg);
-    if (e != cudaSuccess) return e;
+    int c = num_sms() / kCluster;
+    if (PAIR) {
+      e = cudaOccupancyMaxActiveClusters(&c, kern, &cfg);
+      if (e != cudaSuccess) return e;
+    }
     max_clusters[dev] = c > 0 ? c : 1;
   }
   const long pairs =
       static_cast<long>((m_cap + 2 * BM - 1) / (2 * BM)) * ((n + BN - 1) / BN);
   const long clusters = pairs < max_clusters[dev] ? pairs : max_clusters[dev];
   cfg.gridDim = dim3(static_cast<unsigned>(kCluster * clusters));
-  cfg.numAttrs = pdl_enabled() ? 2 : 1;          // dependent launch (the kernel waits)
+  if (pdl_enabled()) {                           // dependent launch (the kernel waits)
+    cfg.attrs = attr;
+    ++cfg.numAttrs;
+  }
   return cudaLaunchKernelEx(&cfg, kern, ta, tb, ty, tr, y, ep, m_cap, m_dev, n, k, status);
 }
 
