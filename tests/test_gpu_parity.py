@@ -834,6 +834,15 @@ def test_attention_chunk_edges_with_odd_and_even_head_counts(heads):
     assert torch.all(buf[:off] == 9.0) and torch.all(buf[off + t * heads * 64:] == 9.0)
 
 
+@pytest.mark.parametrize("extra", [-1, 0, 1])
+def test_attention_where_every_unit_has_its_own_cta(extra):
+    """Batches on both sides of one possible unit per SM, images shorter than
+    max_seqlen (whose later tiles do not exist) and empty ones among them."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    lens = np.resize(np.array([197, 128, 0, 129, 1]), sms // 2 + extra)
+    _check_attn(lens, 2, 28)
+
+
 def test_attention_first_chunk_of_minus_infinities():
     """Logits of -inf (an infinite key component) in the whole first key
     chunk weigh nothing; the later chunk's keys get the weight."""
