@@ -79,6 +79,14 @@ template <int BN, int EPI, bool PAIR>
 struct Cfg {
   static constexpr bool kPair = PAIR;
   static constexpr int kBRows = kPair ? BN / 2 : BN;   // W rows held per CTA
+  // The tiles of a last wave that would leave half of the clusters idle are cut
+  // into two column halves, one a cluster (same bits).  us at 129 x 3 tile pairs on
+  // 76 clusters (5.09 waves): fc2 106 -> 100, QKV (15.3) 75.8 -> 73.8, fc1 (20.4)
+  // 116 -> 115; ViT-L's fc2 at 59 x 4 (3.1) 91 -> 84; no change where the last
+  // wave is fuller.  Quarters gave no more, and cost fc2 1.3 % everywhere.
+  // Not in the short-K residual epilogue, which fills its main loop: the
+  // run-time column count costs it more (47.4 -> 48.6 us) than the halves give.
+  static constexpr bool kSplit = PAIR && EPI != DORA_EPI_BIAS_RESIDUAL;
   static constexpr bool kLn = EPI == kEpiLn || EPI == kEpiLnGelu;
   static constexpr bool kResTma =
       EPI == DORA_EPI_BIAS_RESIDUAL || EPI == kEpiResidualLongK || EPI == kEpiTokens;
@@ -91,8 +99,10 @@ struct Cfg {
   static constexpr int kColGroups = kEpiWarps / 4;
   static constexpr int kCols = BN / kColGroups;         // columns per epilogue warp
   static constexpr int kChunks = kCols / 32;
-  // chunks per TMEM load: two (64 registers) unless 16 warps cap registers at 96
-  static constexpr int kBatch = kEpiWarps == 16 ? 1 : (kChunks < 2 ? kChunks : 2);
+  // chunks per TMEM load: two (64 registers) unless 16 warps cap registers at
+  // 96, or a long K hides the loads anyway (two would spill)
+  static constexpr int kBatch =
+      (kEpiWarps == 16 || EPI == kEpiResidualLongK) ? 1 : (kChunks < 2 ? kChunks : 2);
   // staging buffers per epilogue warp: one per chunk for the residual (its
   // TMA load lands there; two for a long K), one with 16 warps or the folded
   // LayerNorm, else two
@@ -156,6 +166,7 @@ __device__ __forceinline__ void epilogue_math(const uint32_t (&r)[32], float (&v
 template <int BN, int EPI, bool PAIR>
 __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
     gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                const __grid_constant__ CUtensorMap tmBt,
                 const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUtensorMap tmR,
                 uint16_t* __restrict__ Y, const LinearEpi ep, int m_cap,
                 const int32_t* __restrict__ m_dev, int N, int K, int32_t* status) {
@@ -232,6 +243,21 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
   }
   const int m_pairs = (M + 2 * BM - 1) / (2 * BM);
   const int num_pairs = m_pairs * n_tiles;
+  // Work items: the tile pairs, those of a sparse last wave as column halves.
+  int full = num_pairs;                         // tile pairs left whole
+  if constexpr (C::kSplit) {
+    const int rest = num_pairs % n_clusters;
+    if (2 * rest <= n_clusters) full -= rest;
+  }
+  const int items = full + 2 * (num_pairs - full);
+  struct Item {
+    int pair, n0, cols;                         // tile pair, first output column, columns
+  };
+  auto item = [&](int w) -> Item {
+    if (!C::kSplit || w < full) return {w, (w % n_tiles) * BN, BN};
+    const int p = full + ((w - full) >> 1);
+    return {p, (p % n_tiles) * BN + ((w - full) & 1) * (BN / 2), BN / 2};
+  };
   const uint32_t tmem = s.tmem_base;
   volatile int* abort = &s.abort_flag;
   // row pair of work item p; m_reverse walks them from the last, so that a
@@ -246,9 +272,9 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
     if (elect_one()) {
       int it = 0;
       bool ok = true;
-      for (int pr = cid; ok && pr < num_pairs; pr += n_clusters) {
-        const int mt = 2 * mpair(pr) + rank;
-        const int nt = pr % n_tiles;
+      for (int w = cid; ok && w < items; w += n_clusters) {
+        const Item t = item(w);
+        const int mt = 2 * mpair(t.pair) + rank;
         for (int kb = 0; kb < kb_count; ++kb) {
           const int st = it % kStages;
           const uint32_t ph = (it / kStages) & 1;
@@ -259,15 +285,20 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
           if constexpr (kPair) {
             // this CTA's X rows and half of the W tile; the bytes of both CTAs
             // are counted on the first CTA's barrier, which its MMA waits on
-            if (rank == 0) mbar_arrive_expect_tx(&s.full[st], 2 * C::kStageBytes);
+            // (half a tile loads boxes half as high)
+            const bool whole = !C::kSplit || t.cols == BN;
+            if (rank == 0)
+              mbar_arrive_expect_tx(&s.full[st],
+                                    2 * (BM + (whole ? kHalfB : kHalfB / 2)) * BK * 2);
             tma_load_2d_pair(s.a[st], &tmA, &s.full[st], 0, kb * BK, mt * BM);
-            tma_load_2d_pair(s.b[st], &tmB, &s.full[st], 0, kb * BK, nt * BN + rank * kHalfB);
+            tma_load_2d_pair(s.b[st], whole ? &tmB : &tmBt, &s.full[st], 0, kb * BK,
+                             t.n0 + rank * (t.cols >> 1));
           } else {
             // the X tile and both halves of the W tile (the map's box is BN/2 rows)
             mbar_arrive_expect_tx(&s.full[st], (BM + BN) * BK * 2);
             tma_load_2d(s.a[st], &tmA, &s.full[st], kb * BK, mt * BM);
-            tma_load_2d(s.b[st], &tmB, &s.full[st], kb * BK, nt * BN);
-            tma_load_2d(s.b[st] + kHalfB * BK, &tmB, &s.full[st], kb * BK, nt * BN + kHalfB);
+            tma_load_2d(s.b[st], &tmB, &s.full[st], kb * BK, t.n0);
+            tma_load_2d(s.b[st] + kHalfB * BK, &tmB, &s.full[st], kb * BK, t.n0 + kHalfB);
           }
           ++it;
         }
@@ -278,10 +309,10 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
     const bool issuer = elect_one();
     if (issuer && kPair && rank == 0) {
       // pair MMA issuer: M = 256 over both CTAs, D in both CTAs' TMEM
-      constexpr uint32_t idesc = idesc_bf16(2 * BM, BN, false);
       int it = 0, ti = 0;
       bool ok = true;
-      for (int pr = cid; ok && pr < num_pairs; pr += n_clusters, ++ti) {
+      for (int w = cid; ok && w < items; w += n_clusters, ++ti) {
+        const uint32_t idesc = idesc_bf16(2 * BM, C::kSplit && w >= full ? BN / 2 : BN, false);
         const int acc = ti & 1;
         const uint32_t aph = (ti >> 1) & 1;
         if (!mbar_wait(&s.acc_empty[acc], aph ^ 1, abort)) break;
@@ -313,7 +344,7 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
       constexpr uint32_t idesc = idesc_bf16(BM, BN, false);
       int it = 0, ti = 0;
       bool ok = true;
-      for (int pr = cid; ok && pr < num_pairs; pr += n_clusters, ++ti) {
+      for (int w = cid; ok && w < items; w += n_clusters, ++ti) {
         const int acc = ti & 1;
         const uint32_t aph = (ti >> 1) & 1;
         if (!mbar_wait(&s.acc_empty[acc], aph ^ 1, abort)) break;
@@ -343,12 +374,14 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
      }
     }
   } else {
-    constexpr int kCols = C::kCols;                // columns per epilogue warp
-    constexpr int kChunks = C::kChunks;
     constexpr int kBatch = C::kBatch;              // chunks per TMEM load
     const int ew = warp - 2;                      // epilogue warp index
     const int q = warp & 3;                       // TMEM lanes this warp may read
     const int slot = ew >> 2;                     // which column slice
+    // chunks of 32 columns of each warp in an item
+    auto warp_chunks = [&](const Item& t) {
+      return !C::kSplit || t.cols == BN ? C::kChunks : C::kChunks / 2;
+    };
     const uint32_t lane_sel = static_cast<uint32_t>(q * 32) << 16;
     int buf = 0;                                  // staging buffer to write next
     uint32_t res_pend = 0;                        // staging buffers with a residual load in flight
@@ -374,15 +407,17 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
     };
     // Residual of the warp's whole 32-row chunks of tile pair `p` (the first
     // kBufs chunks), once the stores of the previous tile have read the buffers.
-    auto prefetch_residual = [&](int p) {
-      const int row0 = (2 * mpair(p) + rank) * BM + q * 32;
+    auto prefetch_residual = [&](int w) {
+      const Item t = item(w);
+      const int row0 = (2 * mpair(t.pair) + rank) * BM + q * 32;
       if (row0 + 32 > M) return;
-      const int col0 = (p % n_tiles) * BN + slot * kCols;
+      const int chunks = warp_chunks(t);
+      const int col0 = t.n0 + slot * 32 * chunks;
       if (lane == 0) bulk_wait_group_read0();
       __syncwarp();
 #pragma unroll
       for (int c = 0; c < kBufs; ++c) {
-        if (col0 + c * 32 >= N) break;
+        if (c >= chunks || col0 + c * 32 >= N) break;
         load_residual(c, row0, col0);
       }
     };
@@ -403,9 +438,11 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
     // previous tile's values.
     bool cd_pend = false;
     uint32_t cd_par = 0;
-    auto prefetch_cd = [&](int p) {
-      const int col0 = (p % n_tiles) * BN + slot * kCols;
-      const int cols = N - col0 < kCols ? N - col0 : kCols;
+    auto prefetch_cd = [&](int w) {
+      const Item t = item(w);
+      const int mine = 32 * warp_chunks(t);
+      const int col0 = t.n0 + slot * mine;
+      const int cols = N - col0 < mine ? N - col0 : mine;
       if (cols <= 0) return;
       __syncwarp();                               // every lane's reads of the buffer are done
       if (lane == 0) {
@@ -419,24 +456,26 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
     // Folded LayerNorm: (mean, var) of this lane's row, loaded a tile ahead
     // (a warp's 32 rows are one 256-byte load).
     float2 mv = make_float2(0.f, 0.f);
-    auto load_mv = [&](int p) {
-      const int row_p = (2 * mpair(p) + rank) * BM + q * 32 + lane;
+    auto load_mv = [&](int w) {
+      const int row_p = (2 * mpair(item(w).pair) + rank) * BM + q * 32 + lane;
       if (row_p < M) mv = __ldg(reinterpret_cast<const float2*>(ep.stats_in) + row_p);
     };
     if constexpr (C::kLn)
-      if (cid < num_pairs) {
+      if (cid < items) {
         prefetch_cd(cid);
         load_mv(cid);
       }
     if constexpr (C::kResTma)
-      if (cid < num_pairs) prefetch_residual(cid);
+      if (cid < items) prefetch_residual(cid);
     int ti = 0;
     bool ok = true;
-    for (int pr = cid; ok && pr < num_pairs; pr += n_clusters, ++ti) {
+    for (int w = cid; ok && w < items; w += n_clusters, ++ti) {
       const int acc = ti & 1;
       const uint32_t aph = (ti >> 1) & 1;
-      const int mt = 2 * mpair(pr) + rank;
-      const int nt = pr % n_tiles;
+      const Item t = item(w);
+      const int mt = 2 * mpair(t.pair) + rank;
+      const int chunks = warp_chunks(t);
+      const int wcol0 = slot * 32 * chunks;       // this warp's first column of the tile
       const int row0 = mt * BM + q * 32;          // first row of this warp
       const int row = row0 + lane;
       const bool whole = row0 + 32 <= M;          // all 32 rows live: TMA store
@@ -445,7 +484,7 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
       if constexpr (C::kLn) {
         neg_mean = -mv.x;
         rstd = rsqrtf(mv.y + ep.eps);
-        if (pr + n_clusters < num_pairs) load_mv(pr + n_clusters);
+        if (w + n_clusters < items) load_mv(w + n_clusters);
       }
       if (!mbar_wait_warp(&s.acc_full[acc], aph, abort)) break;
       tc_fence_after();
@@ -457,15 +496,15 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
         }
       }
 #pragma unroll 1
-      for (int cb = 0; cb < kChunks; cb += kBatch) {
+      for (int cb = 0; cb < chunks; cb += kBatch) {
         uint32_t r[kBatch][32];
 #pragma unroll
         for (int c = 0; c < kBatch; ++c)
           tmem_ld32(tmem + lane_sel +
-                        static_cast<uint32_t>(acc * BN + slot * kCols + (cb + c) * 32),
+                        static_cast<uint32_t>(acc * BN + wcol0 + (cb + c) * 32),
                     r[c]);
         tmem_ld_wait();
-        if (cb + kBatch == kChunks) {
+        if (cb + kBatch == chunks) {
           // the accumulator is in registers: hand it back to the MMA warp
           tc_fence_before();
           __syncwarp();
@@ -476,7 +515,7 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
         }
 #pragma unroll
         for (int c = 0; c < kBatch; ++c) {
-          const int gcol = nt * BN + slot * kCols + (cb + c) * 32;
+          const int gcol = t.n0 + wcol0 + (cb + c) * 32;
           if (gcol >= N || row0 >= M) continue;    // warp-uniform
           float v[32];
           uint32_t o[16];
@@ -540,11 +579,11 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
               tma_store_2d(&tmY, stage, gcol, row0);
               bulk_commit_group();
             }
-            if constexpr (C::kResTma && kBufs < kChunks) {
+            if constexpr (C::kResTma && kBufs < C::kChunks) {
               // the chunk kBufs on goes into this buffer once the store has read it
               const int nc = cb + c + kBufs;
-              const int col0 = nt * BN + slot * kCols;
-              if (nc < kChunks && col0 + nc * 32 < N) {
+              const int col0 = t.n0 + wcol0;
+              if (nc < chunks && col0 + nc * 32 < N) {
                 if (lane == 0) bulk_wait_group_read0();
                 __syncwarp();
                 load_residual(nc, row0, col0);
@@ -568,9 +607,9 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
         if (!ok) break;
       }
       if constexpr (C::kResTma)
-        if (ok && pr + n_clusters < num_pairs) prefetch_residual(pr + n_clusters);
+        if (ok && w + n_clusters < items) prefetch_residual(w + n_clusters);
       if constexpr (C::kLn)
-        if (ok && pr + n_clusters < num_pairs) prefetch_cd(pr + n_clusters);
+        if (ok && w + n_clusters < items) prefetch_cd(w + n_clusters);
     }
     if (lane == 0) {
       bulk_wait_group0();                         // stores done before the CTA exits
@@ -607,9 +646,10 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
 
 template <int BN, int EPI, bool PAIR>
 static cudaError_t launch_bn_epi(const CUtensorMap& ta, const CUtensorMap& tb,
-                                 const CUtensorMap& ty, const CUtensorMap& tr, uint16_t* y,
-                                 const LinearEpi& ep, int m_cap, const int32_t* m_dev, int n,
-                                 int k, int32_t* status, cudaStream_t stream) {
+                                 const CUtensorMap& tbt, const CUtensorMap& ty,
+                                 const CUtensorMap& tr, uint16_t* y, const LinearEpi& ep,
+                                 int m_cap, const int32_t* m_dev, int n, int k, int32_t* status,
+                                 cudaStream_t stream) {
   static_assert(sizeof(Smem<BN, EPI, PAIR>) <= kSmemLimit, "shared memory");
   const size_t smem = sizeof(Smem<BN, EPI, PAIR>);
   auto kern = gemm_kernel<BN, EPI, PAIR>;
@@ -651,38 +691,35 @@ static cudaError_t launch_bn_epi(const CUtensorMap& ta, const CUtensorMap& tb,
     cfg.attrs = attr;
     ++cfg.numAttrs;
   }
-  return cudaLaunchKernelEx(&cfg, kern, ta, tb, ty, tr, y, ep, m_cap, m_dev, n, k, status);
+  return cudaLaunchKernelEx(&cfg, kern, ta, tb, tbt, ty, tr, y, ep, m_cap, m_dev, n, k, status);
 }
 
 // BN = 256 tiles run in pair mode.
 template <int BN>
-static cudaError_t launch_bn(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& ty,
-                             const CUtensorMap& tr, uint16_t* y, const LinearEpi& ep, int epi,
-                             int m_cap, const int32_t* m_dev, int n, int k, int32_t* status,
+static cudaError_t launch_bn(const CUtensorMap& ta, const CUtensorMap& tb,
+                             const CUtensorMap& tbt, const CUtensorMap& ty, const CUtensorMap& tr,
+                             uint16_t* y, const LinearEpi& ep, int epi, int m_cap,
+                             const int32_t* m_dev, int n, int k, int32_t* status,
                              cudaStream_t stream) {
   constexpr bool kPair = BN == 256;
+  const auto launch = [&](auto kernel) {
+    return kernel(ta, tb, tbt, ty, tr, y, ep, m_cap, m_dev, n, k, status, stream);
+  };
   switch (epi) {
     case DORA_EPI_BIAS_GELU:
-      return launch_bn_epi<BN, DORA_EPI_BIAS_GELU, kPair>(ta, tb, ty, tr, y, ep, m_cap, m_dev, n, k,
-                                                          status, stream);
+      return launch(launch_bn_epi<BN, DORA_EPI_BIAS_GELU, kPair>);
     case DORA_EPI_BIAS_RESIDUAL:
-      return launch_bn_epi<BN, DORA_EPI_BIAS_RESIDUAL, kPair>(ta, tb, ty, tr, y, ep, m_cap, m_dev,
-                                                              n, k, status, stream);
+      return launch(launch_bn_epi<BN, DORA_EPI_BIAS_RESIDUAL, kPair>);
     case kEpiResidualLongK:
-      return launch_bn_epi<BN, kEpiResidualLongK, kPair>(ta, tb, ty, tr, y, ep, m_cap, m_dev, n,
-                                                         k, status, stream);
+      return launch(launch_bn_epi<BN, kEpiResidualLongK, kPair>);
     case kEpiTokens:
-      return launch_bn_epi<BN, kEpiTokens, kPair>(ta, tb, ty, tr, y, ep, m_cap, m_dev, n, k,
-                                                  status, stream);
+      return launch(launch_bn_epi<BN, kEpiTokens, kPair>);
     case kEpiLn:
-      return launch_bn_epi<BN, kEpiLn, kPair>(ta, tb, ty, tr, y, ep, m_cap, m_dev, n, k, status,
-                                              stream);
+      return launch(launch_bn_epi<BN, kEpiLn, kPair>);
     case kEpiLnGelu:
-      return launch_bn_epi<BN, kEpiLnGelu, kPair>(ta, tb, ty, tr, y, ep, m_cap, m_dev, n, k, status,
-                                                  stream);
+      return launch(launch_bn_epi<BN, kEpiLnGelu, kPair>);
     default:
-      return launch_bn_epi<BN, DORA_EPI_BIAS, kPair>(ta, tb, ty, tr, y, ep, m_cap, m_dev, n, k,
-                                                     status, stream);
+      return launch(launch_bn_epi<BN, DORA_EPI_BIAS, kPair>);
   }
 }
 
@@ -703,13 +740,19 @@ cudaError_t launch_linear(const uint16_t* x, int32_t m_cap, const int32_t* m_dev
   int bn = (n % 256 == 0) ? 256 : 128;
   if (row_pairs * ((n + 63) / 64) <= wave) bn = 64;
   else if (bn == 256 && row_pairs * ((n + 127) / 128) <= wave) bn = 128;
-  CUtensorMap ta, tb, ty, tr;
+  CUtensorMap ta, tb, tbt, ty, tr;
   if (lda != 0 && (lda < k || lda % 8 != 0)) return cudaErrorInvalidValue;
   if (encode_tmap_2d_bf16(&ta, x, static_cast<uint64_t>(k), static_cast<uint64_t>(m_cap),
                           static_cast<uint64_t>(lda != 0 ? lda : k) * 2, gemm::BK, gemm::BM) != 0)
     return cudaErrorInvalidValue;
   if (encode_tmap_2d_bf16(&tb, w, static_cast<uint64_t>(k), static_cast<uint64_t>(n),
                           static_cast<uint64_t>(k) * 2, gemm::BK, static_cast<uint32_t>(bn / 2)) != 0)
+    return cudaErrorInvalidValue;
+  // the same with boxes half as high, for column halves of a tile (unused otherwise)
+  tbt = tb;
+  if (bn == 256 &&
+      encode_tmap_2d_bf16(&tbt, w, static_cast<uint64_t>(k), static_cast<uint64_t>(n),
+                          static_cast<uint64_t>(k) * 2, gemm::BK, 64) != 0)
     return cudaErrorInvalidValue;
   if (encode_tmap_2d_bf16(&ty, y, static_cast<uint64_t>(n), static_cast<uint64_t>(m_cap),
                           static_cast<uint64_t>(n) * 2, 32, 32, 64) != 0)
@@ -726,11 +769,14 @@ cudaError_t launch_linear(const uint16_t* x, int32_t m_cap, const int32_t* m_dev
     const int epi = (epilogue == DORA_EPI_BIAS_RESIDUAL && k >= gemm::kLongK)
                         ? gemm::kEpiResidualLongK
                         : epilogue;
-    return gemm::launch_bn<256>(ta, tb, ty, tr, y, ep, epi, m_cap, m_dev, n, k, status, stream);
+    return gemm::launch_bn<256>(ta, tb, tbt, ty, tr, y, ep, epi, m_cap, m_dev, n, k, status,
+                                stream);
   }
   if (bn == 64)
-    return gemm::launch_bn<64>(ta, tb, ty, tr, y, ep, epilogue, m_cap, m_dev, n, k, status, stream);
-  return gemm::launch_bn<128>(ta, tb, ty, tr, y, ep, epilogue, m_cap, m_dev, n, k, status, stream);
+    return gemm::launch_bn<64>(ta, tb, tbt, ty, tr, y, ep, epilogue, m_cap, m_dev, n, k, status,
+                               stream);
+  return gemm::launch_bn<128>(ta, tb, tbt, ty, tr, y, ep, epilogue, m_cap, m_dev, n, k, status,
+                              stream);
 }
 
 }  // namespace dora

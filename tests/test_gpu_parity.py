@@ -708,6 +708,69 @@ def test_linear_residual_long_k_many_tiles(m_cap, m_live):
     assert np.all(np.abs(got[:, :, 0] - s_mean) <= 4e-6 * s_scale + 1e-30)
 
 
+# With 152 SMs (76 CTA pairs): the last row count of one wave of 64- and of
+# 128-wide tiles and the one past it, 256-wide tiles whose last wave is cut into
+# halves (78 = 76 + 2 tile pairs; 36 of them live) and one that is not (39).
+TILE_WIDTH_CASES = [
+    # m_cap, m_live, k, n
+    (6400, 6400, 64, 192), (6401, 6401, 64, 192),
+    (2304, 2303, 128, 512), (2305, 2305, 128, 512),
+    (4864, 4864, 128, 512), (4865, 4865, 128, 512),
+    (6556, 6556, 2048, 768), (6556, 3001, 2048, 768), (3201, 3201, 2048, 768),
+]
+
+
+@pytest.mark.parametrize("m_cap,m_live,k,n", TILE_WIDTH_CASES)
+def test_linears_where_the_tile_width_changes(m_cap, m_live, k, n):
+    """Every linear at the edges of the rules that choose the tile width and
+    cut a sparse last wave's tiles in halves: sampled rows against the fp64
+    oracle, all rows bit for bit against launches of 256 rows (one wave of the
+    narrowest tiles; the order of the sums does not depend on the width), and
+    nothing written past the live rows."""
+    rng = np.random.default_rng(m_cap + n)
+    xb = S.f32_to_bf16_bits(rng.standard_normal((m_cap, k)))
+    wb = S.f32_to_bf16_bits(0.05 * rng.standard_normal((n, k)))
+    bb = S.f32_to_bf16_bits(0.1 * rng.standard_normal(n))
+    rb = S.f32_to_bf16_bits(rng.standard_normal((m_cap, n)))
+    x, w, b, r = bf(xb), bf(wb), bf(bb), bf(rb)
+    mv = torch.zeros(m_cap, 2, dtype=torch.float32, device=dev())
+    P.dora_row_stats(x, mv)
+    cs = w.float().sum(1)
+    cb = b.float()
+    st = _status()
+
+    def run(kind, rows, m_dev=None):
+        xr = x[rows]
+        m = xr.shape[0]
+        y = torch.full((m, n), 7.0, dtype=torch.bfloat16, device=dev())
+        sm = torch.full((n // 64, m, 2), -3.0, dtype=torch.float32, device=dev())
+        if kind == "bias":
+            P.dora_linear(xr, w, y, bias=b, m_dev=m_dev, status=st)
+        elif kind == "gelu":
+            P.dora_linear(xr, w, y, bias=b, epilogue=P.EPI_BIAS_GELU, m_dev=m_dev, status=st)
+        elif kind == "residual":
+            P.dora_linear_residual_stats(xr, w, r[rows], y, sm, bias=b, m_dev=m_dev, status=st)
+        else:
+            P.dora_linear_ln(xr, mv[rows].contiguous(), 1e-6, w, cs, cb, y, gelu=kind == "ln_gelu",
+                             m_dev=m_dev, status=st)
+        return y, sm
+
+    at = np.unique(np.concatenate([np.arange(0, m_live, 127), [m_live - 1]]))
+    lin = O.linear(O.bf16_to_f64(xb[at]), O.bf16_to_f64(wb), O.bf16_to_f64(bb))
+    for kind in ("bias", "gelu", "residual", "ln", "ln_gelu"):
+        y, sm = run(kind, slice(0, m_cap), i32([m_live]))
+        if kind == "bias":
+            assert_close(f64(y)[at], lin, f"bias {m_cap}x{n}")
+        elif kind == "residual":
+            assert_close(f64(y)[at], lin + O.bf16_to_f64(rb[at]), f"residual {m_cap}x{n}")
+        assert torch.all(y[m_live:] == 7.0) and torch.all(sm[:, m_live:] == -3.0), kind
+        for i in range(0, m_live, 256):
+            rows = slice(i, min(i + 256, m_live))
+            y1, sm1 = run(kind, rows)
+            assert torch.equal(y[rows], y1) and torch.equal(sm[:, rows], sm1), (kind, i)
+    assert int(st.item()) == 0
+
+
 # ---------------------------------------------------------------------------
 # varlen attention (tcgen05)
 # ---------------------------------------------------------------------------
