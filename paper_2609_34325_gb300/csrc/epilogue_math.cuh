@@ -98,6 +98,46 @@ __device__ __forceinline__ float2 slice_moments(const uint32_t (&lo)[16], const 
   return make_float2(mean, (q4[0] + q4[1]) + (q4[2] + q4[3]));
 }
 
+// Row moments (mean, var) of one row from its S slice moments (mean_s, M2_s)
+// over 64 columns each, stored slice-major with `stride` rows between slices:
+// mean = (1/S) sum mean_s, M2 = sum (M2_s + 64 (mean_s - mean)^2) (the
+// pairwise update of Chan, Golub & LeVeque with equal counts), var = M2 / (64 S).
+// Every rounding is explicit, so each caller gets the same bits.
+__device__ __forceinline__ float2 merge_slice_moments(const float2* __restrict__ p, size_t stride,
+                                                      int slices) {
+  constexpr int kHeld = 16;     // slice means held in registers (dim <= 1024)
+  const float inv_s = __frcp_rn(static_cast<float>(slices));
+  float mean, m2 = 0.f;
+  if (slices <= kHeld) {
+    float mu[kHeld];
+#pragma unroll
+    for (int j = 0; j < kHeld; ++j)
+      if (j < slices) mu[j] = __ldg(&p[j * stride].x);
+    float sum = 0.f;
+#pragma unroll
+    for (int j = 0; j < kHeld; ++j)
+      if (j < slices) sum = __fadd_rn(sum, mu[j]);
+    mean = __fmul_rn(sum, inv_s);
+#pragma unroll
+    for (int j = 0; j < kHeld; ++j)
+      if (j < slices) {             // the M2 halves are read again (L1)
+        const float d = __fsub_rn(mu[j], mean);
+        m2 = __fadd_rn(m2, __fmaf_rn(__fmul_rn(static_cast<float>(kSliceCols), d), d,
+                                     __ldg(&p[j * stride].y)));
+      }
+  } else {
+    float sum = 0.f;
+    for (int j = 0; j < slices; ++j) sum = __fadd_rn(sum, __ldg(&p[j * stride].x));
+    mean = __fmul_rn(sum, inv_s);
+    for (int j = 0; j < slices; ++j) {
+      const float2 t = __ldg(p + j * stride);
+      const float d = __fsub_rn(t.x, mean);
+      m2 = __fadd_rn(m2, __fmaf_rn(__fmul_rn(static_cast<float>(kSliceCols), d), d, t.y));
+    }
+  }
+  return make_float2(mean, __fmul_rn(__fmul_rn(m2, inv_s), 1.0f / kSliceCols));
+}
+
 // Row moments (mean, biased variance) of a 128-column row from its two slices'
 // moments, rounded as the general merge rounds.
 __device__ __forceinline__ float2 merge_two_slices(float2 lo, float2 hi) {

@@ -458,7 +458,10 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
     float2 mv = make_float2(0.f, 0.f);
     auto load_mv = [&](int w) {
       const int row_p = (2 * mpair(item(w).pair) + rank) * BM + q * 32 + lane;
-      if (row_p < M) mv = __ldg(reinterpret_cast<const float2*>(ep.stats_in) + row_p);
+      if (row_p >= M) return;
+      const float2* p = reinterpret_cast<const float2*>(ep.stats_in) + row_p;
+      if (BN < 256 && ep.slices_in > 0) mv = merge_slice_moments(p, m_cap, ep.slices_in);
+      else mv = __ldg(p);
     };
     if constexpr (C::kLn)
       if (cid < items) {
@@ -723,7 +726,18 @@ static cudaError_t launch_bn(const CUtensorMap& ta, const CUtensorMap& tb,
   }
 }
 
+// Whether one wave of CTA pairs holds every tile pair of that width.
+static bool one_wave(int32_t m_cap, int32_t n, int bn) {
+  const long row_pairs = (static_cast<long>(m_cap) + 2 * BM - 1) / (2 * BM);
+  return row_pairs * ((n + bn - 1) / bn) <= num_sms() / kCluster;
+}
+
 }  // namespace gemm
+
+// In one wave a CTA merges its rows' moments once, under the loads and MMAs of
+// its only tile; in more, every tile would again, and the wide tiles' epilogues
+// have no registers for it (a forward of 256 DeiT-B images 4.91 -> 5.23 ms).
+bool linear_merges(int32_t m_cap, int32_t n) { return gemm::one_wave(m_cap, n, 128); }
 
 cudaError_t launch_linear(const uint16_t* x, int32_t m_cap, const int32_t* m_dev, int32_t k,
                           const uint16_t* w, int32_t n, int32_t epilogue, const LinearEpi& ep,
@@ -735,11 +749,9 @@ cudaError_t launch_linear(const uint16_t* x, int32_t m_cap, const int32_t* m_dev
   // (DINOv2's head) on 16 clusters instead of 4, us with the pooling: 29.2 -> 25.2; a
   // DeiT-B block on one image 70.2 -> 53.2 and on eight 74.3 -> 63.1, DeiT-Tiny's on
   // eight 47.1 -> 43.8.
-  const long row_pairs = (static_cast<long>(m_cap) + 2 * gemm::BM - 1) / (2 * gemm::BM);
-  const long wave = num_sms() / gemm::kCluster;
   int bn = (n % 256 == 0) ? 256 : 128;
-  if (row_pairs * ((n + 63) / 64) <= wave) bn = 64;
-  else if (bn == 256 && row_pairs * ((n + 127) / 128) <= wave) bn = 128;
+  if (gemm::one_wave(m_cap, n, 64)) bn = 64;
+  else if (gemm::one_wave(m_cap, n, 128)) bn = 128;
   CUtensorMap ta, tb, tbt, ty, tr;
   if (lda != 0 && (lda < k || lda % 8 != 0)) return cudaErrorInvalidValue;
   if (encode_tmap_2d_bf16(&ta, x, static_cast<uint64_t>(k), static_cast<uint64_t>(m_cap),

@@ -109,17 +109,22 @@ constexpr int kEpiTokens = 6;
 struct LinearEpi {
   const uint16_t* bias = nullptr;       // bf16 [n], nullable (plain epilogues)
   const uint16_t* residual = nullptr;   // bf16 [m, n] (residual epilogue)
-  const float* stats_in = nullptr;      // row moments of x, [m_cap][2] (LN epilogues)
+  const float* stats_in = nullptr;      // moments of x (LN epilogues): of rows, [m_cap][2],
+                                        // or with slices_in > 0 slice moments
   const float* colsum = nullptr;        // fp32 [n] (LN epilogues)
   const float* colbias = nullptr;       // fp32 [n] (LN epilogues)
   float* stats_out = nullptr;           // slice moments of y, [n/64][m_cap], nullable
   float eps = 0.f;                      // LayerNorm epsilon (LN epilogues)
-  int32_t slices = 0;                   // n / 64 (stats_out)
+  int32_t slices_in = 0;                // > 0: k / 64, stats_in is [k/64][m_cap][2]
+                                        // (only where linear_merges says so)
   const uint16_t* cls = nullptr;        // bf16 [n] (kEpiTokens)
   const uint16_t* pos = nullptr;        // bf16 [tokens, n] (kEpiTokens)
   int32_t tokens = 0;                   // rows per image (kEpiTokens)
   int32_t m_reverse = 0;                // 1: walk the row blocks from the last one
 };
+// Whether a LayerNorm linear of this shape takes its input's slice moments
+// and merges them itself (the same bits as launch_merge_moments).
+bool linear_merges(int32_t m_cap, int32_t n);
 // lda: row pitch of x in elements (0 = k; a multiple of 8).
 cudaError_t launch_linear(const uint16_t* x, int32_t m_cap, const int32_t* m_dev, int32_t k,
                           const uint16_t* w, int32_t n, int32_t epilogue, const LinearEpi& ep,

@@ -2,6 +2,8 @@
 against the fp64 oracle on the same seeded inputs.  Integer and byte outputs
 (kept_idx, cu_seqlens, ids, packed rows) must match bit for bit; floating
 outputs within |err| <= 2e-2 or |err| <= 1e-2 |ref|."""
+from dataclasses import replace
+
 import numpy as np
 import pytest
 import torch
@@ -1047,6 +1049,21 @@ def test_block_prefolded_weights_give_the_same_bits():
         assert a["status"] == 0 and b["status"] == 0
         assert torch.equal(a["x_out"], b["x_out"])
         assert np.array_equal(a["cu_out"], b["cu_out"])
+
+
+@pytest.mark.parametrize("dim", [64, 128, 1024, 1152])
+def test_block_in_one_wave_merges_its_moments_in_fc1(dim):
+    """A small block's fc1 merges its input's slice moments itself (1, 2, 16 or
+    18 of them); a buffer of more rows takes the separate merge: same bits."""
+    cfg = replace(S.get_config("cfg1"), batch=3, n_tokens=67, dim=dim, heads=dim // 64,
+                  mlp_dim=4 * dim)
+    cu, ids = S.initial_layout(cfg)
+    x = S.activations_bf16(cfg, 29)
+    wf = _device_weights(cfg, S.block_weights(cfg, 1, 29, random_affine=True)).fold()
+    one = _run_block(cfg, x, cu, ids, wf)
+    many = _run_block(cfg, x, cu, ids, wf, t_cap=256 * 80)
+    assert one["status"] == many["status"] == 0
+    assert torch.equal(one["x_out"][:cu[-1]], many["x_out"][:cu[-1]])
 
 
 @pytest.mark.parametrize("name,scored", [("cfg1", False), ("cfg1", True), ("cfg2", True)])
