@@ -1,19 +1,24 @@
 // The deterministic actor of DORA at deployment (Sec. 3.2 "The actor";
 // Appendix A.1-A.3), at one block, for every image of a packed batch:
 //   gate      p = sigmoid(MLP_G([K_CLS, e^G_l, h_l])), a (d + 19) -> 64 -> 1
-//             SiLU MLP: one CTA per image;
+//             SiLU MLP;
 //   encoder   X = W_in K + b_in + e^C_l (+ W_h h_l on the CLS row), then one
 //             pre-LayerNorm Transformer block of width 128 (four heads of 32,
-//             GELU feed-forward 128 -> 256 -> 128): input projection and QKV on
-//             the library's tcgen05 GEMM (LayerNorm folded in), the varlen
-//             attention, and all that follows it in one kernel
-//             (actor_tail.cu);
+//             GELU feed-forward 128 -> 256 -> 128): input projection (writing the
+//             slice moments of X) and QKV (LayerNorm folded in) on the library's
+//             tcgen05 GEMM, the varlen attention, and all that follows it in one
+//             kernel (actor_tail.cu);
 //   budget    the highest logit of MLP_B(LayerNorm(Z_CLS)) among the budgets
 //             k <= N_l - 4 (ties to the smaller), and
 //   selector  s_j = MLP_S(Z_j + W_k k / N_l), a 128 -> 64 -> 1 SiLU MLP,
 //             written W_1 Z_j + b_1 + (k / N_l) W_1 W_k: the first term comes
 //             with Z, W_1 W_k is made once per set of weights, and the rest runs
 //             per token.
+// Six launches: gate, budget and the selector's rest are the last one (one CTA
+// per image), and the history term a small one after the input projection.  With
+// a launch each for gate with history, row moments, budget and selector the call
+// took 133.6 us at 256 x 197 tokens, now 111.9; 8 ragged images of d = 384 took
+// 53.5, now 37.9.
 // The attention kernel has an instance for heads of 32 (softmax scale
 // 1/sqrt(32)).  On heads zero-padded to 64 the QKV linear wrote twice the bytes
 // and both MMAs did twice the work: 256 x 197 tokens, QKV 29.7 -> 16.5 us,
@@ -40,7 +45,6 @@ constexpr int SH = 64;          // selector hidden units
 constexpr int kMaxDim = 2048;
 constexpr int kMaxN0 = 1028;    // budget-head outputs (n0 - 4) / 2 <= 512
 constexpr int kMaxBudgets = (kMaxN0 - 4) / 2;
-constexpr int kGateStagedInputs = 1536;   // gate weights staged in shared memory up to d + 19 = 1536
 
 __device__ __forceinline__ float ld(const uint16_t* __restrict__ p, size_t i) {
   return __uint_as_float(static_cast<uint32_t>(p[i]) << 16);
@@ -48,6 +52,10 @@ __device__ __forceinline__ float ld(const uint16_t* __restrict__ p, size_t i) {
 __device__ __forceinline__ uint16_t to_bf16(float v) {
   const __nv_bfloat16 h = __float2bfloat16_rn(v);
   return *reinterpret_cast<const uint16_t*>(&h);
+}
+__device__ __forceinline__ float4 bf16x4(uint2 v) {
+  return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u),
+                     __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xFFFF0000u));
 }
 __device__ __forceinline__ float silu(float x) { return x / (1.f + expf(-x)); }
 __device__ __forceinline__ float gelu(float x) {
@@ -80,10 +88,7 @@ __global__ void bias_in_kernel(const uint16_t* __restrict__ b_in, const uint16_t
 }
 
 // ---------------------------------------------------------------------------
-// gate (Appendix A.1) and budget head (Sec. 3.2; Appendix A.1-A.3): one CTA per
-// image.  Their weights are transposed once ([inputs, outputs]), so the
-// threads computing neighbouring outputs read each input's weights together,
-// and every thread keeps several independent loads in flight.
+// W^T of the gate's first layer, [inputs, outputs]
 // ---------------------------------------------------------------------------
 __global__ void transpose_kernel(const uint16_t* __restrict__ w, int rows, int cols,
                                  uint16_t* __restrict__ wt) {
@@ -94,232 +99,326 @@ __global__ void transpose_kernel(const uint16_t* __restrict__ w, int rows, int c
   }
 }
 
-// Copy n16 16-byte words from global to shared memory, 8 loads in flight.
-__device__ __forceinline__ void stage(uint4* __restrict__ dst, const uint4* __restrict__ src,
-                                      int n16) {
-  int i = threadIdx.x;
-  for (; i + 7 * static_cast<int>(blockDim.x) < n16; i += 8 * blockDim.x) {
-    uint4 v[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = src[i + e * blockDim.x];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) dst[i + e * blockDim.x] = v[e];
-  }
-  for (; i < n16; i += blockDim.x) dst[i] = src[i];
+// h_l = [N_l / N0, rho_l, E_<l / (L - 1)]
+struct History {
+  float h0, h1, h2;
+};
+__device__ __forceinline__ History history(int n, int n0, const float* __restrict__ rho,
+                                           const int32_t* __restrict__ interventions, int depth,
+                                           int i) {
+  return {static_cast<float>(n) / static_cast<float>(n0), rho[i],
+          static_cast<float>(interventions[i]) / static_cast<float>(max(depth - 1, 1))};
+}
+// Visual tokens of the image with bounds [lo, hi); -1 if it is empty or
+// outside the buffer.
+__device__ __forceinline__ int visual_tokens(int lo, int hi, int t_cap) {
+  return (lo < 0 || hi > t_cap) ? -1 : hi - lo - 1;
 }
 
-// sum_c wt[c * stride + o] * v[c] over c in [c0, c1), 8 loads in flight
-__device__ __forceinline__ float dot_t(const uint16_t* __restrict__ wt, int stride, int o,
-                                       const float* __restrict__ v, int c0, int c1) {
-  float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  int c = c0;
-  for (; c + 7 < c1; c += 8) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) a[e] = fmaf(ld(wt, static_cast<size_t>(c + e) * stride + o), v[c + e], a[e]);
-  }
-  for (; c < c1; ++c) a[0] = fmaf(ld(wt, static_cast<size_t>(c) * stride + o), v[c], a[0]);
-  return ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
-}
-
-// h_l = [N_l / N0, rho_l, E_<l / (L - 1)]; the gate logit and p^G; and W_h h_l
-// added to the image's CLS row of the encoder input x [rows, 128].  256
-// threads: hidden unit t % 64 over a quarter t / 64 of the d + 19 inputs.
-__global__ void __launch_bounds__(256) gate_kernel(
-    const uint16_t* __restrict__ qkv, int dim, const int32_t* __restrict__ cu, int t_cap,
-    int block, int depth, int n0, const float* __restrict__ rho,
-    const int32_t* __restrict__ interventions, const uint16_t* __restrict__ w1t,
-    const uint16_t* __restrict__ b1, const uint16_t* __restrict__ w2,
-    const uint16_t* __restrict__ b2, const uint16_t* __restrict__ emb,
-    const uint16_t* __restrict__ w_h, uint16_t* __restrict__ x, float* __restrict__ glogit,
-    float* __restrict__ p_gate) {
-  __shared__ float z[kMaxDim + GE + 3];
-  __shared__ float part[4][GH];
-  extern __shared__ __align__(16) uint4 wsm[];          // W_1^T when it fits (else empty)
+// ---------------------------------------------------------------------------
+// history: W_h h_l enters the encoder's input x [rows, 128] on each image's CLS
+// row, whose slice moments sm [2][t_cap] change with it.  One warp per image,
+// four columns a lane (a slice is half a warp).
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(128) history_kernel(
+    const int32_t* __restrict__ cu, int batch, int t_cap, int depth, int n0,
+    const float* __restrict__ rho, const int32_t* __restrict__ interventions,
+    const uint16_t* __restrict__ w_h, uint16_t* __restrict__ x, float2* __restrict__ sm) {
   pdl_trigger();
   pdl_wait();
-  const int i = blockIdx.x, t = threadIdx.x;
-  const int lo = cu[i], hi = cu[i + 1];
-  const int n = (lo < 0 || hi > t_cap) ? -1 : hi - lo - 1;   // visual tokens
-  const int kin_ = dim + GE + 3;
-  const bool staged = kin_ <= kGateStagedInputs;
-  if (staged && n >= 0) stage(wsm, reinterpret_cast<const uint4*>(w1t), kin_ * GH * 2 / 16);
-  if (n < 0) {                                       // empty (or outside the buffer): closed
-    if (t == 0) {
-      glogit[i] = -INFINITY;
-      if (p_gate != nullptr) p_gate[i] = 0.f;
-    }
-    return;
-  }
-  const float h0 = static_cast<float>(n) / static_cast<float>(n0);
-  const float h1 = rho[i];
-  const float h2 = static_cast<float>(interventions[i]) / static_cast<float>(max(depth - 1, 1));
-  const int kin = dim + GE + 3;
-  const size_t krow = static_cast<size_t>(lo) * 3 * dim + dim;   // the CLS key
-  for (int c = t; c < dim; c += blockDim.x) z[c] = ld(qkv, krow + c);
-  if (t < GE) z[dim + t] = ld(emb, static_cast<size_t>(block) * GE + t);
-  if (t == 0) {
-    z[dim + GE] = h0;
-    z[dim + GE + 1] = h1;
-    z[dim + GE + 2] = h2;
-  }
-  __syncthreads();
-  {
-    const int h = t % GH, q = t / GH;
-    const int c0 = (kin * q) / 4, c1 = (kin * (q + 1)) / 4;
-    part[q][h] = dot_t(staged ? reinterpret_cast<const uint16_t*>(wsm) : w1t, GH, h, z, c0, c1);
-  }
-  __syncthreads();
-  if (t < 32) {
-    float s = 0.f;
+  const int i = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32, lane = threadIdx.x & 31;
+  if (i >= batch) return;
+  const int lo = cu[i], n = visual_tokens(lo, cu[i + 1], t_cap);
+  if (n < 0) return;
+  const History hs = history(n, n0, rho, interventions, depth, i);
+  uint2* const xr = reinterpret_cast<uint2*>(x + static_cast<size_t>(lo) * W) + lane;
+  const uint2 old = *xr;
+  const uint32_t o[2] = {old.x, old.y};
+  uint32_t r[2];
+  float v[4];
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int h = t + 32 * e;
-      s += ld(w2, h) * silu(((part[0][h] + part[1][h]) + (part[2][h] + part[3][h])) + ld(b1, h));
-    }
-    s = warp_sum(s);
-    if (t == 0) {
-      const float lg = s + ld(b2, 0);
-      glogit[i] = lg;
-      if (p_gate != nullptr) p_gate[i] = 1.f / (1.f + expf(-lg));
-    }
+  for (int e = 0; e < 4; ++e) {
+    const int c = 4 * lane + e;
+    const float t = ld(w_h, c * 3) * hs.h0 + ld(w_h, c * 3 + 1) * hs.h1 + ld(w_h, c * 3 + 2) * hs.h2;
+    const float was = __uint_as_float((e & 1) ? o[e >> 1] & 0xFFFF0000u : o[e >> 1] << 16);
+    const uint16_t b = to_bf16(was + t);
+    v[e] = __uint_as_float(static_cast<uint32_t>(b) << 16);
+    r[e >> 1] = (e & 1) ? r[e >> 1] | (static_cast<uint32_t>(b) << 16) : b;
   }
-  // the history enters the encoder on the CLS token only
-  if (t < W) {
-    uint16_t* xr = x + static_cast<size_t>(lo) * W;
-    const float v = ld(w_h, t * 3) * h0 + ld(w_h, t * 3 + 1) * h1 + ld(w_h, t * 3 + 2) * h2;
-    xr[t] = to_bf16(ld(xr, t) + v);
+  *xr = make_uint2(r[0], r[1]);
+  float s = (v[0] + v[1]) + (v[2] + v[3]);
+#pragma unroll
+  for (int d = 8; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+  const float mean = s * (1.f / kSliceCols);
+  float q = 0.f;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) q += (v[e] - mean) * (v[e] - mean);
+#pragma unroll
+  for (int d = 8; d > 0; d >>= 1) q += __shfl_xor_sync(0xffffffffu, q, d);
+  if ((lane & 15) == 0)
+    sm[static_cast<size_t>(lane >> 4) * t_cap + lo] = make_float2(mean, q);
+}
+
+// ---------------------------------------------------------------------------
+// gate, budget head and selector tail (Appendix A.1-A.3; Eq. 2): one CTA of 16
+// warps per image.  Warps 8-15 run the gate, its first layer reading the
+// transposed weights 16 bytes (eight hidden units) at a time; warps 0-7 run the
+// budget head, each normalising Z_CLS for itself (four columns a lane) and
+// taking an output at a time of each layer.  Then the selector's tail with two
+// threads per visual token, s = w_2 . silu(S1_j + (k / N_l) W_1 W_k) + b_2, where
+// S1_j = W_1 Z_j + b_1 came with Z and k is the image's budget.
+// Latency bounds it: the chain of dependent loads, so each phase's weights are
+// in flight before its input is known.  13.8 us at 256 x 197 tokens, d = 768,
+// where the three kernels it replaces took 14, 13 and 10 (the gate staged 100 KB
+// of weights for two-byte reads, so the second wave of images waited for the
+// first); one group of 8 warps doing all in turn took 23.
+// ---------------------------------------------------------------------------
+constexpr int kDecideThreads = 512;
+constexpr int kHeadThreads = kDecideThreads / 2;     // of the budget head, and of the gate
+constexpr int kHeadWarps = kHeadThreads / 32;
+constexpr int kFlight = 8;                           // a warp's weight rows in flight
+
+__device__ __forceinline__ void bar_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+__device__ __forceinline__ void fma_bf16x8(float (&acc)[8], const uint4& w, float x) {
+  const uint32_t p[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    acc[2 * e] = fmaf(__uint_as_float(p[e] << 16), x, acc[2 * e]);
+    acc[2 * e + 1] = fmaf(__uint_as_float(p[e] & 0xFFFF0000u), x, acc[2 * e + 1]);
   }
 }
 
-// LayerNorm(Z_CLS) -> 128 -> 128 GELU -> M logits; the highest feasible logit
-// (k <= N_l - 4, ties to the smaller k) is the budget.  128 threads.
-__global__ void __launch_bounds__(128) budget_kernel(
-    const uint16_t* __restrict__ z, const int32_t* __restrict__ cu, int t_cap, int n0, float eps,
-    const uint16_t* __restrict__ ln_w, const uint16_t* __restrict__ ln_b,
-    const uint16_t* __restrict__ bw1t, const uint16_t* __restrict__ bb1,
-    const uint16_t* __restrict__ bw2t, const uint16_t* __restrict__ bb2,
-    const float* __restrict__ glogit, const int32_t* __restrict__ interventions,
-    int32_t* __restrict__ gate, int32_t* __restrict__ budget, int32_t* __restrict__ k_out,
-    int32_t* __restrict__ keep, float* __restrict__ rho_next, int32_t* __restrict__ e_next,
-    float* __restrict__ scores) {
-  __shared__ float u[W], hb[W], logit[kMaxBudgets];
-  extern __shared__ __align__(16) uint4 bsm[];          // W_1^T [128, 128], W_2^T [128, M]
+// Rows m0, m0 + kHeadWarps, ... of w [rows, 128], this lane's four columns.
+__device__ __forceinline__ void load_rows(uint2 (&r)[kFlight], const uint16_t* __restrict__ w,
+                                          int m0, int rows) {
+#pragma unroll
+  for (int e = 0; e < kFlight; ++e) {
+    const int m = m0 + e * kHeadWarps;
+    r[e] = m < rows ? __ldg(reinterpret_cast<const uint2*>(w + static_cast<size_t>(m) * W) +
+                            (threadIdx.x & 31))
+                    : make_uint2(0u, 0u);
+  }
+}
+// Their dot products with x (this lane's columns): lane e < kFlight gets row e's.
+__device__ __forceinline__ float dot_rows(const uint2 (&r)[kFlight], const float4& x) {
+  const int lane = threadIdx.x & 31;
+  float mine = 0.f;
+#pragma unroll
+  for (int e = 0; e < kFlight; ++e) {
+    float s = __uint_as_float(r[e].x << 16) * x.x;
+    s = fmaf(__uint_as_float(r[e].x & 0xFFFF0000u), x.y, s);
+    s = fmaf(__uint_as_float(r[e].y << 16), x.z, s);
+    s = fmaf(__uint_as_float(r[e].y & 0xFFFF0000u), x.w, s);
+    s = warp_sum(s);
+    if (lane == e) mine = s;
+  }
+  return mine;
+}
+
+struct DecideArgs {
+  const uint16_t* qkv;              // the block's, [t_cap, 3 dim]
+  const int32_t* cu;
+  int t_cap, dim, block, depth, n0;
+  float eps;
+  const float* rho;
+  const int32_t* interventions;
+  const uint16_t *gate_w1t, *gate_b1, *gate_w2, *gate_b2, *gate_emb;
+  const uint16_t* z;                // Z [t_cap, 128]
+  const uint16_t *ln_w, *ln_b, *bw1, *bb1, *bw2, *bb2;
+  const uint16_t* s1;               // S1 [t_cap, 64]
+  const float* sel_wk;
+  const uint16_t *sw2, *sb2;
+  float* p_gate;                    // nullable
+  int32_t *gate, *budget, *k_out, *keep;
+  float* rho_next;                  // nullable
+  int32_t* e_next;                  // nullable
+  float* scores;
+};
+
+__global__ void __launch_bounds__(kDecideThreads, 2) decide_kernel(const DecideArgs a) {
+  __shared__ float zin[kMaxDim + GE + 3];
+  __shared__ float part[kHeadWarps][GH];
+  __shared__ __align__(16) float hb[W];
+  __shared__ float logit[kMaxBudgets], swk[SH], sw2s[SH];
+  __shared__ float glogit;
+  __shared__ int s_best;
   pdl_trigger();
   pdl_wait();
   const int i = blockIdx.x, t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int lo = cu[i], hi = cu[i + 1];
-  const int n = (lo < 0 || hi > t_cap) ? -1 : hi - lo - 1;
-  const int m_out = (n0 - 4) / 2;
-  uint16_t* const w1s = reinterpret_cast<uint16_t*>(bsm);
-  uint16_t* const w2s = w1s + W * W;
-  if (n >= 0) {
-    stage(bsm, reinterpret_cast<const uint4*>(bw1t), W * W * 2 / 16);
-    stage(reinterpret_cast<uint4*>(w2s), reinterpret_cast<const uint4*>(bw2t), W * m_out * 2 / 16);
-  }
-  if (n < 0) {
+  const int lo = a.cu[i], n = visual_tokens(lo, a.cu[i + 1], a.t_cap);
+  if (n < 0) {                                       // empty (or outside the buffer): closed
     if (t == 0) {
-      gate[i] = budget[i] = k_out[i] = keep[i] = 0;
-      if (rho_next != nullptr) rho_next[i] = 0.f;
-      if (e_next != nullptr) e_next[i] = interventions[i];
+      if (a.p_gate != nullptr) a.p_gate[i] = 0.f;
+      a.gate[i] = a.budget[i] = a.k_out[i] = a.keep[i] = 0;
+      if (a.rho_next != nullptr) a.rho_next[i] = 0.f;
+      if (a.e_next != nullptr) a.e_next[i] = a.interventions[i];
     }
     return;
   }
-  const size_t zc = static_cast<size_t>(lo) * W;
-  if (warp == 0) {                                   // LayerNorm(Z_CLS)
-    float v[4];
+  const int m_out = (a.n0 - 4) / 2;
+  if (t < kHeadThreads) {
+    // ---- budget head: LayerNorm(Z_CLS) -> 128 GELU -> M logits ----
+    const uint2 zr = reinterpret_cast<const uint2*>(a.z + static_cast<size_t>(lo) * W)[lane];
+    const uint2 gr = reinterpret_cast<const uint2*>(a.ln_w)[lane];
+    const uint2 br = reinterpret_cast<const uint2*>(a.ln_b)[lane];
+    uint2 r[kFlight];
+    load_rows(r, a.bw1, warp, W);
+    const float4 zv = bf16x4(zr), gv = bf16x4(gr), bv = bf16x4(br);
+    const float mean = warp_sum((zv.x + zv.y) + (zv.z + zv.w)) * (1.f / W);
+    float4 x = make_float4(zv.x - mean, zv.y - mean, zv.z - mean, zv.w - mean);
+    const float rstd =
+        rsqrtf(warp_sum((x.x * x.x + x.y * x.y) + (x.z * x.z + x.w * x.w)) * (1.f / W) + a.eps);
+    x = make_float4(x.x * rstd * gv.x + bv.x, x.y * rstd * gv.y + bv.y, x.z * rstd * gv.z + bv.z,
+                    x.w * rstd * gv.w + bv.w);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] = ld(z, zc + lane + 32 * q);
-    const float mean = warp_sum(v[0] + v[1] + v[2] + v[3]) * (1.f / W);
-    float d2 = 0.f;
+    for (int m0 = 0; m0 < W; m0 += kFlight * kHeadWarps) {
+      const float s = dot_rows(r, x);
+      if (m0 + kFlight * kHeadWarps < W) load_rows(r, a.bw1, m0 + kFlight * kHeadWarps + warp, W);
+      else load_rows(r, a.bw2, warp, m_out);
+      const int m = m0 + lane * kHeadWarps + warp;
+      if (lane < kFlight) hb[m] = gelu(s + ld(a.bb1, m));
+    }
+    bar_sync(1, kHeadThreads);
+    const float4 h = reinterpret_cast<const float4*>(hb)[lane];
+    for (int m0 = 0; m0 < m_out; m0 += kFlight * kHeadWarps) {
+      const float s = dot_rows(r, h);
+      load_rows(r, a.bw2, m0 + kFlight * kHeadWarps + warp, m_out);
+      const int m = m0 + lane * kHeadWarps + warp;
+      if (lane < kFlight && m < m_out) logit[m] = s + ld(a.bb2, m);
+    }
+    bar_sync(1, kHeadThreads);
+    if (warp == 0) {
+      // the first of the highest among the feasible (2 (m + 1) <= n - 4); a NaN
+      // counts only in the first place, where nothing is higher than it
+      const int feasible = min(n >= 6 ? (n - 4) / 2 : 0, m_out);
+      int best = feasible;
+      float bv_ = -INFINITY;
+      for (int m = lane; m < feasible; m += 32)
+        if (logit[m] > bv_ || (best == feasible && logit[m] == bv_)) {
+          best = m;
+          bv_ = logit[m];
+        }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) d2 += (v[q] - mean) * (v[q] - mean);
-    const float rstd = rsqrtf(warp_sum(d2) * (1.f / W) + eps);
+      for (int o = 16; o > 0; o >>= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, bv_, o);
+        const int om = __shfl_xor_sync(0xffffffffu, best, o);
+        if (ov > bv_ || (ov == bv_ && om < best)) {
+          best = om;
+          bv_ = ov;
+        }
+      }
+      if (feasible == 0) best = -1;
+      else if (best == feasible || logit[0] != logit[0]) best = 0;
+      if (lane == 0) s_best = best;
+    }
+  } else {
+    // ---- gate: SiLU MLP of [K_CLS, e^G_l, h_l] ----
+    const int tg = t - kHeadThreads, kin = a.dim + GE + 3;
+    const size_t krow = static_cast<size_t>(lo) * 3 * a.dim + a.dim;   // the CLS key
+    for (int c = tg; c < a.dim; c += kHeadThreads) zin[c] = ld(a.qkv, krow + c);
+    if (tg < GE) zin[a.dim + tg] = ld(a.gate_emb, static_cast<size_t>(a.block) * GE + tg);
+    if (tg == kHeadThreads - 1) {
+      const History hs = history(n, a.n0, a.rho, a.interventions, a.depth, i);
+      zin[a.dim + GE] = hs.h0;
+      zin[a.dim + GE + 1] = hs.h1;
+      zin[a.dim + GE + 2] = hs.h2;
+    }
+    if (tg < SH) {
+      swk[tg] = a.sel_wk[tg];
+      sw2s[tg] = ld(a.sw2, tg);
+    }
+    bar_sync(2, kHeadThreads);
+    // hidden units 8 (tg % 8) .. + 7 over inputs tg / 8, tg / 8 + 32, ...
+    const uint4* w = reinterpret_cast<const uint4*>(a.gate_w1t) + tg % 8;
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int c = tg / 8; c < kin; c += 8 * 32) {
+      uint4 r[8];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int c = lane + 32 * q;
-      u[c] = (v[q] - mean) * rstd * ld(ln_w, c) + ld(ln_b, c);
+      for (int e = 0; e < 8; ++e)
+        r[e] = c + 32 * e < kin ? __ldg(w + static_cast<size_t>(c + 32 * e) * (GH / 8))
+                                : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (c + 32 * e < kin) fma_bf16x8(acc, r[e], zin[c + 32 * e]);
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], 8);
+      acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], 16);
+      if (lane < 8) part[warp - kHeadWarps][8 * lane + e] = acc[e];
+    }
+    bar_sync(2, kHeadThreads);
+    if (warp == kHeadWarps) {
+      float s = 0.f;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int h = lane + 32 * e;
+        float p[kHeadWarps];
+#pragma unroll
+        for (int q = 0; q < kHeadWarps; ++q) p[q] = part[q][h];
+        s += ld(a.gate_w2, h) *
+             silu((((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]))) +
+                  ld(a.gate_b1, h));
+      }
+      s = warp_sum(s);
+      if (lane == 0) {
+        const float lg = s + ld(a.gate_b2, 0);
+        glogit = lg;
+        if (a.p_gate != nullptr) a.p_gate[i] = 1.f / (1.f + expf(-lg));
+      }
     }
   }
-  __syncthreads();
-  hb[t] = gelu(dot_t(w1s, W, t, u, 0, W) + ld(bb1, t));
-  __syncthreads();
-  for (int m = t; m < m_out; m += blockDim.x) logit[m] = dot_t(w2s, m_out, m, hb, 0, W) + ld(bb2, m);
-  __syncthreads();
-  if (warp == 0) {
-    // the first of the highest among the feasible (2 (m + 1) <= n - 4); a NaN
-    // counts only in the first place, where nothing is higher than it
-    const int feasible = min(n >= 6 ? (n - 4) / 2 : 0, m_out);
-    int best = feasible;
-    float bv = -INFINITY;
-    for (int m = lane; m < feasible; m += 32)
-      if (logit[m] > bv || (best == feasible && logit[m] == bv)) {
-        best = m;
-        bv = logit[m];
-      }
+  // ---- selector tail: threads 2 j and 2 j + 1 take 32 hidden units each of token j ----
+  const int half = t & 1;
+  uint4 v[SH / 16];
+  auto load_s1 = [&](int j) {
+    if (j <= n) {
+      const uint4* p = reinterpret_cast<const uint4*>(a.s1 + static_cast<size_t>(lo + j) * SH) +
+                       half * (SH / 16);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-      const int om = __shfl_xor_sync(0xffffffffu, best, o);
-      if (ov > bv || (ov == bv && om < best)) {
-        best = om;
-        bv = ov;
-      }
+      for (int q = 0; q < SH / 16; ++q) v[q] = p[q];
     }
-    if (feasible == 0) best = -1;
-    else if (best == feasible || logit[0] != logit[0]) best = 0;
-    if (lane != 0) return;
-    const int bud = best < 0 ? 0 : 2 * (best + 1);
-    const int g = (glogit[i] >= 0.f && bud > 0) ? 1 : 0;
+  };
+  load_s1(1 + t / 2);
+  const float b2 = ld(a.sb2, 0);
+  __syncthreads();
+  const int bud = s_best < 0 ? 0 : 2 * (s_best + 1);
+  if (t == 0) {
+    const int g = (glogit >= 0.f && bud > 0) ? 1 : 0;
     const int kk = g ? bud : 0;
-    budget[i] = bud;
-    gate[i] = g;
-    k_out[i] = kk;
-    keep[i] = n + 1 - kk;
-    if (rho_next != nullptr) rho_next[i] = n > 0 ? static_cast<float>(kk) / n : 0.f;
-    if (e_next != nullptr) e_next[i] = interventions[i] + g;
-    scores[lo] = 0.f;
+    a.budget[i] = bud;
+    a.gate[i] = g;
+    a.k_out[i] = kk;
+    a.keep[i] = n + 1 - kk;
+    if (a.rho_next != nullptr) a.rho_next[i] = n > 0 ? static_cast<float>(kk) / n : 0.f;
+    if (a.e_next != nullptr) a.e_next[i] = a.interventions[i] + g;
+    a.scores[lo] = 0.f;
   }
-}
-
-// ---------------------------------------------------------------------------
-// selector tail (Eq. 2): one thread per visual token, s = w_2 . silu(S1_j +
-// (k / N_l) W_1 W_k) + b_2, with S1_j = W_1 Z_j + b_1 from the GEMM and k the
-// image's budget
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) selector_kernel(
-    const uint16_t* __restrict__ s1, const int32_t* __restrict__ cu, int t_cap,
-    const int32_t* __restrict__ budget, const float* __restrict__ sel_wk,
-    const uint16_t* __restrict__ sw2, const uint16_t* __restrict__ sb2,
-    float* __restrict__ scores) {
-  __shared__ float sck[SH], sw2s[SH];
-  pdl_trigger();
-  pdl_wait();
-  const int i = blockIdx.x, t = threadIdx.x;
-  const int lo = cu[i], hi = cu[i + 1];
-  const int n = (lo < 0 || hi > t_cap) ? -1 : hi - lo - 1;
-  if (n <= 0) return;
-  const float kr = static_cast<float>(budget[i]) / n;
-  if (t < SH) {
-    sck[t] = kr * sel_wk[t];
-    sw2s[t] = ld(sw2, t);
-  }
-  __syncthreads();
-  const float b2 = ld(sb2, 0);
-  for (int j = 1 + t; j <= n; j += blockDim.x) {
-    const uint4* sr = reinterpret_cast<const uint4*>(s1 + static_cast<size_t>(lo + j) * SH);
+  const float kr = static_cast<float>(bud) / n;      // n = 0: no token uses it
+  const float* wk = swk + half * (SH / 2);
+  const float* w2 = sw2s + half * (SH / 2);
+#pragma unroll 1
+  for (int j0 = 0; j0 < n; j0 += kDecideThreads / 2) {
+    const int j = 1 + j0 + t / 2;
     float acc = 0.f;
-#pragma unroll 2
-    for (int q = 0; q < SH / 8; ++q) {
-      const uint4 v = sr[q];
-      const uint32_t wv[4] = {v.x, v.y, v.z, v.w};
+    if (j <= n) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int hh = 8 * q + 2 * e;
-        acc = fmaf(sw2s[hh], silu(__uint_as_float(wv[e] << 16) + sck[hh]), acc);
-        acc = fmaf(sw2s[hh + 1], silu(__uint_as_float(wv[e] & 0xFFFF0000u) + sck[hh + 1]), acc);
+      for (int q = 0; q < SH / 16; ++q) {
+        const uint32_t wv[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int h = 8 * q + 2 * e;
+          acc = fmaf(w2[h], silu(__uint_as_float(wv[e] << 16) + kr * wk[h]), acc);
+          acc = fmaf(w2[h + 1], silu(__uint_as_float(wv[e] & 0xFFFF0000u) + kr * wk[h + 1]), acc);
+        }
       }
     }
-    scores[lo + j] = acc + b2;
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    if (j <= n && half == 0) a.scores[lo + j] = acc + b2;
+    load_s1(j + kDecideThreads / 2);
   }
 }
 
@@ -329,7 +428,7 @@ __global__ void __launch_bounds__(256) selector_kernel(
 size_t up256(size_t v) { return (v + 255) & ~static_cast<size_t>(255); }
 
 struct Prep {
-  size_t bias_in, wqkv, cqkv, dqkv, wfc1, cfc1, dfc1, sel_wk, gate_w1t, bud_w1t, bud_w2t, total;
+  size_t bias_in, wqkv, cqkv, dqkv, wfc1, cfc1, dfc1, sel_wk, gate_w1t, total;
 };
 
 Prep prep_layout(const dora_actor_weights* w) {
@@ -344,14 +443,12 @@ Prep prep_layout(const dora_actor_weights* w) {
   P.dfc1 = off;    off += up256(FF * 4);
   P.sel_wk = off;  off += up256(SH * 4);
   P.gate_w1t = off; off += up256(static_cast<size_t>(w->dim + GE + 3) * GH * 2);
-  P.bud_w1t = off; off += up256(W * W * 2);
-  P.bud_w2t = off; off += up256(static_cast<size_t>(W) * ((w->n0 - 4) / 2) * 2);
   P.total = off;
   return P;
 }
 
 struct Ws {
-  size_t status, x, mv, qkv, o, z, s1, glogit, prep, total;
+  size_t status, x, sm, qkv, o, z, s1, prep, total;
 };
 
 Ws ws_layout(int32_t t_cap, int32_t batch, const dora_actor_weights* w) {
@@ -360,16 +457,16 @@ Ws ws_layout(int32_t t_cap, int32_t batch, const dora_actor_weights* w) {
   size_t off = 0;
   L.status = off; off += 256;
   L.x = off;      off += up256(t * W * 2);
-  L.mv = off;     off += up256(t * 8);
+  L.sm = off;     off += up256(t * 2 * 8);
   L.qkv = off;    off += up256(t * 3 * W * 2);
   L.o = off;      off += up256(t * W * 2);
   L.z = off;      off += up256(t * W * 2);
   L.s1 = off;     off += up256(t * SH * 2);
-  L.glogit = off; off += up256(b * 4);
   // the size stays what it was when heads were padded to 64 and Z1, its slice
-  // moments and the feed-forward's hidden rows were kept: callers that sized
-  // the workspace by that are not refused, nor is its size a surprise to them
-  off += up256(t * (3 * W * 2 + W * 2 + W * 2 + 2 * 8 + FF * 2));
+  // moments, the feed-forward's hidden rows and the gate's logits were kept:
+  // callers that sized the workspace by that are not refused, nor is its size a
+  // surprise to them
+  off += up256(b * 4) + up256(t * (3 * W * 2 + W * 2 + W * 2 + 8 + FF * 2));
   L.prep = off;   off += w->prepared != nullptr ? 0 : prep_layout(w).total;
   L.total = off;
   return L;
@@ -404,10 +501,6 @@ cudaError_t prepare(const dora_actor_weights* w, uint8_t* prep, cudaStream_t str
   sel_wk_kernel<<<1, SH, 0, stream>>>(w->sel_w1, w->sel_w_k, reinterpret_cast<float*>(prep + P.sel_wk));
   transpose_kernel<<<64, 256, 0, stream>>>(w->gate_w1, GH, w->dim + GE + 3,
                                            reinterpret_cast<uint16_t*>(prep + P.gate_w1t));
-  transpose_kernel<<<64, 256, 0, stream>>>(w->bud_w1, W, W,
-                                           reinterpret_cast<uint16_t*>(prep + P.bud_w1t));
-  transpose_kernel<<<64, 256, 0, stream>>>(w->bud_w2, (w->n0 - 4) / 2, W,
-                                           reinterpret_cast<uint16_t*>(prep + P.bud_w2t));
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_fold_ln(w->enc_w_fc1, FF, W, w->enc_ln2_w, w->enc_ln2_b, w->enc_b_fc1,
@@ -480,11 +573,10 @@ int dora_actor(const dora_bf16* qkv, const int32_t* cu, int32_t batch, int32_t m
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   int32_t* status = reinterpret_cast<int32_t*>(ws + L.status);
   uint16_t* x = reinterpret_cast<uint16_t*>(ws + L.x);
-  float* mv = reinterpret_cast<float*>(ws + L.mv);
+  float* sm = reinterpret_cast<float*>(ws + L.sm);
   uint16_t* qkv_e = reinterpret_cast<uint16_t*>(ws + L.qkv);
   uint16_t* o_e = reinterpret_cast<uint16_t*>(ws + L.o);
   uint16_t* z = z_out != nullptr ? z_out : reinterpret_cast<uint16_t*>(ws + L.z);
-  float* glogit = reinterpret_cast<float*>(ws + L.glogit);
   uint8_t* prep = ws + L.prep;
   if (w->prepared != nullptr) prep = static_cast<uint8_t*>(const_cast<void*>(w->prepared));
   else if (prepare(w, prep, stream) != cudaSuccess) return DORA_ERR_CUDA;
@@ -492,40 +584,31 @@ int dora_actor(const dora_bf16* qkv, const int32_t* cu, int32_t batch, int32_t m
   const int32_t* rows = cu + batch;
   const int d = w->dim;
 
-  // X = W_in K + (b_in + e^C_l), K read in place from the block's qkv rows
+  // X = W_in K + (b_in + e^C_l), K read in place from the block's qkv rows, and
+  // the slice moments of its rows; then the history term on every CLS row
   LinearEpi e_in;
   e_in.bias = reinterpret_cast<const uint16_t*>(prep + P.bias_in) + static_cast<size_t>(block) * W;
-  if (launch_linear(qkv + d, t_cap, rows, d, w->enc_w_in, W, DORA_EPI_BIAS, e_in, x, status,
-                    stream, 3 * d) != cudaSuccess)
+  e_in.stats_out = sm;
+  if (launch_linear(qkv + d, t_cap, rows, d, w->enc_w_in, W, kEpiStats, e_in, x, status, stream,
+                    3 * d) != cudaSuccess ||
+      launch_pdl(history_kernel, dim3((batch + 3) / 4), dim3(128), 0, stream, cu, batch, t_cap,
+                 w->depth, w->n0, rho, interventions, w->enc_w_h, x,
+                 reinterpret_cast<float2*>(sm)) != cudaSuccess)
     return DORA_ERR_CUDA;
-  // gate, and the history term on every CLS row
-  const int kin = d + GE + 3;
-  const size_t gate_smem = kin <= kGateStagedInputs ? static_cast<size_t>(kin) * GH * 2 : 0;
-  const size_t bud_smem = static_cast<size_t>(W) * (W + (w->n0 - 4) / 2) * 2;
-  if (cudaFuncSetAttribute(gate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(gate_smem)) != cudaSuccess ||
-      cudaFuncSetAttribute(budget_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(bud_smem)) != cudaSuccess)
-    return DORA_ERR_CUDA;
-  if (launch_pdl(gate_kernel, dim3(batch), dim3(256), gate_smem, stream, qkv, d, cu, t_cap, block,
-                 w->depth, w->n0, rho, interventions,
-                 reinterpret_cast<const uint16_t*>(prep + P.gate_w1t), w->gate_b1, w->gate_w2,
-                 w->gate_b2, w->gate_emb, w->enc_w_h, x, glogit, p_gate) != cudaSuccess)
-    return DORA_ERR_CUDA;
-  // Attention(LayerNorm1(X))
+  // Attention(LayerNorm1(X)); the 384-column linear merges the two slices itself
   LinearEpi e_q;
-  e_q.stats_in = mv;
+  e_q.stats_in = sm;
+  e_q.slices_in = W / kSliceCols;
   e_q.colsum = reinterpret_cast<const float*>(prep + P.cqkv);
   e_q.colbias = reinterpret_cast<const float*>(prep + P.dqkv);
   e_q.eps = w->eps;
-  if (launch_row_stats(x, t_cap, rows, W, mv, stream) != cudaSuccess ||
-      launch_linear(x, t_cap, rows, W, reinterpret_cast<const uint16_t*>(prep + P.wqkv),
-                    3 * W, kEpiLn, e_q, qkv_e, status, stream) != cudaSuccess ||
+  if (launch_linear(x, t_cap, rows, W, reinterpret_cast<const uint16_t*>(prep + P.wqkv), 3 * W,
+                    kEpiLn, e_q, qkv_e, status, stream) != cudaSuccess ||
       launch_varlen_attn(qkv_e, cu, batch, max_seqlen, t_cap, HEADS, 0.17677669529663688f, o_e,
                          status, stream, HD) != cudaSuccess)
     return DORA_ERR_CUDA;
   // output projection, feed-forward and the selector's first layer on every
-  // token, then budget head and selector tail
+  // token, then gate, budget head and selector tail
   uint16_t* s1 = reinterpret_cast<uint16_t*>(ws + L.s1);
   TailArgs ta;
   ta.x = x;
@@ -540,15 +623,42 @@ int dora_actor(const dora_bf16* qkv, const int32_t* cu, int32_t batch, int32_t m
   if (launch_actor_tail(o_e, w->enc_w_o, reinterpret_cast<const uint16_t*>(prep + P.wfc1),
                         w->enc_w_fc2, w->sel_w1, ta, t_cap, rows, status, stream) != cudaSuccess)
     return DORA_ERR_CUDA;
-  if (launch_pdl(budget_kernel, dim3(batch), dim3(128), bud_smem, stream, z, cu, t_cap, w->n0,
-                 w->eps, w->bud_ln_w, w->bud_ln_b,
-                 reinterpret_cast<const uint16_t*>(prep + P.bud_w1t), w->bud_b1,
-                 reinterpret_cast<const uint16_t*>(prep + P.bud_w2t), w->bud_b2, glogit,
-                 interventions, gate, budget, k, keep_counts, rho_next, interventions_next,
-                 scores) != cudaSuccess ||
-      launch_pdl(selector_kernel, dim3(batch), dim3(256), 0, stream, s1, cu, t_cap, budget,
-                 reinterpret_cast<const float*>(prep + P.sel_wk), w->sel_w2, w->sel_b2,
-                 scores) != cudaSuccess)
+  DecideArgs da;
+  da.qkv = qkv;
+  da.cu = cu;
+  da.t_cap = t_cap;
+  da.dim = d;
+  da.block = block;
+  da.depth = w->depth;
+  da.n0 = w->n0;
+  da.eps = w->eps;
+  da.rho = rho;
+  da.interventions = interventions;
+  da.gate_w1t = reinterpret_cast<const uint16_t*>(prep + P.gate_w1t);
+  da.gate_b1 = w->gate_b1;
+  da.gate_w2 = w->gate_w2;
+  da.gate_b2 = w->gate_b2;
+  da.gate_emb = w->gate_emb;
+  da.z = z;
+  da.ln_w = w->bud_ln_w;
+  da.ln_b = w->bud_ln_b;
+  da.bw1 = w->bud_w1;
+  da.bb1 = w->bud_b1;
+  da.bw2 = w->bud_w2;
+  da.bb2 = w->bud_b2;
+  da.s1 = s1;
+  da.sel_wk = reinterpret_cast<const float*>(prep + P.sel_wk);
+  da.sw2 = w->sel_w2;
+  da.sb2 = w->sel_b2;
+  da.p_gate = p_gate;
+  da.gate = gate;
+  da.budget = budget;
+  da.k_out = k;
+  da.keep = keep_counts;
+  da.rho_next = rho_next;
+  da.e_next = interventions_next;
+  da.scores = scores;
+  if (launch_pdl(decide_kernel, dim3(batch), dim3(kDecideThreads), 0, stream, da) != cudaSuccess)
     return DORA_ERR_CUDA;
   return DORA_OK;
 }

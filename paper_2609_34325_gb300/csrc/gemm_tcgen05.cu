@@ -90,11 +90,13 @@ struct Cfg {
   static constexpr bool kLn = EPI == kEpiLn || EPI == kEpiLnGelu;
   static constexpr bool kResTma =
       EPI == DORA_EPI_BIAS_RESIDUAL || EPI == kEpiResidualLongK || EPI == kEpiTokens;
+  // slice moments of the output rows, where the caller takes them
+  static constexpr bool kMoments = (kResTma && EPI != kEpiTokens) || EPI == kEpiStats;
   // the two GELU epilogues are ALU-bound: 16 warps; the others 8.  A 64-wide
-  // tile has 32 columns for each of 8 warps; the residual's need whole
-  // 64-column slices: 4
+  // tile has 32 columns for each of 8 warps; those that write moments need
+  // whole 64-column slices: 4
   static constexpr int kEpiWarps =
-      BN == 64 ? (kResTma ? 4 : 8)
+      BN == 64 ? (kResTma || EPI == kEpiStats ? 4 : 8)
                : ((EPI == DORA_EPI_BIAS_GELU || EPI == kEpiLnGelu) ? 16 : 8);
   static constexpr int kColGroups = kEpiWarps / 4;
   static constexpr int kCols = BN / kColGroups;         // columns per epilogue warp
@@ -455,13 +457,17 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
     };
     // Folded LayerNorm: (mean, var) of this lane's row, loaded a tile ahead
     // (a warp's 32 rows are one 256-byte load).
-    float2 mv = make_float2(0.f, 0.f);
+    float2 mv = make_float2(0.f, 0.f), mv2 = mv;
     auto load_mv = [&](int w) {
       const int row_p = (2 * mpair(item(w).pair) + rank) * BM + q * 32 + lane;
       if (row_p >= M) return;
       const float2* p = reinterpret_cast<const float2*>(ep.stats_in) + row_p;
-      if (BN < 256 && ep.slices_in > 0) mv = merge_slice_moments(p, m_cap, ep.slices_in);
-      else mv = __ldg(p);
+      if (BN < 256 && ep.slices_in > 0 && ep.slices_in != 2) {
+        mv = merge_slice_moments(p, m_cap, ep.slices_in);
+        return;
+      }
+      mv = __ldg(p);
+      if (BN < 256 && ep.slices_in == 2) mv2 = __ldg(p + m_cap);    // merged when used
     };
     if constexpr (C::kLn)
       if (cid < items) {
@@ -485,6 +491,7 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
       const bool past_image = EPI == kEpiTokens && row0 % ep.tokens + lane >= ep.tokens;
       float neg_mean = 0.f, rstd = 0.f;           // folded LayerNorm of this row
       if constexpr (C::kLn) {
+        if (BN < 256 && ep.slices_in == 2) mv = merge_two_slices(mv, mv2);
         neg_mean = -mv.x;
         rstd = rsqrtf(mv.y + ep.eps);
         if (w + n_clusters < items) load_mv(w + n_clusters);
@@ -570,7 +577,7 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
                                             rowp + ((j ^ ((lane >> 1) & 3)) << 4)));
             }
             pack_row(v, o);
-            if constexpr (C::kResTma && EPI != kEpiTokens)
+            if constexpr (C::kMoments)
               if (ep.stats_out != nullptr) emit_moments(o, row, gcol);
 #pragma unroll
             for (int j = 0; j < 4; ++j)
@@ -599,7 +606,7 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
               for (int j = 0; j < 4; ++j) add_bf16x8(v + 8 * j, __ldg(rp + j));
             }
             pack_row(v, o);
-            if constexpr (C::kResTma && EPI != kEpiTokens)
+            if constexpr (C::kMoments)
               if (ep.stats_out != nullptr) emit_moments(o, row, gcol);
             uint4* yp = reinterpret_cast<uint4*>(Y + static_cast<size_t>(row) * N + gcol);
 #pragma unroll
@@ -717,6 +724,9 @@ static cudaError_t launch_bn(const CUtensorMap& ta, const CUtensorMap& tb,
       return launch(launch_bn_epi<BN, kEpiResidualLongK, kPair>);
     case kEpiTokens:
       return launch(launch_bn_epi<BN, kEpiTokens, kPair>);
+    case kEpiStats:                             // the actor's width: never 256 wide
+      if constexpr (BN < 256) return launch(launch_bn_epi<BN, kEpiStats, kPair>);
+      return cudaErrorInvalidValue;
     case kEpiLn:
       return launch(launch_bn_epi<BN, kEpiLn, kPair>);
     case kEpiLnGelu:

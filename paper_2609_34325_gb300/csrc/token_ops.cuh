@@ -103,9 +103,12 @@ cudaError_t launch_gather_scores(const float* table, int32_t stride, const int32
 // with rstd_r = 1/sqrt(var_r + eps) from the row moments (stats_in);
 // and the patch embedding's, row r being token j = r mod tokens of its image:
 //   kEpiTokens  y = x w^T + bias + pos[j], for j = 0 (CLS) y = cls + pos[0]
+// and, for n that is no multiple of 256,
+//   kEpiStats   y = x w^T + bias, with the slice moments of y's rows
 constexpr int kEpiLn = 3;
 constexpr int kEpiLnGelu = 4;
 constexpr int kEpiTokens = 6;
+constexpr int kEpiStats = 7;
 struct LinearEpi {
   const uint16_t* bias = nullptr;       // bf16 [n], nullable (plain epilogues)
   const uint16_t* residual = nullptr;   // bf16 [m, n] (residual epilogue)
@@ -116,7 +119,8 @@ struct LinearEpi {
   float* stats_out = nullptr;           // slice moments of y, [n/64][m_cap], nullable
   float eps = 0.f;                      // LayerNorm epsilon (LN epilogues)
   int32_t slices_in = 0;                // > 0: k / 64, stats_in is [k/64][m_cap][2]
-                                        // (only where linear_merges says so)
+                                        // (where linear_merges says so, or n is no
+                                        // multiple of 256)
   const uint16_t* cls = nullptr;        // bf16 [n] (kEpiTokens)
   const uint16_t* pos = nullptr;        // bf16 [tokens, n] (kEpiTokens)
   int32_t tokens = 0;                   // rows per image (kEpiTokens)

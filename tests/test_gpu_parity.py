@@ -1407,6 +1407,34 @@ def test_actor_edges_short_images_and_gate_bias():
         _check_actor(cfg, cu, qkv, rho, e_prev, wa, got, 0, [0, 1, 2, 3, 4, 6, 7])
 
 
+@pytest.mark.parametrize("lens,dim,n0", [
+    ([1], 64, 6), ([7, 120], 64, 10), ([128], 128, 140), ([129], 128, 140),
+    ([700, 1029, 0, 300], 64, 1028), ([50, 2, 130], 2048, 196), ([197] * 100, 64, 196),
+])
+def test_actor_at_tile_edges_and_the_ends_of_its_ranges(lens, dim, n0):
+    """Rows on both sides of a 128-row tile and more tiles than SMs (19,700
+    rows); 1, 3 and 512 budgets, images of more tokens than the selector takes
+    at once, the narrowest and the widest keys; and Z on a 16-byte boundary."""
+    cfg = replace(S.get_config("cfg1"), dim=dim, heads=dim // 64, n_tokens=n0 + 1,
+                  batch=len(lens), depth=3)
+    cu, qkv, rho, e_prev, wa, aw = _actor_case(cfg, 51, gate_bias=0.5, lens=np.array(lens))
+    got = _run_actor(cfg, cu, qkv, rho, e_prev, aw, 1, max(lens))
+    b, t = len(lens), int(cu[-1])
+    images = [i for i in (range(b) if b <= 8 else (0, 1, 64, b - 1)) if lens[i] > 0]
+    _check_actor(cfg, cu, qkv, rho, e_prev, wa, got, 1, images)
+    buf = torch.zeros(t * 128 + 16, dtype=torch.bfloat16, device=dev())
+    off = 8 if buf.data_ptr() % 32 == 0 else 16
+    z = buf[off:off + t * 128].view(t, 128)
+    assert z.data_ptr() % 32 == 16
+    scores = torch.full((t,), 5.0, dtype=torch.float32, device=dev())
+    i32z = [torch.zeros(b, dtype=torch.int32, device=dev()) for _ in range(4)]
+    P.dora_actor(bf(qkv), i32(cu), aw, 1, max(lens), f32(rho), i32(e_prev), *i32z, scores,
+                 P.alloc_actor_workspace(t, b, aw), z_out=z)
+    torch.cuda.synchronize()
+    assert np.array_equal(f64(z), got["z"]) and np.array_equal(scores.cpu().numpy(), got["scores"])
+    assert torch.all(buf[:off] == 0) and torch.all(buf[off + t * 128:] == 0)
+
+
 @pytest.mark.parametrize("given_counts", [True, False])
 def test_block_with_actor_equals_actor_then_block(given_counts):
     """dora_pruned_block_actor gives the same bits as running dora_actor on the
