@@ -16,10 +16,9 @@ warmup + iters launches, then the attention.
 With ``--mixes CFG`` it times only the varlen attention, on the length mixes
 of that configuration's seeded deletion schedule (the full-length batch, then
 the batch after each pruning block), each twice: with max_seqlen set to the
-mix's own longest image and to the configuration's token count N.  The
-attention picks its kernel from max_seqlen (the short-image kernel up to 256,
-the per-key-half kernel beyond), so the two lines show what a caller that
-knows the kept maximum would gain over one that passes N.
+mix's own longest image and to the configuration's token count N.  max_seqlen
+bounds the attention's grid, so the two lines show what a caller that knows
+the kept maximum would gain over one that passes N.
 """
 from __future__ import annotations
 

@@ -87,13 +87,14 @@ class ShadowRollout:
 
     def launches(self) -> int:
         """Kernel launches of one forward() without the head (for reporting)."""
-        n = 2                                           # Native branch: scan + copy
+        branch = 1 if self.groups["native"] <= 4096 else 2   # past that scan and copy
+        n = branch                                      # Native
         for l in range(self.depth):
             n += 6 + (l == 0) + (l + 1 < self.depth)
             if l in self.prune:
-                n += 3                                  # gather, select, compact
+                n += 1                                  # gather; deletion for the merge
                 if l in self.branch_at:
-                    n += 2
+                    n += branch
         return n
 
     def forward(self, x0, cu0, ids0, tables, keeps, stream=None, stop=None, gumbel=None,
