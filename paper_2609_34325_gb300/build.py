@@ -23,7 +23,7 @@ LIB_PATH = os.path.join(HERE, "libdora.so")
 TIMEOUT_TEST_LIB_PATH = os.path.join(HERE, "libdora_timeout_test.so")
 TIMEOUT_TEST_FLAGS = ["-DDORA_TEST_WITHHOLD_KV_LOAD", "-DDORA_TEST_WAIT_LIMIT_NS=5000000ull"]
 SOURCES = ["token_ops.cu", "gemm_tcgen05.cu", "attn_tcgen05.cu", "api.cu", "noalloc.cu",
-           "actor.cu", "actor_tail.cu", "embed_head.cu", "training.cu"]
+           "actor.cu", "actor_front.cu", "actor_tail.cu", "embed_head.cu", "training.cu"]
 # the attention translation unit, rebuilt with the test flags for the timeout-path library
 ATTN_SOURCES = ("attn_tcgen05.cu",)
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

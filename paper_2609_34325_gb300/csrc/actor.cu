@@ -4,21 +4,19 @@
 //             SiLU MLP;
 //   encoder   X = W_in K + b_in + e^C_l (+ W_h h_l on the CLS row), then one
 //             pre-LayerNorm Transformer block of width 128 (four heads of 32,
-//             GELU feed-forward 128 -> 256 -> 128): input projection (writing the
-//             slice moments of X) and QKV (LayerNorm folded in) on the library's
-//             tcgen05 GEMM, the varlen attention, and all that follows it in one
-//             kernel (actor_tail.cu);
+//             GELU feed-forward 128 -> 256 -> 128): X and QKV in one kernel
+//             (actor_front.cu), the varlen attention, and all that follows it in
+//             another (actor_tail.cu);
 //   budget    the highest logit of MLP_B(LayerNorm(Z_CLS)) among the budgets
 //             k <= N_l - 4 (ties to the smaller), and
 //   selector  s_j = MLP_S(Z_j + W_k k / N_l), a 128 -> 64 -> 1 SiLU MLP,
 //             written W_1 Z_j + b_1 + (k / N_l) W_1 W_k: the first term comes
 //             with Z, W_1 W_k is made once per set of weights, and the rest runs
 //             per token.
-// Six launches: gate, budget and the selector's rest are the last one (one CTA
-// per image), and the history term a small one after the input projection.  With
-// a launch each for gate with history, row moments, budget and selector the call
-// took 133.6 us at 256 x 197 tokens, now 111.9; 8 ragged images of d = 384 took
-// 53.5, now 37.9.
+// Four launches: gate, budget and the selector's rest are the last one (one CTA
+// per image).  With a launch each for the input projection, gate with history, row
+// moments, QKV, budget and selector the call took 133.6 us at 256 x 197 tokens, now
+// 107.3; 8 ragged images of d = 384 took 53.5, now 37.9.
 // The attention kernel has an instance for heads of 32 (softmax scale
 // 1/sqrt(32)).  On heads zero-padded to 64 the QKV linear wrote twice the bytes
 // and both MMAs did twice the work: 256 x 197 tokens, QKV 29.7 -> 16.5 us,
@@ -113,50 +111,6 @@ __device__ __forceinline__ History history(int n, int n0, const float* __restric
 // outside the buffer.
 __device__ __forceinline__ int visual_tokens(int lo, int hi, int t_cap) {
   return (lo < 0 || hi > t_cap) ? -1 : hi - lo - 1;
-}
-
-// ---------------------------------------------------------------------------
-// history: W_h h_l enters the encoder's input x [rows, 128] on each image's CLS
-// row, whose slice moments sm [2][t_cap] change with it.  One warp per image,
-// four columns a lane (a slice is half a warp).
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) history_kernel(
-    const int32_t* __restrict__ cu, int batch, int t_cap, int depth, int n0,
-    const float* __restrict__ rho, const int32_t* __restrict__ interventions,
-    const uint16_t* __restrict__ w_h, uint16_t* __restrict__ x, float2* __restrict__ sm) {
-  pdl_trigger();
-  pdl_wait();
-  const int i = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32, lane = threadIdx.x & 31;
-  if (i >= batch) return;
-  const int lo = cu[i], n = visual_tokens(lo, cu[i + 1], t_cap);
-  if (n < 0) return;
-  const History hs = history(n, n0, rho, interventions, depth, i);
-  uint2* const xr = reinterpret_cast<uint2*>(x + static_cast<size_t>(lo) * W) + lane;
-  const uint2 old = *xr;
-  const uint32_t o[2] = {old.x, old.y};
-  uint32_t r[2];
-  float v[4];
-#pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    const int c = 4 * lane + e;
-    const float t = ld(w_h, c * 3) * hs.h0 + ld(w_h, c * 3 + 1) * hs.h1 + ld(w_h, c * 3 + 2) * hs.h2;
-    const float was = __uint_as_float((e & 1) ? o[e >> 1] & 0xFFFF0000u : o[e >> 1] << 16);
-    const uint16_t b = to_bf16(was + t);
-    v[e] = __uint_as_float(static_cast<uint32_t>(b) << 16);
-    r[e >> 1] = (e & 1) ? r[e >> 1] | (static_cast<uint32_t>(b) << 16) : b;
-  }
-  *xr = make_uint2(r[0], r[1]);
-  float s = (v[0] + v[1]) + (v[2] + v[3]);
-#pragma unroll
-  for (int d = 8; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-  const float mean = s * (1.f / kSliceCols);
-  float q = 0.f;
-#pragma unroll
-  for (int e = 0; e < 4; ++e) q += (v[e] - mean) * (v[e] - mean);
-#pragma unroll
-  for (int d = 8; d > 0; d >>= 1) q += __shfl_xor_sync(0xffffffffu, q, d);
-  if ((lane & 15) == 0)
-    sm[static_cast<size_t>(lane >> 4) * t_cap + lo] = make_float2(mean, q);
 }
 
 // ---------------------------------------------------------------------------
@@ -448,7 +402,7 @@ Prep prep_layout(const dora_actor_weights* w) {
 }
 
 struct Ws {
-  size_t status, x, sm, qkv, o, z, s1, prep, total;
+  size_t status, x, qkv, o, z, s1, prep, total;
 };
 
 Ws ws_layout(int32_t t_cap, int32_t batch, const dora_actor_weights* w) {
@@ -457,16 +411,14 @@ Ws ws_layout(int32_t t_cap, int32_t batch, const dora_actor_weights* w) {
   size_t off = 0;
   L.status = off; off += 256;
   L.x = off;      off += up256(t * W * 2);
-  L.sm = off;     off += up256(t * 2 * 8);
   L.qkv = off;    off += up256(t * 3 * W * 2);
   L.o = off;      off += up256(t * W * 2);
   L.z = off;      off += up256(t * W * 2);
   L.s1 = off;     off += up256(t * SH * 2);
-  // the size stays what it was when heads were padded to 64 and Z1, its slice
-  // moments, the feed-forward's hidden rows and the gate's logits were kept:
-  // callers that sized the workspace by that are not refused, nor is its size a
-  // surprise to them
-  off += up256(b * 4) + up256(t * (3 * W * 2 + W * 2 + W * 2 + 8 + FF * 2));
+  // the size stays what it was when heads were padded to 64 and Z1, moments, the
+  // feed-forward's hidden rows and the gate's logits were kept: callers that sized
+  // the workspace by that are not refused, nor is its size a surprise to them
+  off += up256(b * 4) + up256(t * (3 * W * 2 + W * 2 + W * 2 + 3 * 8 + FF * 2));
   L.prep = off;   off += w->prepared != nullptr ? 0 : prep_layout(w).total;
   L.total = off;
   return L;
@@ -573,7 +525,6 @@ int dora_actor(const dora_bf16* qkv, const int32_t* cu, int32_t batch, int32_t m
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   int32_t* status = reinterpret_cast<int32_t*>(ws + L.status);
   uint16_t* x = reinterpret_cast<uint16_t*>(ws + L.x);
-  float* sm = reinterpret_cast<float*>(ws + L.sm);
   uint16_t* qkv_e = reinterpret_cast<uint16_t*>(ws + L.qkv);
   uint16_t* o_e = reinterpret_cast<uint16_t*>(ws + L.o);
   uint16_t* z = z_out != nullptr ? z_out : reinterpret_cast<uint16_t*>(ws + L.z);
@@ -584,26 +535,25 @@ int dora_actor(const dora_bf16* qkv, const int32_t* cu, int32_t batch, int32_t m
   const int32_t* rows = cu + batch;
   const int d = w->dim;
 
-  // X = W_in K + (b_in + e^C_l), K read in place from the block's qkv rows, and
-  // the slice moments of its rows; then the history term on every CLS row
-  LinearEpi e_in;
-  e_in.bias = reinterpret_cast<const uint16_t*>(prep + P.bias_in) + static_cast<size_t>(block) * W;
-  e_in.stats_out = sm;
-  if (launch_linear(qkv + d, t_cap, rows, d, w->enc_w_in, W, kEpiStats, e_in, x, status, stream,
-                    3 * d) != cudaSuccess ||
-      launch_pdl(history_kernel, dim3((batch + 3) / 4), dim3(128), 0, stream, cu, batch, t_cap,
-                 w->depth, w->n0, rho, interventions, w->enc_w_h, x,
-                 reinterpret_cast<float2*>(sm)) != cudaSuccess)
-    return DORA_ERR_CUDA;
-  // Attention(LayerNorm1(X)); the 384-column linear merges the two slices itself
-  LinearEpi e_q;
-  e_q.stats_in = sm;
-  e_q.slices_in = W / kSliceCols;
-  e_q.colsum = reinterpret_cast<const float*>(prep + P.cqkv);
-  e_q.colbias = reinterpret_cast<const float*>(prep + P.dqkv);
-  e_q.eps = w->eps;
-  if (launch_linear(x, t_cap, rows, W, reinterpret_cast<const uint16_t*>(prep + P.wqkv), 3 * W,
-                    kEpiLn, e_q, qkv_e, status, stream) != cudaSuccess ||
+  // X = W_in K + (b_in + e^C_l), K read in place from the block's qkv rows, with the
+  // history term on every CLS row, and the attention's LayerNorm and QKV linear
+  FrontArgs fa;
+  fa.cu = cu;
+  fa.batch = batch;
+  fa.n0 = w->n0;
+  fa.depth = w->depth;
+  fa.rho = rho;
+  fa.interventions = interventions;
+  fa.w_h = w->enc_w_h;
+  fa.bias = reinterpret_cast<const uint16_t*>(prep + P.bias_in) + static_cast<size_t>(block) * W;
+  fa.c = reinterpret_cast<const float*>(prep + P.cqkv);
+  fa.d = reinterpret_cast<const float*>(prep + P.dqkv);
+  fa.eps = w->eps;
+  fa.x = x;
+  fa.qkv = qkv_e;
+  if (launch_actor_front(qkv + d, 3 * d, d, w->enc_w_in,
+                         reinterpret_cast<const uint16_t*>(prep + P.wqkv), fa, t_cap, status,
+                         stream) != cudaSuccess ||
       launch_varlen_attn(qkv_e, cu, batch, max_seqlen, t_cap, HEADS, 0.17677669529663688f, o_e,
                          status, stream, HD) != cudaSuccess)
     return DORA_ERR_CUDA;

@@ -91,12 +91,12 @@ struct Cfg {
   static constexpr bool kResTma =
       EPI == DORA_EPI_BIAS_RESIDUAL || EPI == kEpiResidualLongK || EPI == kEpiTokens;
   // slice moments of the output rows, where the caller takes them
-  static constexpr bool kMoments = (kResTma && EPI != kEpiTokens) || EPI == kEpiStats;
+  static constexpr bool kMoments = kResTma && EPI != kEpiTokens;
   // the two GELU epilogues are ALU-bound: 16 warps; the others 8.  A 64-wide
-  // tile has 32 columns for each of 8 warps; those that write moments need
-  // whole 64-column slices: 4
+  // tile has 32 columns for each of 8 warps; the residual's need whole
+  // 64-column slices: 4
   static constexpr int kEpiWarps =
-      BN == 64 ? (kResTma || EPI == kEpiStats ? 4 : 8)
+      BN == 64 ? (kResTma ? 4 : 8)
                : ((EPI == DORA_EPI_BIAS_GELU || EPI == kEpiLnGelu) ? 16 : 8);
   static constexpr int kColGroups = kEpiWarps / 4;
   static constexpr int kCols = BN / kColGroups;         // columns per epilogue warp
@@ -457,17 +457,13 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
     };
     // Folded LayerNorm: (mean, var) of this lane's row, loaded a tile ahead
     // (a warp's 32 rows are one 256-byte load).
-    float2 mv = make_float2(0.f, 0.f), mv2 = mv;
+    float2 mv = make_float2(0.f, 0.f);
     auto load_mv = [&](int w) {
       const int row_p = (2 * mpair(item(w).pair) + rank) * BM + q * 32 + lane;
       if (row_p >= M) return;
       const float2* p = reinterpret_cast<const float2*>(ep.stats_in) + row_p;
-      if (BN < 256 && ep.slices_in > 0 && ep.slices_in != 2) {
-        mv = merge_slice_moments(p, m_cap, ep.slices_in);
-        return;
-      }
-      mv = __ldg(p);
-      if (BN < 256 && ep.slices_in == 2) mv2 = __ldg(p + m_cap);    // merged when used
+      if (BN < 256 && ep.slices_in > 0) mv = merge_slice_moments(p, m_cap, ep.slices_in);
+      else mv = __ldg(p);
     };
     if constexpr (C::kLn)
       if (cid < items) {
@@ -491,7 +487,6 @@ __global__ void __launch_bounds__(Cfg<BN, EPI, PAIR>::kThreads, 1)
       const bool past_image = EPI == kEpiTokens && row0 % ep.tokens + lane >= ep.tokens;
       float neg_mean = 0.f, rstd = 0.f;           // folded LayerNorm of this row
       if constexpr (C::kLn) {
-        if (BN < 256 && ep.slices_in == 2) mv = merge_two_slices(mv, mv2);
         neg_mean = -mv.x;
         rstd = rsqrtf(mv.y + ep.eps);
         if (w + n_clusters < items) load_mv(w + n_clusters);
@@ -724,9 +719,6 @@ static cudaError_t launch_bn(const CUtensorMap& ta, const CUtensorMap& tb,
       return launch(launch_bn_epi<BN, kEpiResidualLongK, kPair>);
     case kEpiTokens:
       return launch(launch_bn_epi<BN, kEpiTokens, kPair>);
-    case kEpiStats:                             // the actor's width: never 256 wide
-      if constexpr (BN < 256) return launch(launch_bn_epi<BN, kEpiStats, kPair>);
-      return cudaErrorInvalidValue;
     case kEpiLn:
       return launch(launch_bn_epi<BN, kEpiLn, kPair>);
     case kEpiLnGelu:

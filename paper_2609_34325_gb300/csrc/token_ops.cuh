@@ -103,12 +103,9 @@ cudaError_t launch_gather_scores(const float* table, int32_t stride, const int32
 // with rstd_r = 1/sqrt(var_r + eps) from the row moments (stats_in);
 // and the patch embedding's, row r being token j = r mod tokens of its image:
 //   kEpiTokens  y = x w^T + bias + pos[j], for j = 0 (CLS) y = cls + pos[0]
-// and, for n that is no multiple of 256,
-//   kEpiStats   y = x w^T + bias, with the slice moments of y's rows
 constexpr int kEpiLn = 3;
 constexpr int kEpiLnGelu = 4;
 constexpr int kEpiTokens = 6;
-constexpr int kEpiStats = 7;
 struct LinearEpi {
   const uint16_t* bias = nullptr;       // bf16 [n], nullable (plain epilogues)
   const uint16_t* residual = nullptr;   // bf16 [m, n] (residual epilogue)
@@ -119,8 +116,7 @@ struct LinearEpi {
   float* stats_out = nullptr;           // slice moments of y, [n/64][m_cap], nullable
   float eps = 0.f;                      // LayerNorm epsilon (LN epilogues)
   int32_t slices_in = 0;                // > 0: k / 64, stats_in is [k/64][m_cap][2]
-                                        // (where linear_merges says so, or n is no
-                                        // multiple of 256)
+                                        // (only where linear_merges says so)
   const uint16_t* cls = nullptr;        // bf16 [n] (kEpiTokens)
   const uint16_t* pos = nullptr;        // bf16 [tokens, n] (kEpiTokens)
   int32_t tokens = 0;                   // rows per image (kEpiTokens)
@@ -133,6 +129,26 @@ bool linear_merges(int32_t m_cap, int32_t n);
 cudaError_t launch_linear(const uint16_t* x, int32_t m_cap, const int32_t* m_dev, int32_t k,
                           const uint16_t* w, int32_t n, int32_t epilogue, const LinearEpi& ep,
                           uint16_t* y, int32_t* status, cudaStream_t stream, int32_t lda = 0);
+
+// The actor's encoder before its attention in one kernel: keys [m, dim] (row pitch
+// in elements), W_in [128, dim], W_qkv' [384, 128] (LayerNorm folded in); the live
+// rows are cu[batch].
+struct FrontArgs {
+  const int32_t* cu;        // [batch + 1]
+  int32_t batch;
+  int32_t n0, depth;        // of the history term
+  const float* rho;         // [batch]
+  const int32_t* interventions;
+  const uint16_t* w_h;      // bf16 [128, 3]
+  const uint16_t* bias;     // bf16 [128], b_in + e^C of the block
+  const float *c, *d;       // fp32 [384], of the folded W_qkv
+  float eps;
+  uint16_t* x;              // bf16 [m, 128]
+  uint16_t* qkv;            // bf16 [m, 384]
+};
+cudaError_t launch_actor_front(const uint16_t* keys, int32_t pitch, int32_t dim,
+                               const uint16_t* w_in, const uint16_t* w_qkv, const FrontArgs& args,
+                               int32_t m_cap, int32_t* status, cudaStream_t stream);
 
 // The actor's encoder after its attention, and the selector's first layer, in
 // one kernel: o [m, 128], W_o [128, 128], W_1' [256, 128] (LayerNorm folded in),
