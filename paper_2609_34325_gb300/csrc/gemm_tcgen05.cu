@@ -92,12 +92,18 @@ struct Cfg {
       EPI == DORA_EPI_BIAS_RESIDUAL || EPI == kEpiResidualLongK || EPI == kEpiTokens;
   // slice moments of the output rows, where the caller takes them
   static constexpr bool kMoments = kResTma && EPI != kEpiTokens;
-  // the two GELU epilogues are ALU-bound: 16 warps; the others 8.  A 64-wide
+  // the two GELU epilogues are ALU-bound: 16 warps; so is the patch embedding's
+  // on 256 columns, with its short K (128 images of 16 x 16 patches, the call: 55.0
+  // -> 51.8 us); the others 8 (the residual's spills with 16: 61.5 -> 67.6 us at
+  // 50432 x 768 x 768, and the plain LayerNorm's runs 108.5 -> 113.0).  A 64-wide
   // tile has 32 columns for each of 8 warps; the residual's need whole
   // 64-column slices: 4
   static constexpr int kEpiWarps =
       BN == 64 ? (kResTma ? 4 : 8)
-               : ((EPI == DORA_EPI_BIAS_GELU || EPI == kEpiLnGelu) ? 16 : 8);
+               : ((EPI == DORA_EPI_BIAS_GELU || EPI == kEpiLnGelu ||
+                   (EPI == kEpiTokens && BN == 256))
+                      ? 16
+                      : 8);
   static constexpr int kColGroups = kEpiWarps / 4;
   static constexpr int kCols = BN / kColGroups;         // columns per epilogue warp
   static constexpr int kChunks = kCols / 32;
