@@ -1546,6 +1546,26 @@ def test_patch_embed_epilogue_where_a_chunk_spans_images(gw):
     assert_close(f64(x0), ref, f"patch embed, {gw} patches")
 
 
+@pytest.mark.parametrize("b", [60, 100, 175])
+def test_patch_embed_epilogue_at_every_tile_width(b):
+    """768 columns over 2,220, 3,700 and 6,475 rows (with 152 SMs): one wave of
+    128-wide tiles, one of 256-wide ones, and 78 of these, the last two in halves;
+    images of 37 tokens, so most 32-row chunks span two."""
+    gw, patch, d = 36, 8, 768
+    rng = np.random.default_rng(b)
+    im = S.f32_to_bf16_bits(rng.standard_normal((b, 1, patch, gw * patch)))
+    wpe = S.f32_to_bf16_bits(rng.standard_normal((d, patch * patch)) / patch)
+    bpe, cls = (S.f32_to_bf16_bits(rng.standard_normal(d)) for _ in range(2))
+    pos = S.f32_to_bf16_bits(rng.standard_normal((gw + 1, d)))
+    x0 = torch.full((b * (gw + 1), d), 9.0, dtype=torch.bfloat16, device=dev())
+    ws = P.dora_patch_embed(bf(im), bf(wpe), bf(bpe), bf(cls), bf(pos), patch, x0)
+    torch.cuda.synchronize()
+    assert P.dora_read_status(P.dora_workspace_status(ws)) == 0
+    ref = O.patch_embed(im, O.bf16_to_f64(wpe), O.bf16_to_f64(bpe), O.bf16_to_f64(cls),
+                        O.bf16_to_f64(pos), patch)
+    assert_close(f64(x0), ref, f"patch embed of {b} images")
+
+
 @pytest.mark.parametrize("name", ["cfg1", "cfg3"])
 def test_classifier_head_matches_oracle(name):
     cfg = S.get_config(name)
