@@ -54,7 +54,12 @@ struct Smem {
   float c[NQ], d[NQ];                   // folded LayerNorm of W_qkv
   float wh[3][W];                       // W_h, transposed
   float bias[W];
-  float2 half_moments[2][BM];           // slice moments of X's two halves
+  // Slice moments of X's two halves, by tile parity.  A half reads the other's of
+  // tile n after x_ready(n), and nothing orders the next tile's X (x_full(n + 1),
+  // behind q_full[2](n) alone) after that read; x_full(n + 2) is behind
+  // x_ready(n + 1), at which every warp arrives after its reads of tile n.  So one
+  // buffer would let a late warp take the next tile's moments, two do not.
+  float2 half_moments[2][2][BM];
   uint64_t full[kStages];
   uint64_t empty[kStages];
   uint64_t x_full;                      // first product of the tile done
@@ -253,7 +258,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       const float2 mine = slice_moments(*reinterpret_cast<const uint32_t(*)[16]>(&x[0]),
                                         *reinterpret_cast<const uint32_t(*)[16]>(&x[16]));
-      s.half_moments[half][r] = mine;
+      s.half_moments[n & 1][half][r] = mine;
       // X over this thread's own accumulator columns
       tmem_st16(lanes + kDX + c0, *reinterpret_cast<const uint32_t(*)[16]>(&x[0]));
       tmem_st16(lanes + kDX + c0 + 16, *reinterpret_cast<const uint32_t(*)[16]>(&x[16]));
@@ -261,7 +266,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       warp_arrive(&s.x_ready);
       if (live) store64(a.x + static_cast<size_t>(row) * W + c0, x);
       if (!mbar_wait_warp(&s.x_ready, ph, abort)) break;
-      const float2 other = s.half_moments[half ^ 1][r];
+      const float2 other = s.half_moments[n & 1][half ^ 1][r];
       const float2 mv = merge_two_slices(half ? other : mine, half ? mine : other);
       const float neg_mean = -mv.x, rstd = rsqrtf(mv.y + a.eps);
       bool ok = true;

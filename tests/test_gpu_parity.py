@@ -1435,6 +1435,45 @@ def test_actor_at_tile_edges_and_the_ends_of_its_ranges(lens, dim, n0):
     assert torch.all(buf[:off] == 0) and torch.all(buf[off + t * 128:] == 0)
 
 
+@pytest.mark.parametrize("dim", [64, 768])
+def test_actor_with_three_tiles_a_cta(dim):
+    """More than three 128-row tiles per SM, in ragged images: the same bits on
+    every repeat, and the bits of launches of at most one tile per SM (no row
+    depends on another image's), which the oracle checks on a few images."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    lens = []
+    rng = np.random.default_rng(61)
+    while sum(lens) <= 3 * 128 * sms:
+        lens.append(int(rng.integers(20, 578)))
+    cfg = replace(S.get_config("cfg1"), dim=dim, heads=dim // 64, n_tokens=577, batch=len(lens),
+                  depth=3)
+    gen = torch.Generator(device=dev()).manual_seed(61)
+    qkv = torch.empty(sum(lens), 3 * dim, device=dev()).normal_(generator=gen).bfloat16()
+    qkv = bits(qkv)
+    _, _, _, _, wa, aw = _actor_case(cfg, 61, gate_bias=0.5, lens=np.array([5]))
+    cu = O.cu_from_counts(np.array(lens))
+    rho = rng.uniform(0, 0.5, len(lens)).astype(np.float32)
+    e_prev = rng.integers(0, 3, len(lens)).astype(np.int32)
+    first = _run_actor(cfg, cu, qkv, rho, e_prev, aw, 1, 577)
+    for _ in range(3):
+        again = _run_actor(cfg, cu, qkv, rho, e_prev, aw, 1, 577)
+        for name in first:
+            assert np.array_equal(first[name], again[name]), name
+    i = 0
+    while i < len(lens):
+        j = i + 1
+        while j < len(lens) and cu[j + 1] - cu[i] <= 128 * sms:
+            j += 1
+        part = _run_actor(cfg, cu[i:j + 1] - cu[i], qkv[cu[i]:cu[j]], rho[i:j], e_prev[i:j], aw, 1,
+                          577)
+        for name in first:
+            rows = slice(cu[i], cu[j]) if name in ("z", "scores") else slice(i, j)
+            assert np.array_equal(first[name][rows], part[name]), (name, i, j)
+        i = j
+    images = [0, len(lens) // 3, len(lens) // 2, len(lens) - 1]
+    _check_actor(cfg, cu, qkv, rho, e_prev, wa, first, 1, images)
+
+
 @pytest.mark.parametrize("given_counts", [True, False])
 def test_block_with_actor_equals_actor_then_block(given_counts):
     """dora_pruned_block_actor gives the same bits as running dora_actor on the
