@@ -463,10 +463,14 @@ __device__ __forceinline__ float warp_sum(float v) {
 // 16 bytes at a time, into registers (the maximum, the sum and the divergence
 // all come from there).  Latency-bound: 768 rows of 1000 classes 15.5 us with
 // 2-byte loads read twice and a running log-sum-exp per element -> 6.1 us.
-constexpr int kHeldChunks = 4;                       // 8 classes a lane each
-constexpr int kHeldClasses = 32 * 8 * kHeldChunks;
+// kHeldChunks pieces of 8 classes a lane, as few as hold the row: every piece
+// costs its exponentials, used or not.  4096 rows, inputs out of L2, us: 10
+// classes 14.3 with four pieces, 8.4 with one (streamed 8.2); 512 classes 15.6
+// with four, 12.2 with two (streamed 14.4); 1000 classes 16.7 (streamed 20.7).
+constexpr int kHeldClasses = 32 * 8 * 4;
 constexpr int kHeldThreads = 128;
 
+template <int kHeldChunks>
 __global__ void __launch_bounds__(kHeldThreads)
     kd_cost_held_kernel(const uint4* __restrict__ zn, const uint4* __restrict__ z,
                         const int32_t* __restrict__ map, int shadows, int batch, int classes,
@@ -690,11 +694,16 @@ int dora_kd_cost(const dora_bf16* z_native, const dora_bf16* z, const int32_t* s
   if (e != DORA_OK) return e;
   if (shadows == 0) return DORA_OK;
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
-  if (classes <= train::kHeldClasses && ld % 8 == 0 && aligned16(z_native) && aligned16(z))
-    return launched(launch_pdl(
-        train::kd_cost_held_kernel, dim3((shadows + 3) / 4), dim3(train::kHeldThreads), 0, stream,
-        reinterpret_cast<const uint4*>(z_native), reinterpret_cast<const uint4*>(z), shadow_image,
-        shadows, batch, classes, ld / 8, 1.f / tau, tau * tau, cost, status));
+  if (classes <= train::kHeldClasses && ld % 8 == 0 && aligned16(z_native) && aligned16(z)) {
+    constexpr decltype(&train::kd_cost_held_kernel<1>) kern[] = {
+        train::kd_cost_held_kernel<1>, train::kd_cost_held_kernel<2>,
+        train::kd_cost_held_kernel<3>, train::kd_cost_held_kernel<4>};
+    return launched(launch_pdl(kern[(classes - 1) / 256], dim3((shadows + 3) / 4),
+                               dim3(train::kHeldThreads), 0, stream,
+                               reinterpret_cast<const uint4*>(z_native),
+                               reinterpret_cast<const uint4*>(z), shadow_image, shadows, batch,
+                               classes, ld / 8, 1.f / tau, tau * tau, cost, status));
+  }
   return launched(launch_pdl(train::kd_cost_kernel, dim3((shadows * 32 + 255) / 256), dim3(256), 0,
                              stream, z_native, z, shadow_image, shadows, batch, classes, ld,
                              1.f / tau, tau * tau, cost, status));

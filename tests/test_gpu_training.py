@@ -470,11 +470,13 @@ def test_branch_on_both_sides_of_the_one_launch_limit(nb):
 
 
 @pytest.mark.parametrize("classes,ld", [(1, 8), (7, 8), (8, 8), (257, 264), (1000, 1024),
-                                        (1023, 1024), (1024, 1024), (1025, 1032), (1000, 1004)])
+                                        (1023, 1024), (1024, 1024), (1025, 1032), (1000, 1004),
+                                        (256, 256), (512, 512), (513, 520), (768, 768),
+                                        (769, 776)])
 def test_kd_cost_held_and_streamed_rows(classes, ld):
-    """Rows held in registers (up to 1024 classes, 16-byte rows) and streamed
-    (more classes, or a row pitch that is no multiple of eight), the padding
-    ignored in both."""
+    """Rows held in registers (up to 1024 classes, 16-byte rows, one piece a lane
+    for every 256) and streamed (more classes, or a row pitch that is no multiple
+    of eight), the padding ignored in both."""
     rng = np.random.default_rng(17)
     zn, z = (rng.standard_normal((n, ld)).astype(np.float32) * 3 for n in (3, 6))
     z[:, classes:] = 60.0
