@@ -439,7 +439,7 @@ def test_branch_scan_across_chunks_and_overflow():
 @pytest.mark.parametrize("nb", [1, 3, 255, 257, 4096, 4097])
 def test_branch_on_both_sides_of_the_one_launch_limit(nb):
     """Up to 4096 appended sequences in one launch (every CTA summing the
-    lengths before its sequence, its rows in up to 16 parts), more by the
+    lengths before its sequence, its rows in several parts), more by the
     scan; row counts on both sides of the copy's 1024-piece strides; bad and
     empty sources among them."""
     rng = np.random.default_rng(16)
@@ -467,6 +467,22 @@ def test_branch_on_both_sides_of_the_one_launch_limit(nb):
     rows = np.concatenate([np.arange(cu[s], cu[s + 1]) for s in src if s < 64]).astype(np.int64)
     assert np.array_equal(bits(xt)[int(cu[-1]):int(want[-1])], x[rows])
     assert np.array_equal(it.cpu().numpy()[int(cu[-1]):int(want[-1])], ids[rows])
+
+
+@pytest.mark.parametrize("n,d,room", [(1, 8, 0), (1, 8, 100000), (173, 192, 1), (3000, 768, 0)])
+def test_branch_of_one_sequence_in_many_parts(n, d, room):
+    """One sequence split over up to 912 CTAs: fewer pieces than parts, parts
+    that are no whole stride, and a long one; nothing written past its rows."""
+    rng = np.random.default_rng(18)
+    t_cap = 2 * n + room
+    x = S.f32_to_bf16_bits(rng.standard_normal((t_cap, d)))
+    xt, cu_out = bf(x), torch.zeros(3, dtype=torch.int32, device=dev())
+    P.dora_branch(xt, i32([0, n]), i32([0]), cu_out)
+    torch.cuda.synchronize()
+    assert cu_out.cpu().tolist() == [0, n, 2 * n]
+    got = bits(xt)
+    assert np.array_equal(got[n:2 * n], x[:n])
+    assert np.array_equal(got[:n], x[:n]) and np.array_equal(got[2 * n:], x[2 * n:])
 
 
 @pytest.mark.parametrize("classes,ld", [(1, 8), (7, 8), (8, 8), (257, 264), (1000, 1024),
