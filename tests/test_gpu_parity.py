@@ -1710,3 +1710,43 @@ def test_classifier_head_lc1_matches_oracle(name, dim):
     assert_close(f64(logits), ref, f"lc1 head {name}")
     assert torch.all(logits[:, 1000:] == 0)
 
+
+def _lc1_features(x, cu):
+    """The LC1 features themselves: an identity head on them, unit affine."""
+    d, b = x.shape[1], cu.numel() - 1
+    one, zero = (torch.full((d,), v, dtype=torch.bfloat16, device=dev()) for v in (1.0, 0.0))
+    eye = torch.eye(2 * d, dtype=torch.bfloat16, device=dev())
+    out = torch.empty(b, 2 * d, dtype=torch.bfloat16, device=dev())
+    P.dora_classifier_head_lc1(x, cu, one, zero, 1e-6, eye, torch.zeros_like(eye[0]), out)
+    torch.cuda.synchronize()
+    return out
+
+
+def test_lc1_features_round_as_with_an_exact_division():
+    """Of 1.2 million mean features (dim 384) 1.06e-4 round to another bf16 value
+    than in 64 bits when mean and variance are divided by dim, 1.7e-4 when they
+    are multiplied by fp32 1/384; the bound lies more than 2.5 standard
+    deviations of the count from both."""
+    d, wrong, total = 384, 0, 0
+    for seed in range(12):
+        gen = torch.Generator(device=dev()).manual_seed(seed)
+        lens = np.random.default_rng(seed).integers(9, 120, 256)
+        cu = O.cu_from_counts(lens)
+        x = torch.empty(int(cu[-1]), d, device=dev()).normal_(generator=gen)
+        x *= torch.empty(1, d, device=dev()).uniform_(0.5, 1.5, generator=gen)
+        x = (x + 0.2).bfloat16()
+        got = _lc1_features(x, i32(cu))[:, d:]
+        v = x.double()
+        v = (v - v.mean(1, keepdim=True)) / (v.var(1, unbiased=False, keepdim=True) + 1e-6).sqrt()
+        ref = torch.stack([v[a + 1:b].mean(0) for a, b in zip(cu[:-1], cu[1:])]).bfloat16()
+        wrong += int((got != ref).sum())
+        total += ref.numel()
+    assert wrong <= 1.35e-4 * total, (wrong, total)
+
+
+@pytest.mark.parametrize("d", [384, 1024])
+def test_lc1_of_a_row_whose_variance_overflows(d):
+    """A sum of squares past fp32 gives a row of zeros, not NaN."""
+    x = torch.full((3, d), 2.0 ** 70, dtype=torch.bfloat16, device=dev())
+    x[:, ::2] *= -1
+    assert torch.all(_lc1_features(x, i32([0, 3])) == 0)
