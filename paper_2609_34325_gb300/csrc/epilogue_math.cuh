@@ -9,25 +9,29 @@
 namespace dora {
 
 // GELU(x) = x * Phi(x) = max(x, 0) - |x| Q(|x|), Q(a) = 1 - Phi(a): no select on
-// the sign.  Q = 2^p with p a polynomial of degree 7 for log2 Q, which is smooth:
-// fitted on 6000 points of [0, 9] by linear programming to the least largest
-// error of |x| Q (in log2 Q 4e-5 of that weight at least, so that the tail keeps
-// its relative accuracy); past 9, where Q < 2e-19, p only falls.  In fp32, against
-// 64 bits over [-14, 14]: |error| <= 2.7e-7, 5.3e-8 rms, relative 4.5e-4 down to
-// x = -6 and 1.7e-3 to -9; erf by formula 7.1.26 of Abramowitz & Stegun, with its
-// reciprocal and exponential, had 3.3e-7, 7.0e-8, 3.6e-3 and 1.5e-2.
+// the sign.  Q = 2^p with p a polynomial of degree 8 for log2 Q, which is smooth,
+// and p(0) = -1 exactly, so that the relative error does not grow towards zero.
+// Fitted on 5700 points of [0, 7.2] by linear programming to the least largest
+// ratio to bounds a little below the errors of erf by formula 7.1.26 of Abramowitz &
+// Stegun (with its reciprocal and exponential).  In fp32 against 64 bits, in brackets
+// that formula: |error| <= 2.7e-7 (3.3e-7); relative 3.7e-7 (6.5e-7) for |x| < 0.1,
+// 4.7e-7 (7.9e-7) for |x| < 1, 3.7e-6 (4.0e-6) down to x = -2.5, 3.0e-3 (3.6e-3) to
+// -6; not above it in the largest or the rms error of any range down to -7.  Below
+// -7, where |GELU| < 1e-11, p falls too fast: the error stays below 6e-16, but is
+// 0.1 of GELU (0.01) at -8 and 0.5 (0.015) at -9.
 // Evaluated on two values at once with the paired fp32 instructions
-// (fma.rn.f32x2), in -|x|: the epilogue's ALU work is what limits this GEMM, and
-// one exponential a value on the special-function unit instead of two operations
-// there took fc1 at 50432 x 3072 x 768 from 165.9 to 157.7 us (a DeiT-B block on 256
-// images 601 -> 595, the actor's call 108.7 -> 106.9).
+// (fma.rn.f32x2), in -|x|: the epilogue's ALU work is what limits this GEMM, about
+// 2 us for each degree.  fc1 at 50432 x 3072 x 768, us: 162.1, with the formula
+// 168.5; degree 7 with p(0) fitted too 160 (relative 8.3e-6 near zero), degree 10
+// on [0, 11], nowhere further off than the formula, 166.3.
 __device__ __forceinline__ void gelu_erf2(float& x0, float& x1) {
-  constexpr float kP[8] = {-0.999988198f,  1.15125728f,     -0.458570153f,   0.0537337177f,
-                           0.0083378423f,  0.000873989775f, 5.33180246e-05f, 1.39957956e-06f};
+  constexpr float kP[9] = {-1.0f,            1.15111219f,      -0.45913319f,
+                           0.0527509033f,    0.00745460154f,   0.000444294797f,
+                           -5.89050899e-05f, -1.312108e-05f,   -7.22790292e-07f};
   const uint64_t NX = f2_pack(-fabsf(x0), -fabsf(x1));
-  uint64_t p = f2_pack(kP[7], kP[7]);
+  uint64_t p = f2_pack(kP[8], kP[8]);
 #pragma unroll
-  for (int k = 6; k >= 0; --k) p = f2_fma(p, NX, f2_pack(kP[k], kP[k]));
+  for (int k = 7; k >= 0; --k) p = f2_fma(p, NX, f2_pack(kP[k], kP[k]));
   float p0, p1;
   f2_unpack(p, p0, p1);
   f2_unpack(f2_fma(NX, f2_pack(ex2_approx(p0), ex2_approx(p1)),

@@ -468,6 +468,45 @@ def test_linear_gelu_epilogue_within_one_bf16_ulp():
     assert np.all(err <= 2.0 ** -7 * np.abs(ref) + 1e-6), float(err.max())
 
 
+def test_linear_gelu_epilogue_rounds_right_near_zero():
+    """GELU of fp32 values (three bf16 pieces, summed exactly by the product)
+    chosen so that GELU lies 1.5e-6 of itself beside the midpoint of two bf16
+    values: an evaluation within 1.3e-6 relative (the input's own rounding to
+    fp32 moves it by at most 1.2e-7) takes the nearer one, for |x| from 2^-14 to
+    1.  Erf by Abramowitz & Stegun 7.1.26 in fp32 has 7.9e-7 there at most."""
+    rng = np.random.default_rng(32)
+    m = 4096
+    x = np.exp(rng.uniform(np.log(2.0 ** -14), 0.0, m)) * rng.choice([-1.0, 1.0], m)
+    # the midpoint above the bf16 value below GELU(x) in magnitude, moved aside
+    low = np.abs(O.gelu(x)).astype(np.float32).view(np.uint32) & np.uint32(0xFFFF0000)
+    mid = (low | np.uint32(0x8000)).view(np.float32).astype(np.float64) * np.sign(x)
+    keep = ~((x < 0) & (np.abs(mid) > 0.15))              # GELU has its minimum at -0.75
+    x, mid = x[keep], mid[keep]
+    side = rng.choice([-1.0, 1.0], x.size)
+    goal = mid * (1 + 1.5e-6 * side)
+    lo = np.where(x < 0, -0.65, 0.0)                      # GELU rises from there to 1
+    hi = np.where(x < 0, 0.0, 1.2)
+    for _ in range(100):
+        c = 0.5 * (lo + hi)
+        under = O.gelu(c) < goal
+        # on [-0.65, 0] GELU rises as well: its minimum lies below
+        lo, hi = np.where(under, c, lo), np.where(under, hi, c)
+    v = (0.5 * (lo + hi)).astype(np.float32)
+    h = (v.view(np.uint32) & np.uint32(0xFFFF0000)).view(np.float32)
+    mi = ((v - h).view(np.uint32) & np.uint32(0xFFFF0000)).view(np.float32)
+    pieces = np.zeros((v.size, 64))
+    pieces[:, :3] = np.stack([h, mi, v - h - mi], 1)
+    w = np.zeros((32, 64))
+    w[:, :3] = 1.0
+    y = torch.zeros(v.size, 32, dtype=torch.bfloat16, device=dev())
+    P.dora_linear(bf(S.f32_to_bf16_bits(pieces)), bf(S.f32_to_bf16_bits(w)), y,
+                  epilogue=P.EPI_BIAS_GELU)
+    torch.cuda.synchronize()
+    ref = O.bf16_to_f64(S.f32_to_bf16_bits(O.gelu(v.astype(np.float64))))
+    wrong = f64(y)[:, 0] != ref
+    assert not wrong.any(), (int(wrong.sum()), np.abs(v[wrong]).min(), np.abs(v[wrong]).max())
+
+
 def test_linear_no_bias_full_rows():
     rng = np.random.default_rng(9)
     x = S.f32_to_bf16_bits(rng.standard_normal((512, 256)))
