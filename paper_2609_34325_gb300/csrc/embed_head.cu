@@ -107,16 +107,19 @@ __global__ void patchify_any_kernel(const uint16_t* __restrict__ img, int batch,
 // the K-padded patch matrix, consecutive threads consecutive pairs of a
 // token row, so every store is coalesced; the pair (an even pair never
 // straddles two patches) is read from the image, pad pairs and CLS rows are
-// zero.  All counts fit in 32 bits (checked by the caller).
+// zero.  All counts fit in 31 bits (checked by the caller).
 __global__ void patchify_even_kernel(const uint32_t* __restrict__ img, int batch, int ch, int h,
                                      int w, int p, int kpad, uint32_t* __restrict__ out) {
   pdl_trigger();
   pdl_wait();
   const int gw = w / p, gh = h / p, p2 = p / 2, row2 = p * p2, k2 = ch * row2, w2 = w / 2;
   const int kp2 = kpad / 2, g = gw * gh;
-  const int total = batch * (g + 1) * kp2;
-  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < total; s += gridDim.x * blockDim.x) {
-    const int q = s % kp2, r = s / kp2, b = r / (g + 1), tok = r - b * (g + 1) - 1;
+  // unsigned: the last stride may step past 2^31
+  const uint32_t total = static_cast<uint32_t>(batch) * (g + 1) * kp2;
+  for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < total;
+       s += gridDim.x * blockDim.x) {
+    const int r = s / kp2, q = s - static_cast<uint32_t>(r) * kp2, b = r / (g + 1);
+    const int tok = r - b * (g + 1) - 1;
     uint32_t v = 0u;
     if (tok >= 0 && q < k2) {
       const int c = q / row2, rem = q - c * row2, dy = rem / p2, e = rem - dy * p2;

@@ -1644,6 +1644,33 @@ def test_patch_embed_epilogue_at_every_tile_width(b):
     assert_close(f64(x0), ref, f"patch embed of {b} images")
 
 
+def test_patch_embed_whose_pixel_pairs_nearly_fill_31_bits():
+    """65,535 images of 1 x 1023 patches of two by two pixels: 2,147,450,880 pairs
+    of the padded patch matrix, so that the relayout's last stride passes 2^31."""
+    b, gw, d = 65535, 1023, 64
+    if torch.cuda.mem_get_info()[0] < 40 << 30:
+        pytest.skip("needs 40 GB of device memory")
+    gen = torch.Generator(device=dev()).manual_seed(33)
+
+    def draw(*shape):
+        return torch.empty(shape, device=dev()).normal_(generator=gen).bfloat16()
+
+    im, wpe, bpe, cls, pos = draw(b, 1, 2, 2 * gw), draw(d, 4), draw(d), draw(d), draw(gw + 1, d)
+    x0 = torch.full((b * (gw + 1), d), 9.0, dtype=torch.bfloat16, device=dev())
+    ws = P.dora_patch_embed(im, wpe, bpe, cls, pos, 2, x0)
+    torch.cuda.synchronize()
+    assert P.dora_read_status(P.dora_workspace_status(ws)) == 0
+    del ws
+    x0 = x0.view(b, gw + 1, d)
+    for i in range(0, b, 4096):
+        # [images, patches, 4 pixels], pixel (dy, dx) at 2 dy + dx
+        px = im[i:i + 4096].view(-1, 2, gw, 2).transpose(1, 2).reshape(-1, gw, 4).float()
+        ref = sum(px[..., k, None] * wpe[:, k].float() for k in range(4)) + bpe.float()
+        err = (x0[i:i + 4096, 1:].float() - (ref + pos[1:].float())).abs()
+        assert float((err - 1e-2 * (ref + pos[1:].float()).abs()).max()) <= 2e-2, i
+    assert torch.equal(x0[:, 0], (cls.float() + pos[0].float()).bfloat16().expand(b, d))
+
+
 @pytest.mark.parametrize("name", ["cfg1", "cfg3"])
 def test_classifier_head_matches_oracle(name):
     cfg = S.get_config(name)
