@@ -800,9 +800,10 @@ static cudaError_t launch(const uint16_t* qkv, const int32_t* cu, int32_t batch,
       cudaFuncSetAttribute(varlen_attn_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  const long long units =
-      static_cast<long long>(batch) * ((heads + 1) / 2) * ((max_seqlen + BQ - 1) / BQ);
-  if (units > 0x7fffffffLL) return cudaErrorInvalidValue;
+  // Any bound is accepted; a length past t_cap is flagged as one past the buffer.
+  if (max_seqlen > t_cap) max_seqlen = t_cap;
+  const long long units = static_cast<long long>(batch) * ((heads + 1) / 2) *
+                          ((static_cast<long long>(max_seqlen) + BQ - 1) / BQ);
   const long long cap = num_sms();
   const int grid = static_cast<int>(units < cap ? units : cap);
   return launch_pdl(varlen_attn_kernel<HD>, dim3(grid), dim3(kThreads), smem, stream, mp, cu,

@@ -947,6 +947,21 @@ def test_attention_where_every_unit_has_its_own_cta(extra):
     _check_attn(lens, 2, 28)
 
 
+@pytest.mark.parametrize("bound", [1 << 20, 1 << 30, 2 ** 31 - 1])
+@pytest.mark.parametrize("batch", [3, 64])
+def test_attention_with_a_bound_far_above_the_images(bound, batch):
+    """A caller may pass any max_seqlen that bounds its images: the bits are those
+    of the tight bound."""
+    lens = np.resize(np.array([130, 1, 0, 257]), batch)
+    cu, heads = O.cu_from_counts(lens), 12
+    qkv = S.f32_to_bf16_bits(np.random.default_rng(34).standard_normal(
+        (int(cu[-1]), 3 * heads * 64)))
+    tight, st0 = _run_attn(qkv, cu, heads, 257)
+    loose, st1 = _run_attn(qkv, cu, heads, bound)
+    assert st0 == st1 == 0
+    assert torch.equal(tight, loose)
+
+
 def test_attention_first_chunk_of_minus_infinities():
     """Logits of -inf (an infinite key component) in the whole first key
     chunk weigh nothing; the later chunk's keys get the weight."""
