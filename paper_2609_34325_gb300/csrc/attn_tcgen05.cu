@@ -31,6 +31,11 @@
 //                of a chunk's last 16-key group that lie past the image.
 //   warps 12-15  epilogue of both groups: when a unit's last PV is done, O / row
 //                sum, each thread storing its row's 128 bytes.
+// A last head without a partner (odd head counts) is a unit of its own whose second
+// group loads, multiplies and stores nothing of use; its softmax is skipped, so that
+// the first one's exponentials have the MUFU alone: 256 x 197 tokens x 1 head 18.6 ->
+// 16.6 us, 64 x 577 x 1 28.4 -> 24.1, 87 x 577 x 3 51.3 -> 49.5 (one head a unit, in
+// the kernel before: 15.0, 27.0, 48.6).  Skipping its MMAs too gave no more.
 // TMEM (256 columns a group): S/P buffers at 0 and 96, O at 192.  Rows past the
 // image are computed but never stored; keys past it are masked, and V rows past
 // it are zeroed so stale data cannot leak through 0 * NaN.
@@ -87,6 +92,7 @@ constexpr uint32_t kDStage = 0x7u;        // K/V stage
 constexpr uint32_t kDKvPar = 1u << 3;     // phase parity of that stage's load
 constexpr uint32_t kDFirst = 1u << 4;     // first key chunk of a unit
 constexpr uint32_t kDLast = 1u << 5;      // last key chunk of a unit
+constexpr uint32_t kDLone = 1u << 6;      // the unit's second head does not exist
 constexpr uint32_t kDEnd = 1u << 31;      // no more steps
 __device__ __forceinline__ int d_kc(uint32_t d) { return static_cast<int>((d >> 8) & 0x7Fu); }
 __device__ __forceinline__ int d_blocks(uint32_t d) { return (d_kc(d) + 31) >> 5; }
@@ -503,7 +509,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             s.kv_issued = ++loads;
             ok = desc(static_cast<uint32_t>(stg) | (par ? kDKvPar : 0u) | (c == 0 ? kDFirst : 0u) |
-                      (c == nch - 1 ? kDLast : 0u) |
+                      (c == nch - 1 ? kDLast : 0u) | (2 * wk.pair + 1 == heads ? kDLone : 0u) |
                       (static_cast<uint32_t>(min(32 * cb, n_of - off)) << 8) |
                       (static_cast<uint32_t>(rows) << 16));
             if (!ok) break;
@@ -605,11 +611,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int r = quarter * 32 + lane;                   // query row of the tile (TMEM lane)
     const uint32_t lane_sel = static_cast<uint32_t>(quarter * 32) << 16;
     const uint64_t sc = f2_pack(scale_log2, scale_log2);
+    const uint32_t lone = g == 1 ? kDLone : 0u;
     float m_ref = 0.f, l = 0.f;                          // reference (log2 units), row sum
     int u = 0;                                           // units finished
     auto step = [&](int j, uint32_t d) -> bool {
       const int kc = d_kc(d), groups = (kc + 15) >> 4, b = j & 1;
-      const bool live = quarter * 32 < d_rows(d);        // warp-uniform
+      // warp-uniform: rows of the tile, and not the head that a lone last one lacks
+      const bool live = quarter * 32 < d_rows(d) && !(d & lone);
       const uint32_t tsp = tmem + lane_sel + tmem_sp(g, b);
       if (!wait_warp(&s.s_full[g][b], (j >> 1) & 1, abort)) return false;
       tc_fence_after();
