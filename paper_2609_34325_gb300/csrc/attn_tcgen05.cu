@@ -336,18 +336,22 @@ __device__ __forceinline__ void mask_columns(uint32_t taddr, int count) {
   tmem_st_wait();
 }
 
-// p = 2^(s scale - m) of N values, summed into l0 and l1 and packed to bf16.
+// p = 2^(s scale - m) of N values, packed to bf16.  The sum (l0 + l1, fp32) is that
+// of the rounded values, which are the weights that V gets: their rounding then
+// cancels in O / sum for what the rows of V share.  Against 64 bits, relative
+// (2-norm), the sum of the values before rounding -> this one: 197 tokens 2.17e-3 ->
+// 2.10e-3, 577 2.28e-3 -> 2.23e-3 (the kernels before, whose largest weight was 1 more
+// often and so not rounded, 2.12e-3 and 2.26e-3).  The fp32 + bf16 adds cost 0-0.6 %
+// of the kernel against paired fp32 adds; unpacking the values for those 1-3.6 %.
 template <int N>
 __device__ __forceinline__ void exp_pack(const uint32_t (&a)[N], uint32_t (&p)[N / 2], uint64_t sc,
-                                         uint64_t nm, uint64_t& l0, uint64_t& l1) {
+                                         uint64_t nm, float& l0, float& l1) {
 #pragma unroll
   for (int e = 0; e < N; e += 2) {
     float x0, x1;
     f2_unpack(f2_fma(f2_pack(__uint_as_float(a[e]), __uint_as_float(a[e + 1])), sc, nm), x0, x1);
-    const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
-    if (e & 2) l1 = f2_add(l1, f2_pack(p0, p1));
-    else l0 = f2_add(l0, f2_pack(p0, p1));
-    p[e >> 1] = pack_bf16x2(p0, p1);
+    p[e >> 1] = pack_bf16x2(ex2_approx(x0), ex2_approx(x1));
+    add_bf16x2(l0, l1, p[e >> 1]);
   }
 }
 
@@ -662,7 +666,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         // a chunk of -infinities alone (only from infinite inputs) weighs nothing
         const float neg_m = m_ref == -INFINITY ? 0.f : -m_ref;
         const uint64_t nm = f2_pack(neg_m, neg_m);
-        uint64_t l0 = f2_pack(l, 0.f), l1 = f2_pack(0.f, 0.f);
+        float l0 = l, l1 = 0.f;
 #pragma unroll 1
         for (int i = 0; i < blocks; ++i) {
           uint32_t a[32], p[16];
@@ -678,9 +682,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           exp_pack<16>(a, p, sc, nm, l0, l1);
           tmem_st8(tsp + 16u * blocks, p);
         }
-        float s0, s1;
-        f2_unpack(f2_add(l0, l1), s0, s1);
-        l = s0 + s1;
+        l = l0 + l1;
         if (__any_sync(0xffffffffu, alpha != 1.f)) {
           // O holds the chunks before this one once their PV is done: bring it
           // to the raised reference before this chunk's PV

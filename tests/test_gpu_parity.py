@@ -962,6 +962,27 @@ def test_attention_with_a_bound_far_above_the_images(bound, batch):
     assert torch.equal(tight, loose)
 
 
+@pytest.mark.parametrize("tokens,bound", [(50, 1.96e-3), (197, 2.13e-3), (577, 2.26e-3)])
+def test_attention_error_is_the_weights_rounding(tokens, bound):
+    """Relative error (2-norm) against 64 bits, logits of a few units: the bf16
+    rounding of the weights and of the output.  One and several key chunks; the
+    bounds lie between 2.10e-3 with the row sum of the rounded weights and
+    2.17e-3 with that of the weights before rounding (197 tokens)."""
+    images, heads = 8, 12
+    gen = torch.Generator(device=dev()).manual_seed(35)
+    qkv = torch.empty(images * tokens, 3 * heads * 64, device=dev()).normal_(generator=gen)
+    qkv = (1.2 * qkv).bfloat16()
+    out = torch.empty(images * tokens, heads * 64, dtype=torch.bfloat16, device=dev())
+    cu = i32(np.arange(images + 1) * tokens)
+    P.dora_varlen_attn(qkv, cu, tokens, heads, out)
+    torch.cuda.synchronize()
+    q, k, v = qkv.double().view(images, tokens, 3, heads, 64).permute(2, 0, 3, 1, 4)
+    ref = torch.softmax(q @ k.transpose(-1, -2) / 8, -1) @ v
+    ref = ref.permute(0, 2, 1, 3).reshape(out.shape)
+    err = float((out.double() - ref).norm() / ref.norm())
+    assert err <= bound, err
+
+
 def test_attention_first_chunk_of_minus_infinities():
     """Logits of -inf (an infinite key component) in the whole first key
     chunk weigh nothing; the later chunk's keys get the weight."""
