@@ -77,12 +77,6 @@ struct Maps {
   CUtensorMap k, win, wqkv;
 };
 
-__device__ __forceinline__ void warp_arrive(uint64_t* bar) {
-  tc_fence_before();
-  __syncwarp();
-  if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
-}
-
 // 64 packed columns to global memory (32-byte aligned).
 __device__ __forceinline__ void store64(uint16_t* p, const uint32_t (&r)[32]) {
 #pragma unroll

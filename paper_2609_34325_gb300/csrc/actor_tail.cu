@@ -70,12 +70,6 @@ struct Maps {
   CUtensorMap o, wo, w1, w2, ws;
 };
 
-__device__ __forceinline__ void warp_arrive(uint64_t* bar) {
-  tc_fence_before();
-  __syncwarp();
-  if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
-}
-
 // 32 packed values as two 16-column stores.
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
   tmem_st16(taddr, *reinterpret_cast<const uint32_t(*)[16]>(&r[0]));

@@ -309,13 +309,6 @@ __device__ __forceinline__ bool wait_warp(uint64_t* bar, uint32_t parity, volati
   return __all_sync(0xffffffffu, wait_one(bar, parity, abort)) != 0;
 }
 
-// One arrival for the whole warp, after every lane's prior tcgen05 accesses.
-__device__ __forceinline__ void warp_arrive(uint64_t* bar) {
-  tc_fence_before();
-  __syncwarp();
-  if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
-}
-
 // -infinity in `count` (1 to 15) columns from taddr on, of this lane's row.
 __device__ __forceinline__ void mask_columns(uint32_t taddr, int count) {
   const uint32_t v = __float_as_uint(-INFINITY);

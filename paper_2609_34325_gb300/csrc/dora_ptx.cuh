@@ -158,12 +158,6 @@ __device__ __forceinline__ bool mbar_wait_sleep(uint64_t* bar, uint32_t parity,
   }
 }
 
-__device__ __forceinline__ bool mbar_wait_warp_sleep(uint64_t* bar, uint32_t parity,
-                                                     volatile int* abort, uint32_t hint_ns) {
-  const bool ok = mbar_wait_sleep(bar, parity, abort, hint_ns);
-  return __all_sync(0xffffffffu, ok) != 0;
-}
-
 // Same, with its own limit and no abort flag: used while draining.
 __device__ __forceinline__ bool mbar_wait_limited(uint64_t* bar, uint32_t parity,
                                                   uint64_t limit_ns) {
@@ -350,6 +344,13 @@ __device__ __forceinline__ void tc_fence_before() {
 }
 __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
+
+// One arrival for the whole warp, after every lane's prior tcgen05 accesses.
+__device__ __forceinline__ void warp_arrive(uint64_t* bar) {
+  tc_fence_before();
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
 }
 
 // Shared-memory matrix descriptor for a tile stored with the 128-byte swizzle
@@ -548,11 +549,6 @@ __device__ __forceinline__ void f2_unpack(uint64_t v, float& lo, float& hi) {
 __device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
   uint64_t d;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
 __device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {

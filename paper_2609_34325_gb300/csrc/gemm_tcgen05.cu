@@ -721,8 +721,9 @@ static cudaError_t launch_bn(const CUtensorMap& ta, const CUtensorMap& tb,
       return launch(launch_bn_epi<BN, DORA_EPI_BIAS_GELU, kPair>);
     case DORA_EPI_BIAS_RESIDUAL:
       return launch(launch_bn_epi<BN, DORA_EPI_BIAS_RESIDUAL, kPair>);
-    case kEpiResidualLongK:
-      return launch(launch_bn_epi<BN, kEpiResidualLongK, kPair>);
+    case kEpiResidualLongK:                        // only wide tiles
+      if constexpr (BN == 256) return launch(launch_bn_epi<BN, kEpiResidualLongK, kPair>);
+      return cudaErrorInvalidValue;
     case kEpiTokens:
       return launch(launch_bn_epi<BN, kEpiTokens, kPair>);
     case kEpiLn:
@@ -749,7 +750,7 @@ bool linear_merges(int32_t m_cap, int32_t n) { return gemm::one_wave(m_cap, n, 1
 
 cudaError_t launch_linear(const uint16_t* x, int32_t m_cap, const int32_t* m_dev, int32_t k,
                           const uint16_t* w, int32_t n, int32_t epilogue, const LinearEpi& ep,
-                          uint16_t* y, int32_t* status, cudaStream_t stream, int32_t lda) {
+                          uint16_t* y, int32_t* status, cudaStream_t stream) {
   if (m_cap == 0) return cudaSuccess;
   // A tile's main loop and epilogue get shorter with its width, so while one
   // wave of clusters holds all of them the narrowest tile finishes first; past
@@ -761,9 +762,8 @@ cudaError_t launch_linear(const uint16_t* x, int32_t m_cap, const int32_t* m_dev
   if (gemm::one_wave(m_cap, n, 64)) bn = 64;
   else if (gemm::one_wave(m_cap, n, 128)) bn = 128;
   CUtensorMap ta, tb, tbt, ty, tr;
-  if (lda != 0 && (lda < k || lda % 8 != 0)) return cudaErrorInvalidValue;
   if (encode_tmap_2d_bf16(&ta, x, static_cast<uint64_t>(k), static_cast<uint64_t>(m_cap),
-                          static_cast<uint64_t>(lda != 0 ? lda : k) * 2, gemm::BK, gemm::BM) != 0)
+                          static_cast<uint64_t>(k) * 2, gemm::BK, gemm::BM) != 0)
     return cudaErrorInvalidValue;
   if (encode_tmap_2d_bf16(&tb, w, static_cast<uint64_t>(k), static_cast<uint64_t>(n),
                           static_cast<uint64_t>(k) * 2, gemm::BK, static_cast<uint32_t>(bn / 2)) != 0)

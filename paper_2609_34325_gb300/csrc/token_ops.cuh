@@ -125,10 +125,9 @@ struct LinearEpi {
 // Whether a LayerNorm linear of this shape takes its input's slice moments
 // and merges them itself (the same bits as launch_merge_moments).
 bool linear_merges(int32_t m_cap, int32_t n);
-// lda: row pitch of x in elements (0 = k; a multiple of 8).
 cudaError_t launch_linear(const uint16_t* x, int32_t m_cap, const int32_t* m_dev, int32_t k,
                           const uint16_t* w, int32_t n, int32_t epilogue, const LinearEpi& ep,
-                          uint16_t* y, int32_t* status, cudaStream_t stream, int32_t lda = 0);
+                          uint16_t* y, int32_t* status, cudaStream_t stream);
 
 // The actor's encoder before its attention in one kernel: keys [m, dim] (row pitch
 // in elements), W_in [128, dim], W_qkv' [384, 128] (LayerNorm folded in); the live
