@@ -22,6 +22,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -46,12 +47,11 @@ E2E_SETS = 3
 # DRAM traffic of the GEMM (dram__bytes_read.sum + dram__bytes_write.sum)
 # from an ncu capture of the linear micro-benchmark (50432 rows, D = 768, MLP
 # 3072: one launch of each linear, inputs far above L2), keyed by the sha256 of
-# the kernel source it was taken on: bytes per row of each linear.  The bench
-# scales it to its own launches by their row counts (weights are read once a
-# launch, a small share), so it is reported for the DeiT-B shape only, and as
-# null once the source changes.
+# the kernel source it was taken on and its headers: bytes per row of each
+# linear.  The bench scales it to its own launches by their row counts (weights
+# are read once a launch, a small share), so it is reported for the DeiT-B shape
+# only, and as null once one of these files changes.
 NCU_GEMM_BYTES_PER_ROW = {
-    # profiles/gemm_tcgen05_deit_base_b256.md
     "4298482076f1a23124f7aa182f2251e73d4d651bcebaf599293d2ffc7b563d2a": {
         "gemm_qkv": 5110.8, "gemm_proj": 4030.3, "gemm_fc1": 6641.2, "gemm_fc2": 9188.8},
 }
@@ -60,10 +60,9 @@ NCU_GEMM_BYTES_PER_ROW = {
 # DRAM traffic of one launch of the fused selection + compaction, from an ncu
 # capture (dram__bytes_read.sum + dram__bytes_write.sum) of the token
 # micro-benchmark's DeiT-B case (inputs cycled beyond 2 x L2), keyed by the
-# sha256 of the kernel source; null once the source changes.
+# sha256 of the kernel source and its headers; null once one of them changes.
 NCU_TRAFFIC_SELECT_COMPACT = {
-    # profiles/select_compact_tokens.md: mean of 3 launches, 256 x 197 tokens,
-    # D = 768, 34,284 rows kept (106.5 MB algorithmic)
+    # mean of 3 launches, 256 x 197 tokens, D = 768, 34,284 rows kept (106.5 MB algorithmic)
     "4ab9fc8dc310aa87fe7700563abc77f255bca7fbda6251ecf194d739d78a1f33": {
         "traffic": 59500885, "case": "micro-benchmark: 256 x 197 tokens, D = 768, 34284 kept "
                                      "rows, inputs cycled beyond 2 x L2"},
@@ -98,8 +97,22 @@ def load_peaks():
 
 
 def sha256_of(path):
-    with open(path, "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()
+    """Of a kernel source together with the headers beside it that it includes,
+    directly or through one another: the kernel is made from all of them."""
+    files, todo = [], [path]
+    while todo:
+        p = todo.pop()
+        if p in files or not os.path.exists(p):
+            continue
+        files.append(p)
+        with open(p) as f:
+            todo += [os.path.join(os.path.dirname(p), n)
+                     for n in re.findall(r'^#include "([^"]+)"', f.read(), flags=re.M)]
+    h = hashlib.sha256()
+    for p in sorted(files):
+        with open(p, "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()
 
 
 # ---------------------------------------------------------------------------

@@ -1,5 +1,8 @@
 """Host-side logic of bench.py, on the CPU: the clock record, the roofline
 fractions and the per-block token counts of a workload."""
+import os
+import shutil
+
 import numpy as np
 import pytest
 
@@ -87,6 +90,24 @@ def test_roofline_traffic_only_for_the_captured_source_and_workload(monkeypatch)
     other = B.roofline_report(k, PEAKS, "measured", "cfg6")
     assert other["roofline"]["traffic"] is None
     assert other["roofline_compact"]["traffic"] is None
+
+
+@pytest.mark.parametrize("source", ["gemm_tcgen05.cu", "token_ops.cu"])
+def test_captured_traffic_is_keyed_by_the_headers_too(source, tmp_path):
+    """A kernel's captured figure lapses when a header that its source includes
+    changes, also one included by another header, and not for other files."""
+    csrc = os.path.join(B.ROOT, "paper_2609_34325_gb300", "csrc")
+    shutil.copytree(csrc, tmp_path / "csrc")
+    path = str(tmp_path / "csrc" / source)
+    key = B.sha256_of(path)
+    assert key == B.sha256_of(os.path.join(csrc, source))
+    for name, counts in (("epilogue_math.cuh", True), ("dora_ptx.cuh", True), (source, True),
+                         ("training.cu", False)):
+        f = tmp_path / "csrc" / name
+        text = f.read_text()
+        f.write_text(text + "// changed\n")
+        assert (B.sha256_of(path) != key) == counts, name
+        f.write_text(text)
 
 
 @pytest.mark.parametrize("name", ["cfg3", "cfg6"])
