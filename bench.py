@@ -52,8 +52,8 @@ E2E_SETS = 3
 # are read once a launch, a small share), so it is reported for the DeiT-B shape
 # only, and as null once one of these files changes.
 NCU_GEMM_BYTES_PER_ROW = {
-    "4298482076f1a23124f7aa182f2251e73d4d651bcebaf599293d2ffc7b563d2a": {
-        "gemm_qkv": 5110.8, "gemm_proj": 4030.3, "gemm_fc1": 6641.2, "gemm_fc2": 9188.8},
+    "ef14536c78ff3993dfd0de04ce6774b6cd77d422b31af5b0794098bdc25544ce": {
+        "gemm_qkv": 5122.7, "gemm_proj": 4028.8, "gemm_fc1": 6643.6, "gemm_fc2": 9165.3},
 }
 
 
@@ -63,8 +63,8 @@ NCU_GEMM_BYTES_PER_ROW = {
 # sha256 of the kernel source and its headers; null once one of them changes.
 NCU_TRAFFIC_SELECT_COMPACT = {
     # mean of 3 launches, 256 x 197 tokens, D = 768, 34,284 rows kept (106.5 MB algorithmic)
-    "4ab9fc8dc310aa87fe7700563abc77f255bca7fbda6251ecf194d739d78a1f33": {
-        "traffic": 59500885, "case": "micro-benchmark: 256 x 197 tokens, D = 768, 34284 kept "
+    "102ad98da83a38f44ba909db9007e45398cfe8d27800db69e832f1a804408076": {
+        "traffic": 59524608, "case": "micro-benchmark: 256 x 197 tokens, D = 768, 34284 kept "
                                      "rows, inputs cycled beyond 2 x L2"},
 }
 

@@ -16,7 +16,7 @@
 // Four launches: gate, budget and the selector's rest are the last one (one CTA
 // per image).  With a launch each for the input projection, gate with history, row
 // moments, QKV, budget and selector the call took 133.6 us at 256 x 197 tokens, now
-// 107.3; 8 ragged images of d = 384 took 53.5, now 37.9.
+// 106.4; 8 ragged images of d = 384 took 53.5, now 37.9.
 // The attention kernel has an instance for heads of 32 (softmax scale
 // 1/sqrt(32)).  On heads zero-padded to 64 the QKV linear wrote twice the bytes
 // and both MMAs did twice the work: 256 x 197 tokens, QKV 29.7 -> 16.5 us,
@@ -415,9 +415,9 @@ Ws ws_layout(int32_t t_cap, int32_t batch, const dora_actor_weights* w) {
   L.o = off;      off += up256(t * W * 2);
   L.z = off;      off += up256(t * W * 2);
   L.s1 = off;     off += up256(t * SH * 2);
-  // the size stays what it was when heads were padded to 64 and Z1, moments, the
-  // feed-forward's hidden rows and the gate's logits were kept: callers that sized
-  // the workspace by that are not refused, nor is its size a surprise to them
+  // More than the present launches use: the size is part of the interface, as it was
+  // when heads were padded to 64 and Z1, moments, the feed-forward's hidden rows and
+  // the gate's logits were kept (a smaller one would refuse nobody, but change it).
   off += up256(b * 4) + up256(t * (3 * W * 2 + W * 2 + W * 2 + 3 * 8 + FF * 2));
   L.prep = off;   off += w->prepared != nullptr ? 0 : prep_layout(w).total;
   L.total = off;

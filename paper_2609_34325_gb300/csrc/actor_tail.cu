@@ -20,8 +20,8 @@
 // then the selector's accumulator, 384-447 Z1, then Z, as bf16.
 //
 // What bounds it: the chain of four products and epilogues of a tile, about
-// 15,000 cycles (the GELU 5,200, the products 5,300, the other epilogues the
-// rest), run 2.6 times by each SM at 256 x 197 tokens; the traffic (46 MB) would
+// 15,500 cycles (the GELU 4,300, the waits for the products 3,500 to 4,900, the
+// other epilogues and the loads of X the rest), run 2.6 times by each SM at 256 x 197 tokens; the traffic (46 MB) would
 // take 7 us.  As five launches (output projection, moments merge, fc1, fc2,
 // selector linear), whose K = 128 tiles are all prologue and epilogue, the same
 // took 60 us of device time, here 31; in the stream the actor's call went from

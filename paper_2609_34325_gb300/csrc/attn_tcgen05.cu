@@ -48,8 +48,8 @@
 // loader and issuers have one call site for each.  Measured against the kernel
 // before it (two threads a row exchanging maxima, MMAs issued from a lane-0
 // branch, one query tile at a time), us: 256 x 197 tokens x 12 heads 93.7 ->
-// 76.7, the same after one and two deletions 69.9 -> 50.5 and 33.0 -> 26.0, 64 x
-// 577 x 12 136.9 -> 109.5, 128 x 257 x 12 91.0 -> 66.1.
+// 77.4, the same after one and three deletions 69.9 -> 49.8 and 33.0 -> 25.8, 64 x
+// 577 x 12 136.9 -> 107.5, 128 x 257 x 12 91.0 -> 65.0.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>

@@ -864,8 +864,9 @@ def test_attention_edge_lengths_and_nan_tail():
 
 
 def test_attention_running_maximum_moves_between_key_chunks():
-    """Keys of later 128-key chunks scaled up (image 0: x4 then x8; image 2:
-    x6) so that the row maximum of a later chunk lies far above the first
+    """Keys from 128 and 256 on scaled up (image 0: x4 then x8; image 2: x6),
+    past the first chunk of at most 96 keys, so that the row maximum of a later
+    chunk lies far above the first
     chunk's and the online softmax has to move its reference; image 1 is the
     reverse (first chunk dominant, later probabilities underflow)."""
     lens = np.array([300, 200, 140])
@@ -899,8 +900,8 @@ def test_attention_range_split_over_many_images(mix):
     """The split of image-heads over the persistent CTAs (each lane of the
     range search reading a block of image bounds): batches above 256 images
     (several rounds of loads per lane), skewed costs with many empty and
-    one-token images beside a few of 300 tokens (the kernel for images past
-    256 tokens), and fewer image-heads than SMs.  Every row of every
+    one-token images beside a few of 300 tokens (three query tiles and four
+    key chunks each), and fewer image-heads than SMs.  Every row of every
     image is compared with the oracle, so an image-head given to no CTA (its
     rows keep the fill value) or to two fails."""
     rng = np.random.default_rng({"many_images": 21, "skewed": 22, "few_image_heads": 23}[mix])
@@ -910,7 +911,7 @@ def test_attention_range_split_over_many_images(mix):
         heads = 2
     elif mix == "skewed":
         lens = rng.integers(0, 4, 700)
-        lens[rng.choice(700, 9, replace=False)] = 300    # the per-key-half kernel
+        lens[rng.choice(700, 9, replace=False)] = 300    # three query tiles, four key chunks
         heads = 3
     else:
         lens = rng.integers(0, 257, 40)
