@@ -184,9 +184,10 @@ __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map) {
 // Programmatic dependent launch.  pdl_trigger lets the next kernel on the
 // stream be scheduled while this one runs (it starts as SMs free up);
 // pdl_wait blocks until the previous kernel has finished and its memory is
-// visible.  Every kernel of this library triggers at its start and waits
-// before its first global access that another kernel may have written or may
-// still read.  Without the launch attribute both return at once.
+// visible.  Every kernel of this library waits before its first global access
+// that another kernel may have written or may still read, and all but the
+// training side's trigger at their start.  Without the launch attribute both
+// return at once.
 __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

@@ -11,6 +11,14 @@
 //                                    extra sequences of the same packed batch;
 //   fidelity cost                    App. B.2: tau^2 KL(softmax(z^N / tau) ||
 //                                    softmax(z^(l) / tau)) per shadow.
+//
+// The kernels here are launched as dependents but let theirs start only when they
+// end.  Triggered early, the next kernels' CTAs are placed, and wait, in the room
+// that this one leaves: the sampling's few CTAs, O(n^2) each, land several on one
+// SM beside a branch copy, and a copy's CTAs unevenly beside waiting kernels.  The
+// five calls of a rollout action, us with the trigger at the start -> without (and
+// with plain launches): 64 images of 577 tokens of 768 96 -> 56 (68), 87 images 111
+// -> 62 (74), 256 of 197 63 -> 46 (57), 8 of 197 34.5 -> 35 (host-bound).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -47,7 +55,6 @@ __global__ void __launch_bounds__(kThreads)
                      int k_cap, int32_t* __restrict__ order, float* __restrict__ keys_out,
                      int32_t* status) {
   __shared__ uint32_t keys[kMaxVisual];
-  pdl_trigger();
   pdl_wait();
   const int img = blockIdx.x;
   const int lo = cu[img], hi = cu[img + 1];
@@ -128,7 +135,6 @@ __global__ void __launch_bounds__(kThreads)
   __shared__ float lt[kMaxVisual];        // L_t, then P_t
   __shared__ Lse part[kThreads / 32];
   __shared__ int bad;
-  pdl_trigger();
   pdl_wait();
   const int img = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int lo = cu[img], hi = cu[img + 1];
@@ -254,7 +260,6 @@ __global__ void __launch_bounds__(kScanThreads)
   __shared__ int warp_fit[kScanThreads / 32];
   __shared__ long long carry;
   __shared__ int last_fit;
-  pdl_trigger();
   pdl_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (cu_out != cu)
@@ -319,7 +324,6 @@ __global__ void branch_rows_kernel(uint4* __restrict__ x, int32_t* __restrict__ 
                                    float2* __restrict__ mv, const int32_t* __restrict__ cu_out,
                                    int batch, const int32_t* __restrict__ src, int nb, int t_cap,
                                    int d8) {
-  pdl_trigger();
   pdl_wait();
   const int warps = gridDim.x * (blockDim.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -378,7 +382,6 @@ __global__ void __launch_bounds__(kBranchThreads)
                   int32_t* len_out, int32_t* status) {
   __shared__ long long scratch[kBranchThreads / 32];
   __shared__ long long ends[kBranchThreads];
-  pdl_trigger();
   pdl_wait();
   const int sq = blockIdx.y, part = blockIdx.x;
   const int base = cu[batch];
@@ -481,7 +484,6 @@ __global__ void __launch_bounds__(kHeldThreads)
                         const int32_t* __restrict__ map, int shadows, int batch, int classes,
                         int ld8, float inv_tau, float tau2, float* __restrict__ cost,
                         int32_t* status) {
-  pdl_trigger();
   pdl_wait();
   const int sh = (blockIdx.x * kHeldThreads + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (sh >= shadows) return;
@@ -549,7 +551,6 @@ __global__ void kd_cost_kernel(const uint16_t* __restrict__ zn, const uint16_t* 
                                const int32_t* __restrict__ map, int shadows, int batch,
                                int classes, int ld, float inv_tau, float tau2,
                                float* __restrict__ cost, int32_t* status) {
-  pdl_trigger();
   pdl_wait();
   const int sh = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (sh >= shadows) return;
@@ -595,7 +596,6 @@ __global__ void step_rewards_kernel(const float* __restrict__ cost,
                                     const int32_t* __restrict__ blocks, int n_blocks, int batch,
                                     int depth, int n0, float a, float* __restrict__ reward,
                                     float* __restrict__ ret) {
-  pdl_trigger();
   pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= batch) return;
