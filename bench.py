@@ -52,8 +52,8 @@ E2E_SETS = 3
 # are read once a launch, a small share), so it is reported for the DeiT-B shape
 # only, and as null once one of these files changes.
 NCU_GEMM_BYTES_PER_ROW = {
-    "ef14536c78ff3993dfd0de04ce6774b6cd77d422b31af5b0794098bdc25544ce": {
-        "gemm_qkv": 5122.7, "gemm_proj": 4028.8, "gemm_fc1": 6643.6, "gemm_fc2": 9165.3},
+    "0f7a3d793ab32041e3294034f4461374a51de3a75938bc3ffd50675bb51163b5": {
+        "gemm_qkv": 5121.4, "gemm_proj": 4028.6, "gemm_fc1": 6640.7, "gemm_fc2": 9202.0},
 }
 
 
@@ -63,8 +63,8 @@ NCU_GEMM_BYTES_PER_ROW = {
 # sha256 of the kernel source and its headers; null once one of them changes.
 NCU_TRAFFIC_SELECT_COMPACT = {
     # mean of 3 launches, 256 x 197 tokens, D = 768, 34,284 rows kept (106.5 MB algorithmic)
-    "102ad98da83a38f44ba909db9007e45398cfe8d27800db69e832f1a804408076": {
-        "traffic": 59524608, "case": "micro-benchmark: 256 x 197 tokens, D = 768, 34284 kept "
+    "19126b5eecdcd31b35d965921f494e6845a85a9663160a9c73c34652f4ed1a06": {
+        "traffic": 59394048, "case": "micro-benchmark: 256 x 197 tokens, D = 768, 34284 kept "
                                      "rows, inputs cycled beyond 2 x L2"},
 }
 
