@@ -2,6 +2,7 @@
 against the fp64 oracle on the same seeded inputs.  Integer and byte outputs
 (kept_idx, cu_seqlens, ids, packed rows) must match bit for bit; floating
 outputs within |err| <= 2e-2 or |err| <= 1e-2 |ref|."""
+import threading
 from dataclasses import replace
 
 import numpy as np
@@ -1853,3 +1854,34 @@ def test_lc1_of_a_row_whose_variance_overflows(d):
     x = torch.full((3, d), 2.0 ** 70, dtype=torch.bfloat16, device=dev())
     x[:, ::2] *= -1
     assert torch.all(_lc1_features(x, i32([0, 3])) == 0)
+
+
+def _in_a_fresh_thread(call):
+    """What `call` raises, if anything, as a new thread's first CUDA work."""
+    raised = []
+
+    def run():
+        try:
+            call()
+        except Exception as e:          # handed to the test's own thread
+            raised.append(e)
+
+    t = threading.Thread(target=run)
+    t.start()
+    t.join()
+    torch.cuda.synchronize()
+    return raised
+
+
+def test_first_call_of_a_thread():
+    """A thread whose first CUDA work is a call of the library: the tensor maps'
+    encoding is a driver call, for which such a thread has no context yet."""
+    x, w = (torch.ones(128, 64, dtype=torch.bfloat16, device=dev()) for _ in range(2))
+    y = torch.zeros(128, 128, dtype=torch.bfloat16, device=dev())
+    qkv = torch.ones(128, 192, dtype=torch.bfloat16, device=dev())
+    out = torch.zeros(128, 64, dtype=torch.bfloat16, device=dev())
+    cu = i32([0, 128])
+    torch.cuda.synchronize()
+    assert _in_a_fresh_thread(lambda: P.dora_linear(x, w, y)) == []
+    assert _in_a_fresh_thread(lambda: P.dora_varlen_attn(qkv, cu, 128, 1, out)) == []
+    assert torch.all(y == 64) and torch.all(out == 1)
